@@ -77,8 +77,9 @@ typedef enum { LBS_VISC_POWER = 0, LBS_VISC_SUTHERLAND = 1 } lbs_visc_law;
  * increments over the step's start state, not stage values, for the same reason.
  * Moment sums: with FP32 storage, in FP32 within a CTA's velocity chunk and in
  * double-float (an FP32 pair, about 48 significant bits) across chunks; with FP64
- * storage, in FP64.  The cell state, the wall flux balance, the profiles and the
- * residual are FP64 in both modes. */
+ * storage, in FP64.  From those sums the cell state (n, u, P, T, q) is formed in the same
+ * arithmetic (double-float or FP64) and rounded to FP64; the half-range coefficients of the
+ * equilibrium, the wall flux balance and the residual are FP64 in both modes. */
 typedef enum { LBS_FP64 = 0, LBS_FP32_STORE_FP64_ACC = 1 } lbs_precision;
 
 /* Velocity-set orders.  N_eq is the order of the truncated Hermite expansion
@@ -286,13 +287,13 @@ lbs_status lbs_set_tiling(lbs_handle h, int V, int ZT, int fuse);
  * CTA.  Any output pointer may be NULL. */
 lbs_status lbs_get_tiling(lbs_handle h, int* V, int* ZT, int* fuse, int* ntiles, long* smem_bytes);
 
-/* Finalisation layout (not in the paper: how the per-cell FP64 work of each stage
- * -- moments, profiles, equilibrium coefficients -- is spread over threads).
- * mode 1: one thread per cell; mode 2: one warp per cell (lanes share the moment
- * sums, the x / y coefficient recurrences and the two half-range tables); mode 0
- * (the default): mode 2 for batches of at most 608 cells, else mode 1.  Results
- * agree to rounding (a few ulps of FP64).  *warp_out (may be NULL) receives 1 if
- * the warp layout is in use.  Synchronises the solver's stream. */
+/* Finalisation layout (not in the paper: how the per-cell work of each stage -- moments,
+ * profiles, equilibrium coefficients -- is spread over the GPU).  A CTA of 128 threads
+ * finalises a few cells at a time: four (mode 2), or 8, 16 or 32 by the cells of the
+ * batch (mode 1); mode 0 (the default) chooses among all four, four up to 1216 cells.
+ * Results agree to rounding (a few ulps of FP64, or of the double-float arithmetic that
+ * FP32 storage uses).  *warp_out (may be NULL) receives 1 if the four-cell layout is
+ * in use.  Synchronises the solver's stream. */
 lbs_status lbs_set_finalize(lbs_handle h, int mode, int* warp_out);
 
 /* The CUDA stream (cudaStream_t) the handle queues its work on: the one given at

@@ -16,11 +16,11 @@
 
 namespace lbs {
 cudaError_t launch_stage(int fp32, int red, int V, int stage, const InstDev* d_inst, const Tile* d_tiles,
-                         int ntiles, size_t smem, int fuse, int ninst, int maxNz, int fin_warp, int nb,
+                         int ntiles, size_t smem, int fuse, int ninst, int maxNz, int fin_cells, int nb,
                          cudaStream_t st);
 cudaError_t launch_stage_only(int fp32, int red, int V, int stage, const InstDev* d_inst, const Tile* d_tiles,
                               int ntiles, size_t smem, int fuse, cudaStream_t st);
-cudaError_t launch_finalize(int fp32, int stage, const InstDev* d_inst, int ninst, int maxNz, int fin_warp,
+cudaError_t launch_finalize(int fp32, int stage, const InstDev* d_inst, int ninst, int maxNz, int fin_cells,
                             int nb, cudaStream_t st);
 cudaError_t launch_seed(int fp32, const InstDev* d_inst, int inst, int Nz, const double* d_macro,
                         cudaStream_t st);
@@ -75,7 +75,7 @@ struct lbs_solver {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int fp32 = 0, esize = 8, V = 1, ZT = 16, fuse = 1, ninst = 0, maxNz = 0, nb = 0;
-    int fin_mode = 0, fin_warp = 0;  // finalisation: 0 auto, 1 thread per cell, 2 warp per cell
+    int fin_mode = 0, fin_cells = 4;  // lbs_set_finalize's mode; cells per CTA of the finalisation
     int reduced = 0;                 // the batch runs the phi / chi model (all instances alike)
     std::vector<InstHost> ih;
     std::vector<InstDev> idev;
@@ -177,6 +177,44 @@ static void put_pairs(std::vector<unsigned char>& host, size_t off, const std::v
     }
 }
 
+static void float_pair(double v, float (&r)[2])
+{
+    r[0] = float(v);
+    r[1] = float(v - double(r[0]));
+}
+
+// coefficients of the monic half-range polynomials pi_0 .. pi_kMaxN, row l ascending in the
+// power: pi_{l+1} = (p - alpha_l) pi_l - beta_l pi_{l-1}, in double-double (the rows enter sums
+// that cancel strongly, so their entries are rounded once)
+static std::vector<double> half_polynomials(const std::vector<double>& al, const std::vector<double>& be)
+{
+    const int n = kMaxN + 1;
+    std::vector<double> hi(n * n, 0.0), lo(n * n, 0.0);
+    hi[0] = 1.0;
+    auto add = [&](int e, double v) {  // entry e += v
+        const double s = hi[e] + v, bb = s - hi[e], t = (hi[e] - (s - bb)) + (v - bb) + lo[e];
+        hi[e] = s + t;
+        lo[e] = t - (hi[e] - s);
+    };
+    auto add_product = [&](int e, double c, int f) {  // entry e += c times entry f
+        const double p = c * hi[f];
+        const double err = std::fma(c, hi[f], -p) + c * lo[f];
+        add(e, p);
+        add(e, err);
+    };
+    for (int l = 0; l + 1 < n; ++l)
+        for (int k = 0; k <= l + 1; ++k) {
+            const int e = (l + 1) * n + k;
+            if (k > 0) {
+                add(e, hi[l * n + k - 1]);
+                add(e, lo[l * n + k - 1]);
+            }
+            add_product(e, -al[l], l * n + k);
+            if (l > 0) add_product(e, -be[l], (l - 1) * n + k);
+        }
+    return hi;
+}
+
 template <typename T>
 static std::vector<double> rounded(const std::vector<double>& v)
 {
@@ -248,18 +286,24 @@ static void build_tiles(lbs_solver* h, std::vector<Tile>& tiles)
 }
 
 
-// Finalisation with one warp per cell pays while the batch has at most one cell per
-// warp scheduler (152 SMs x 4): each cell's FP64 chain then runs on a scheduler of
-// its own, with its loads, coefficient sets and half-range tables spread over the
-// lanes.  Beyond that one thread per cell keeps every lane busy (measured: 320
-// cells 30 us per launch with warps vs 48 us with threads; 2048 cells 57 vs 34 us).
-constexpr long kFinWarpMaxCells = 608;
+// Cells that a CTA of the finalisation takes at a time, by the cells of the batch.  Few cells
+// per CTA spread a small batch over more schedulers' FP64 units and shorten each CTA's chain;
+// many fill the lanes of the FP64 instructions, which cost the same with 1 or 32 active lanes.
+// Measured, us per step (three launches) at 4 / 8 / 16 / 32 cells, FP32 storage on replicas
+// of C2: 128 cells 43 / 45 / 57 / 76, 1024 cells 45 / 48 / 57 / 78, 2048 cells 57 / 51 / 57 /
+// 76, 8192 cells 111 / 71 / 73 / 94, 16384 cells 177 / 117 / 90 / 108, 32768 cells 297 / 190 /
+// 152 / 139; 8192 cells of C3 129 / 92 / 104 / 145, the 11792-cell sweep 182 / 124 / 116 / 137;
+// FP64 storage: 2048 cells 68 / 60 / 69 / 92, 8192 cells 165 / 101 / 97 / 115.
+static int finalize_cells_rule(long cells)
+{
+    return cells <= 1216 ? 4 : cells <= 10240 ? 8 : cells <= 24576 ? 16 : 32;
+}
 static void choose_finalize(lbs_solver* h)
 {
     long cells = 0;
     for (int b = 0; b < h->ninst; ++b) cells += h->ih[b].Nz;
-    h->fin_warp = h->fin_mode == 2 || (h->fin_mode == 0 && cells <= kFinWarpMaxCells);
-    for (int b = 0; b < h->ninst; ++b) h->idev[b].fin_warp = h->fin_warp;
+    const int rule = finalize_cells_rule(cells);
+    h->fin_cells = h->fin_mode == 2 ? 4 : h->fin_mode == 1 ? std::max(8, rule) : rule;
 }
 
 template <typename T>
@@ -269,7 +313,7 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
     std::vector<std::vector<double>> tabs_d;  // per instance, concatenated later
     Pool pool;
     struct Off {
-        size_t Hx, Hy, Pz, Hx2, Hy2, Pz2, alpha, beta, px, py, xi, wx, wy, wz, gxt, gxb, gwy, gwz, idz;
+        size_t Hx, Hy, Pz, Hx2, Hy2, Pz2, poly, px, py, xi, wx, wy, wz, gxt, gxb, gwy, gwz, idz;
         size_t F0, F1, F2, L0, cur, rec, partial, flux, nw, prof, Wold, Wnew, res, steps, active, status, zcount,
             icount;
     };
@@ -406,8 +450,8 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
             szp += wz[m] * xi[m] * (1.0 + gwz[m]);
             szm += wz[m] * (-xi[m]) * (1.0 + gwz[I.Qz + m]);
         }
-        D.Dtop = sxt * sy * szm;
-        D.Dbot = sxb * sy * szp;
+        D.iDtop = 1.0 / (sxt * sy * szm);
+        D.iDbot = 1.0 / (sxb * sy * szp);
         // the rest state f = w: its raw moments (the kernels sum the deviations from it)
         // and its outgoing flux through each wall, over the stored nodes and weights
         for (int a2 = 0; a2 < kNMom; ++a2) D.mrest[a2] = 0.0;
@@ -431,13 +475,14 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
                         else D.frest_top += w * Z;
                     }
         if (half) D.frest_bot = 0.0;  // no wall below a half channel
+        for (int a2 = 0; a2 < kNMom; ++a2) float_pair(D.mrest[a2], D.mrest2[a2]);
         D.wait_limit = kWaitLimit;
         // memory layout
         Off& o = off[b];
         const size_t es = sizeof(T);
         o.Hx = pool.take(t.Hx.size() * 8); o.Hy = pool.take(t.Hy.size() * 8); o.Pz = pool.take(t.Pz.size() * 8);
         o.Hx2 = pool.take(t.Hx.size() * 8); o.Hy2 = pool.take(t.Hy.size() * 8); o.Pz2 = pool.take(t.Pz.size() * 8);
-        o.alpha = pool.take(t.alpha.size() * 8); o.beta = pool.take(t.beta.size() * 8);
+        o.poly = pool.take((kMaxN + 1) * (kMaxN + 1) * 8);
         o.px = pool.take(I.Qx * es); o.py = pool.take(I.Qy * es); o.xi = pool.take(I.Qz * es);
         o.wx = pool.take(I.Qx * es); o.wy = pool.take(I.Qy * es); o.wz = pool.take(I.Qz * es);
         o.gxt = pool.take(I.Qx * es); o.gxb = pool.take(I.Qx * es); o.gwy = pool.take(I.Qy * es);
@@ -508,7 +553,7 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         const InstHost& I = h->ih[b];
         put<double>(img, o.Hx, t.Hx); put<double>(img, o.Hy, t.Hy); put<double>(img, o.Pz, t.Pz);
         put_pairs(img, o.Hx2, t.Hx); put_pairs(img, o.Hy2, t.Hy); put_pairs(img, o.Pz2, t.Pz);
-        put<double>(img, o.alpha, t.alpha); put<double>(img, o.beta, t.beta);
+        put<double>(img, o.poly, half_polynomials(t.alpha, t.beta));
         put<T>(img, o.px, t.px); put<T>(img, o.py, t.py); put<T>(img, o.xi, t.xi);
         put<T>(img, o.wx, t.wx); put<T>(img, o.wy, t.wy); put<T>(img, o.wz, t.wz);
         put<T>(img, o.gxt, t.gxt); put<T>(img, o.gxb, t.gxb); put<T>(img, o.gwy, t.gwy);
@@ -523,12 +568,12 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         D.Hx2 = reinterpret_cast<const float2*>(P + o.Hx2);
         D.Hy2 = reinterpret_cast<const float2*>(P + o.Hy2);
         D.Pz2 = reinterpret_cast<const float2*>(P + o.Pz2);
-        D.sumw_x = D.sumw_y = D.sumw_z = 0.0;  // of the weights as stored
-        for (int i = 0; i < I.Qx; ++i) D.sumw_x += double(T(t.wx[i]));
-        for (int j = 0; j < I.Qy; ++j) D.sumw_y += double(T(t.wy[j]));
-        for (int m = 0; m < I.Qz; ++m) D.sumw_z += 2.0 * double(T(t.wz[m]));
-        D.alpha = reinterpret_cast<const double*>(P + o.alpha);
-        D.beta = reinterpret_cast<const double*>(P + o.beta);
+        D.sumw[0] = D.sumw[1] = D.sumw[2] = 0.0;  // of the weights as stored
+        for (int i = 0; i < I.Qx; ++i) D.sumw[0] += double(T(t.wx[i]));
+        for (int j = 0; j < I.Qy; ++j) D.sumw[1] += double(T(t.wy[j]));
+        for (int m = 0; m < I.Qz; ++m) D.sumw[2] += 2.0 * double(T(t.wz[m]));
+        for (int a = 0; a < 3; ++a) float_pair(D.sumw[a], D.sumw2[a]);
+        D.half_poly = reinterpret_cast<const double*>(P + o.poly);
         D.px = P + o.px; D.py = P + o.py; D.xi = P + o.xi; D.wx = P + o.wx; D.wy = P + o.wy; D.wz = P + o.wz;
         D.gwx_top = P + o.gxt; D.gwx_bot = P + o.gxb; D.gwy = P + o.gwy; D.gwz = P + o.gwz;
         D.inv_dz = P + o.idz;
@@ -582,7 +627,7 @@ static lbs_status analyse(lbs_solver* h)
 {
     NvtxRange r(kStageRange[0]);
     CK(launch_stage(h->fp32, h->reduced, h->V, 0, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->ninst, h->maxNz,
-                    h->fin_warp, h->nb, h->stream));
+                    h->fin_cells, h->nb, h->stream));
     return LBS_OK;
 }
 
@@ -608,7 +653,7 @@ static lbs_status enqueue_step(lbs_solver* h)
         for (int s = 1; s <= 3; ++s) {
             NvtxRange r(kStageRange[s]);
             CK(launch_stage(h->fp32, h->reduced, h->V, s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->ninst,
-                            h->maxNz, h->fin_warp, h->nb, h->stream));
+                            h->maxNz, h->fin_cells, h->nb, h->stream));
         }
         return LBS_OK;
     }
@@ -619,10 +664,10 @@ static lbs_status enqueue_step(lbs_solver* h)
     for (int s = 1; s <= 3; ++s) {
         NvtxRange r(kStageRange[s]);
         CK(launch_stage_only(h->fp32, h->reduced, h->V, s, h->d_inst, h->d_tiles, h->ntilesA, h->smem, 0, h->stream));
-        CK(launch_finalize(h->fp32, s, h->d_inst, h->nA, h->maxNz, h->fin_warp, h->nb, h->stream));
+        CK(launch_finalize(h->fp32, s, h->d_inst, h->nA, h->maxNz, h->fin_cells, h->nb, h->stream));
         CK(launch_stage_only(h->fp32, h->reduced, h->V, s, h->d_inst, h->d_tiles + h->ntilesA, h->ntiles - h->ntilesA, h->smem,
                              0, h->stream2));
-        CK(launch_finalize(h->fp32, s, h->d_inst + h->nA, h->ninst - h->nA, h->maxNz, h->fin_warp, h->nb, h->stream2));
+        CK(launch_finalize(h->fp32, s, h->d_inst + h->nA, h->ninst - h->nA, h->maxNz, h->fin_cells, h->nb, h->stream2));
     }
     CK(cudaEventRecord(h->ev_join, h->stream2));
     CK(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
@@ -938,8 +983,8 @@ lbs_status lbs_run_to_steady(lbs_handle h, double tol, long max_steps, int check
         CK(cudaStreamSynchronize(h->stream));
         for (int b = 0; b < h->ninst; ++b) all &= act[b] == 0;
         // once a quarter of the launched tiles belong to retired instances, launch only
-        // the live ones; once few cells are left, finalise them with a warp per cell
-        // (the automatic layout), whose FP64 chains are shorter
+        // the live ones, and finalise fewer cells per CTA once the live ones are few (the
+        // automatic layout)
         long live = 0, cells = 0;
         for (int b = 0; b < h->ninst; ++b) {
             live += act[b] ? (long)h->ih[b].nchunks * h->ih[b].nzt : 0;
@@ -950,11 +995,8 @@ lbs_status lbs_run_to_steady(lbs_handle h, double tol, long max_steps, int check
             s = upload_tiles(h, &act);
             regraph = true;
         }
-        if (!all && s == LBS_OK && h->fin_mode == 0 && !h->fin_warp && cells <= kFinWarpMaxCells) {
-            h->fin_warp = 1;
-            for (int b = 0; b < h->ninst; ++b) h->idev[b].fin_warp = 1;
-            CK(cudaMemcpyAsync(h->d_inst, h->idev.data(), sizeof(InstDev) * h->ninst, cudaMemcpyHostToDevice,
-                               h->stream));
+        if (!all && s == LBS_OK && h->fin_mode == 0 && finalize_cells_rule(cells) < h->fin_cells) {
+            h->fin_cells = finalize_cells_rule(cells);
             drop_graph(h);
             regraph = true;
         }
@@ -1011,7 +1053,7 @@ lbs_status lbs_profile_steps(lbs_handle h, long nsteps, double* out_ms)
         for (int s = 1; s <= 3; ++s) {
             CK(launch_stage_only(h->fp32, h->reduced, h->V, s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->stream));
             CK(cudaEventRecord(ev[2 * s - 1], h->stream));
-            if (!(h->fuse & 1)) CK(launch_finalize(h->fp32, s, h->d_inst, h->ninst, h->maxNz, h->fin_warp, h->nb, h->stream));
+            if (!(h->fuse & 1)) CK(launch_finalize(h->fp32, s, h->d_inst, h->ninst, h->maxNz, h->fin_cells, h->nb, h->stream));
             CK(cudaEventRecord(ev[2 * s], h->stream));
         }
         CK(cudaEventSynchronize(ev[6]));
@@ -1085,9 +1127,7 @@ lbs_status lbs_set_finalize(lbs_handle h, int mode, int* warp_out)
     drop_graph(h);
     h->fin_mode = mode;
     choose_finalize(h);
-    CK(cudaMemcpyAsync(h->d_inst, h->idev.data(), sizeof(InstDev) * h->ninst, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    if (warp_out) *warp_out = h->fin_warp;
+    if (warp_out) *warp_out = h->fin_cells == 4;
     return check_status(h);
 }
 
@@ -1304,7 +1344,7 @@ lbs_status lbs_set_state(lbs_handle h, int inst, const void* src, int from_host)
             CK(launch_stage_only(h->fp32, h->reduced, h->V, 0, h->d_inst, h->d_tiles + h->tile_first[c0],
                                  h->tile_first[c1] - h->tile_first[c0], h->smem, h->fuse & 1, h->stream2));
             if (!(h->fuse & 1))
-                CK(launch_finalize(h->fp32, 0, h->d_inst + c0, c1 - c0, h->maxNz, h->fin_warp, h->nb, h->stream2));
+                CK(launch_finalize(h->fp32, 0, h->d_inst + c0, c1 - c0, h->maxNz, h->fin_cells, h->nb, h->stream2));
         }
         c0 = c1;
     }

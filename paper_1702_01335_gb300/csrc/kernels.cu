@@ -5,44 +5,22 @@
 
 namespace lbs {
 
-// ---- separate finalisation launches (used when the stage kernel does not fuse them).
-// NB bounds the expansion orders of the batch (the unrolled coefficient loops of the
-// record run to NB, not to the largest order kMaxN).
-template <typename T, int NB>
-__global__ void __launch_bounds__(32) finalize_cells(const InstDev* __restrict__ insts, int stage)
+// ---- separate finalisation launches (used when the stage kernel does not fuse them): C
+// cells per block of 128 threads, blockIdx.y the instance.  NB bounds the expansion orders of
+// the batch (the unrolled coefficient loops run to NB, not to the largest order kMaxN).
+template <typename T, int NB, int C>
+__global__ void __launch_bounds__(kThreads) finalize_cells(const InstDev* __restrict__ insts, int stage)
 {
-    __shared__ double red[kRedSlots];
+    __shared__ FinShared<T, C> sm;
+    __shared__ double red[8 * (kThreads / 32)];
     __shared__ int last;
     __shared__ InstDev sI;
     const InstDev& I = stage_descriptor(insts + blockIdx.y, &sI);
-    const int nblk = (I.Nz + 31) >> 5;
+    const int nblk = (I.Nz + C - 1) / C, c0 = blockIdx.x * C;
     if (blockIdx.x >= nblk || *I.active == 0) return;
-    const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell < I.Nz) finalize_cell<T, NB>(I, cell, stage);
+    finalize_group<T, NB, C>(I, c0, min(C, I.Nz - c0), stage, sm, (blockIdx.x + blockIdx.y) & 3);
     // the instance's last block to finish (threadfence ticket) forms n_w and, after
     // stage 3, the residual; the counter is reset by its last user
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(I.icount, 1) == nblk - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    if (threadIdx.x == 0) *I.icount = 0;
-    finalize_instance(I, stage, red);
-}
-
-// the same with one warp per cell (4 cells per block of 128 threads)
-template <typename T>
-__global__ void __launch_bounds__(128) finalize_cells_warp(const InstDev* __restrict__ insts, int stage)
-{
-    __shared__ double red[kRedSlots];
-    __shared__ int last;
-    __shared__ InstDev sI;
-    const InstDev& I = stage_descriptor(insts + blockIdx.y, &sI);
-    const int nblk = (I.Nz + 3) >> 2;
-    if (blockIdx.x >= nblk || *I.active == 0) return;
-    const int cell = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (cell < I.Nz) finalize_cell_warp<T>(I, cell, threadIdx.x & 31, stage);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(I.icount, 1) == nblk - 1;
@@ -88,7 +66,7 @@ __global__ void __launch_bounds__(128) seed_cells(const InstDev* __restrict__ in
 template <typename T>
 __global__ void __launch_bounds__(128) seed_free_molecular(const InstDev* __restrict__ insts, int inst)
 {
-    __shared__ double red[kRedSlots];
+    __shared__ double red[kThreads / 32];
     const InstDev& I = insts[inst];
     const int cell = blockIdx.x;
     T* F = static_cast<T*>(*I.cur ? I.F1 : I.F0) + (size_t)cell * I.Q;
@@ -175,15 +153,21 @@ static cudaError_t launch_first(K kernel, dim3 g, dim3 b, cudaStream_t st, const
     return cudaLaunchKernelEx(&cfg, kernel, d_inst, stage);
 }
 
-template <typename T>
-static cudaError_t launch_finalize_t(int stage, const InstDev* d_inst, int ninst, int maxNz, int fin_warp,
-                                     int nb, cudaStream_t st)
+template <typename T, int C>
+static cudaError_t launch_finalize_t(int stage, const InstDev* d_inst, int ninst, int maxNz, int nb, cudaStream_t st)
 {
-    const dim3 g((maxNz + 31) / 32, ninst);
-    if (fin_warp) return launch_first(finalize_cells_warp<T>, dim3((maxNz + 3) / 4, ninst), dim3(128), st, d_inst, stage);
-    if (nb <= 4) return launch_first(finalize_cells<T, 4>, g, dim3(32), st, d_inst, stage);
-    if (nb <= 6) return launch_first(finalize_cells<T, 6>, g, dim3(32), st, d_inst, stage);
-    return launch_first(finalize_cells<T, kMaxN>, g, dim3(32), st, d_inst, stage);
+    const dim3 g((maxNz + C - 1) / C, ninst), b(kThreads);
+    if (nb <= 4) return launch_first(finalize_cells<T, 4, C>, g, b, st, d_inst, stage);
+    if (nb <= 6) return launch_first(finalize_cells<T, 6, C>, g, b, st, d_inst, stage);
+    return launch_first(finalize_cells<T, kMaxN, C>, g, b, st, d_inst, stage);
+}
+
+template <int C>
+static cudaError_t launch_finalize_c(int fp32, int stage, const InstDev* d_inst, int ninst, int maxNz, int nb,
+                                     cudaStream_t st)
+{
+    return fp32 ? launch_finalize_t<float, C>(stage, d_inst, ninst, maxNz, nb, st)
+                : launch_finalize_t<double, C>(stage, d_inst, ninst, maxNz, nb, st);
 }
 
 // the stage kernel alone
@@ -199,22 +183,26 @@ cudaError_t launch_stage_only(int fp32, int red, int V, int stage, const InstDev
 }
 
 // the separate finalisation launches of an unfused stage
-cudaError_t launch_finalize(int fp32, int stage, const InstDev* d_inst, int ninst, int maxNz, int fin_warp,
+cudaError_t launch_finalize(int fp32, int stage, const InstDev* d_inst, int ninst, int maxNz, int fin_cells,
                             int nb, cudaStream_t st)
 {
-    return fp32 ? launch_finalize_t<float>(stage, d_inst, ninst, maxNz, fin_warp, nb, st)
-                : launch_finalize_t<double>(stage, d_inst, ninst, maxNz, fin_warp, nb, st);
+    switch (fin_cells) {
+        case 4: return launch_finalize_c<4>(fp32, stage, d_inst, ninst, maxNz, nb, st);
+        case 8: return launch_finalize_c<8>(fp32, stage, d_inst, ninst, maxNz, nb, st);
+        case 16: return launch_finalize_c<16>(fp32, stage, d_inst, ninst, maxNz, nb, st);
+        default: return launch_finalize_c<32>(fp32, stage, d_inst, ninst, maxNz, nb, st);
+    }
 }
 
 // one RK stage (stage 1..3) or the analysis pass (stage 0); without fusion the
 // finalisation follows as two more launches
 cudaError_t launch_stage(int fp32, int red, int V, int stage, const InstDev* d_inst, const Tile* d_tiles,
-                         int ntiles, size_t smem, int fuse, int ninst, int maxNz, int fin_warp, int nb,
+                         int ntiles, size_t smem, int fuse, int ninst, int maxNz, int fin_cells, int nb,
                          cudaStream_t st)
 {
     cudaError_t e = launch_stage_only(fp32, red, V, stage, d_inst, d_tiles, ntiles, smem, fuse, st);
     if (e != cudaSuccess || fuse) return e;
-    return launch_finalize(fp32, stage, d_inst, ninst, maxNz, fin_warp, nb, st);
+    return launch_finalize(fp32, stage, d_inst, ninst, maxNz, fin_cells, nb, st);
 }
 
 cudaError_t launch_seed_free_molecular(int fp32, const InstDev* d_inst, int inst, int Nz, cudaStream_t st)
@@ -227,9 +215,9 @@ cudaError_t launch_seed_free_molecular(int fp32, const InstDev* d_inst, int inst
 cudaError_t launch_seed(int fp32, const InstDev* d_inst, int inst, int Nz, const double* d_macro,
                         cudaStream_t st)
 {
-    const int g = (Nz + 63) / 64;
-    if (fp32) records_from_macro<float><<<g, 64, 0, st>>>(d_inst, inst, d_macro);
-    else records_from_macro<double><<<g, 64, 0, st>>>(d_inst, inst, d_macro);
+    const int g = (Nz + 3) / 4;
+    if (fp32) records_from_macro<float><<<g, kThreads, 0, st>>>(d_inst, inst, d_macro);
+    else records_from_macro<double><<<g, kThreads, 0, st>>>(d_inst, inst, d_macro);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (fp32) seed_cells<float><<<Nz, 128, 0, st>>>(d_inst, inst);

@@ -25,16 +25,13 @@
 //                    chunk in FP32 in FP32 mode; in FP64 in FP64 mode).  Tiles
 //                    that end at a wall also reduce the outgoing WENO flux of
 //                    F_out through the wall.
-//   finalisation     per cell: the sum of the chunks' partials (double-float in
-//                    FP32 mode, FP64 in FP64 mode), n, u, P, T, q (Eq. qdef),
-//                    tau, and the cell record of the next stage; per
+//   finalisation     (finalize.cuh) per cell: the sum of the chunks' partials, n, u, P, T, q
+//                    (Eq. qdef), tau, and the cell record of the next stage; per
 //                    instance: the wall densities n_w (zero net mass
 //                    flux, Appendix) and, after the third stage, the residual.
-//                    Either a launch of its own (finalize_cells, one thread per
-//                    cell, or finalize_cells_warp, one warp per cell, in
-//                    kernels.cu), or folded into the stage kernel (fuse = 1:
-//                    the CTA that ends last among the chunks of a z-tile does
-//                    its cells, threadfence tickets).
+//                    Either a launch of its own (finalize_cells in kernels.cu), or folded
+//                    into the stage kernel (fuse = 1: the CTA that ends last among the
+//                    chunks of a z-tile does its cells, threadfence tickets).
 //
 // Template parameter RED: the reduced phi / chi model of Sec. III (j = 0 phi,
 // j = 1 chi on a two-node transverse axis), otherwise the full 3D velocity set.
@@ -46,13 +43,10 @@
 
 #include <cstdint>
 
+#include "finalize.cuh"
 #include "lbs_internal.h"
 
 namespace lbs {
-
-template <typename T> struct Acc { typedef double type; };
-template <> struct Acc<float> { typedef float type; };
-
 
 // ---- PTX helpers: mbarrier and bulk global -> shared copies ------------------
 static __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -89,17 +83,6 @@ static __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t par
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     return ok != 0;
-}
-
-// 1 / x in FP64 for a finite normal x: the hardware's approximate reciprocal (relative error
-// below 2^-23) and two Newton steps r <- r + r (1 - x r), each squaring the relative error:
-// correct to an ulp in four FMAs, where the IEEE division takes about ten FP64 instructions.
-static __device__ __forceinline__ double rcp_newton(double x)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
 }
 
 // WENO-5 reconstruction of five upwind-ordered values (no advection factor), as the
@@ -180,33 +163,6 @@ __device__ __forceinline__ float weno5_corr<float>(float v0, float v1, float v2,
     return fmaf(w1, e1, fmaf(w2, e2, w3 * e3)) * inv;
 }
 
-// ---- packed FP32 (two lanes of f32x2 per instruction, each element rounded exactly as
-// the scalar operation) ----------------------------------------------------------------
-#define LBS_OP2(name, op)                                                                       \
-    static __device__ __forceinline__ float2 name(float2 a, float2 b)                           \
-    {                                                                                           \
-        float2 d;                                                                               \
-        asm("{.reg .b64 ra, rb, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n " op    \
-            " rd, ra, rb;\n mov.b64 {%0, %1}, rd;\n}"                                           \
-            : "=f"(d.x), "=f"(d.y)                                                              \
-            : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));                                          \
-        return d;                                                                               \
-    }
-LBS_OP2(add2, "add.rn.f32x2")
-LBS_OP2(sub2, "sub.rn.f32x2")
-LBS_OP2(mul2, "mul.rn.f32x2")
-#undef LBS_OP2
-static __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("{.reg .b64 ra, rb, rc, rd;\n mov.b64 ra, {%2, %3};\n mov.b64 rb, {%4, %5};\n mov.b64 rc, {%6, %7};\n"
-        " fma.rn.f32x2 rd, ra, rb, rc;\n mov.b64 {%0, %1}, rd;\n}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-static __device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
-
 // weno5_corr<float> for two velocities at once (the same operations, element by element;
 // the reciprocals and the multiplications by the scaled ideal weights stay scalar): about
 // half the issued arithmetic of two scalar calls
@@ -237,9 +193,6 @@ __device__ __forceinline__ T weno5(T v0, T v1, T v2, T v3, T v4)
     return v2 + weno5_corr<T>(v0, v1, v2, v3, v4);
 }
 
-template <typename T>
-__device__ __forceinline__ T ld(const void* p, int i) { return static_cast<const T*>(p)[i]; }
-
 // Block-wide FP64 sum (all threads get the result); deterministic order.
 static __device__ double block_sum(double v, double* red)
 {
@@ -253,31 +206,6 @@ static __device__ double block_sum(double v, double* red)
     __syncthreads();
     return s;
 }
-
-// N block sums at once (one pair of barriers for all of them); red holds
-// N * (blockDim.x / 32) doubles.  Each sum keeps block_sum's order.
-template <int N>
-__device__ void block_sum_n(double (&v)[N], double* red)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0)
-#pragma unroll
-        for (int i = 0; i < N; ++i) red[i * nw + w] = v[i];
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        double s = 0.0;
-        for (int j = 0; j < nw; ++j) s += red[i * nw + j];
-        v[i] = s;
-    }
-    __syncthreads();
-}
-constexpr int kRedSlots = 8 * (kThreads / 32);  // shared doubles for block_sum_n<8> with 128 threads
 
 // Warp reduce-scatter of 16 values: afterwards lane l holds the warp total of
 // value m(l) = 8 b4 + 4 b3 + 2 b2 + b1 (b = bits of l); lanes l, l^1 agree.
@@ -369,541 +297,6 @@ static __device__ __forceinline__ float lo_decode(unsigned q16, float hi)  // q 
     return q * s;
 }
 
-// ---- double-float arithmetic (an FP32 pair hi + lo, |lo| <= ulp(hi) / 2) for the
-// FP32 records' node sums.  On this GPU an FP64 instruction occupies a scheduler's
-// FP64 unit for about 70 cycles whatever the number of active lanes, FP32 instructions
-// issue every cycle: the error-free transforms below (Knuth's TwoSum, the FMA form of
-// TwoProduct, a Fast2Sum renormalisation) cost a few FP32 instructions per term and
-// carry about 2^-44 of the largest term, well inside the half ulp of FP32 the factors
-// are rounded to.
-struct DF {
-    float hi, lo;
-};
-static __device__ __forceinline__ DF df_of(double x)
-{
-    const float h = __double2float_rn(x);
-    return DF{h, __double2float_rn(x - double(h))};
-}
-static __device__ __forceinline__ void df_add(DF& S, float p, float e)  // S += p + e, |e| << |p|
-{
-    const float s = S.hi + p, bb = s - S.hi;
-    float t = (S.hi - (s - bb)) + (p - bb);  // TwoSum(S.hi, p)
-    t += S.lo + e;
-    S.hi = s + t;
-    S.lo = t - (S.hi - s);  // Fast2Sum
-}
-static __device__ __forceinline__ void df_fma(DF& S, DF c, float2 h)  // S += c h (h = (hi, lo))
-{
-    const float p = c.hi * h.x;
-    const float e = fmaf(c.hi, h.y, fmaf(c.lo, h.x, fmaf(c.hi, h.x, -p)));
-    df_add(S, p, e);
-}
-static __device__ __forceinline__ void df_add_prod(DF& S, float a, float b)  // S += a b, exact product
-{
-    const float p = a * b;
-    df_add(S, p, fmaf(a, b, -p));
-}
-
-// ----------------------------------------------------------------------------
-// Cell record of a macroscopic state: the scalars and the per-node factors of the
-// truncated Hermite equilibrium (Sec. III, Eqs. fyz, Fmn_def), computed in FP64 (the
-// half-range coefficients cancel strongly for N >= 4) and rounded once.  A factor's
-// deviation from 1 is sum_l (c_l - r_l) basis_l(node) with the rest state's
-// coefficients r: (1, 0, 0, ...) on x and y, (1, 1) on the reduced model's y (factors 1
-// and T), (1/2, 0, ...) on each half range of z, for which sum_l r_l basis_l = 1 at every
-// node.  R_SCALE makes the discrete equilibrium carry exactly n: in exact arithmetic
-// sum_i w_i Gx = 1, sum_j w_j Gy = 1 and the sum over both half ranges of w Gz = 1
-// (orthogonality of the bases); with the factors rounded to the storage type the sums
-// miss by a few ulps of the same sign every step, which would let FP32 runs drift in
-// mass, so the sums are taken over the stored values.  Returns false for a non-finite
-// or non-positive state (a neutral state is written instead).
-// ----------------------------------------------------------------------------
-template <typename T, int NB = kMaxN>
-__device__ bool write_record(const InstDev& I, int cell, double n, double in, const double* u, double T_,
-                             const double* q)
-{
-    // in = 1 / n (the callers have it); FP64 divisions are costly here, so 1/T is the
-    // only other one before R_SCALE
-    bool bad = !(n > 0.0) || !(T_ > 0.0) || !isfinite(n) || !isfinite(T_);
-    for (int a = 0; a < 3; ++a) bad |= !isfinite(u[a]) || !isfinite(q[a]);
-    const double nn = bad ? 1.0 : n, inn = bad ? 1.0 : in, Tc = bad ? 1.0 : T_;
-    const double u0 = bad ? 0.0 : u[0], u1 = bad ? 0.0 : u[1], u2 = bad ? 0.0 : u[2];
-    T* rec = static_cast<T*>(I.rec) + (size_t)cell * I.rec_stride;
-    const double iT = 1.0 / Tc;
-    rec[R_N] = T(nn); rec[R_UX] = T(u0); rec[R_UY] = T(u1); rec[R_UZ] = T(u2); rec[R_T] = T(Tc);
-    rec[R_QX] = T(bad ? 0.0 : q[0]); rec[R_QY] = T(bad ? 0.0 : q[1]); rec[R_QZ] = T(bad ? 0.0 : q[2]);
-    rec[R_ITAU] = T(inv_relax_time(I.visc_law, I.iKn, I.visc_param, I.isuth, nn, Tc, iT));
-    rec[R_CS] = T((1.0 - I.Pr) * inn * iT * iT);
-    rec[R_I5T] = T(0.2 * iT);
-    const int Qx = I.Qx, Qy = I.Qy, Qz = I.Qz;
-    T* dx = rec + R_DX;
-    T* dy = dx + Qx;
-    T* dz = dy + Qy;
-    double c[kMaxN + 1], cm[kMaxN + 1], s[3];
-    // x: a_l, l >= 1, against He_l / l!
-    full_coeffs<NB>(u0, Tc, I.Nx, c);
-    s[0] = 0.0;
-    if constexpr (sizeof(T) == 4) {  // FP32 records: the node sums in double-float
-        DF cd[NB + 1], sw = {0.f, 0.f};
-#pragma unroll
-        for (int l = 1; l <= NB; ++l) cd[l] = l <= I.Nx ? df_of(c[l]) : DF{0.f, 0.f};
-#pragma unroll 2
-        for (int i = 0; i < Qx; ++i) {
-            const float2* h = I.Hx2 + i * (I.Nx + 1);
-            DF g = {0.f, 0.f};
-#pragma unroll
-            for (int l = 1; l <= NB; ++l)
-                if (l <= I.Nx) df_fma(g, cd[l], h[l]);
-            const float v = g.hi + g.lo;
-            dx[i] = T(v);
-            df_add_prod(sw, ld<float>(I.wx, i), v);
-        }
-        s[0] = I.sumw_x + (double(sw.hi) + double(sw.lo));  // sum w (1 + v)
-    } else {
-#pragma unroll 4  // independent nodes: four FP64 chains in flight
-        for (int i = 0; i < Qx; ++i) {
-            const double* h = I.Hx + i * (I.Nx + 1);
-            double g = 0.0;
-#pragma unroll
-            for (int l = 1; l <= NB; ++l)
-                if (l <= I.Nx) g += c[l] * h[l];
-            const T v = T(g);
-            dx[i] = v;
-            s[0] += double(ld<T>(I.wx, i)) * (1.0 + double(v));
-        }
-    }
-    // y: the reduced model's factors 1 and T (phi and chi; its mass is phi's alone)
-    s[1] = 0.0;
-    if (I.reduced) {
-        dy[0] = T(0);
-        dy[1] = T(Tc - 1.0);
-        s[1] = 1.0;
-    } else {
-        full_coeffs<NB>(u1, Tc, I.Ny, c);
-        if constexpr (sizeof(T) == 4) {
-            DF cd[NB + 1], sw = {0.f, 0.f};
-#pragma unroll
-            for (int l = 1; l <= NB; ++l) cd[l] = l <= I.Ny ? df_of(c[l]) : DF{0.f, 0.f};
-#pragma unroll 2
-            for (int j = 0; j < Qy; ++j) {
-                const float2* h = I.Hy2 + j * (I.Ny + 1);
-                DF g = {0.f, 0.f};
-#pragma unroll
-                for (int l = 1; l <= NB; ++l)
-                    if (l <= I.Ny) df_fma(g, cd[l], h[l]);
-                const float v = g.hi + g.lo;
-                dy[j] = T(v);
-                df_add_prod(sw, ld<float>(I.wy, j), v);
-            }
-            s[1] = I.sumw_y + (double(sw.hi) + double(sw.lo));
-        } else {
-#pragma unroll 4
-            for (int j = 0; j < Qy; ++j) {
-                const double* h = I.Hy + j * (I.Ny + 1);
-                double g = 0.0;
-#pragma unroll
-                for (int l = 1; l <= NB; ++l)
-                    if (l <= I.Ny) g += c[l] * h[l];
-                const T v = T(g);
-                dy[j] = v;
-                s[1] += double(ld<T>(I.wy, j)) * (1.0 + double(v));
-            }
-        }
-    }
-    // z: b_l on each half range against pi_l / h_l, b_0 - 1/2 in place of b_0
-    half_coeffs_pm<NB>(u2, Tc, iT, I.Nzq, I.alpha, I.beta, c, cm);
-    c[0] -= 0.5;
-    cm[0] -= 0.5;
-    s[2] = 0.0;
-    if constexpr (sizeof(T) == 4) {
-        DF bp[NB + 1], bm[NB + 1], sw = {0.f, 0.f};
-#pragma unroll
-        for (int l = 0; l <= NB; ++l) {
-            bp[l] = l <= I.Nzq ? df_of(c[l]) : DF{0.f, 0.f};
-            bm[l] = l <= I.Nzq ? df_of(cm[l]) : DF{0.f, 0.f};
-        }
-        for (int m = 0; m < Qz; ++m) {
-            const float2* h = I.Pz2 + m * (I.Nzq + 1);
-            DF gp = {0.f, 0.f}, gm = {0.f, 0.f};
-#pragma unroll
-            for (int l = 0; l <= NB; ++l)
-                if (l <= I.Nzq) {
-                    df_fma(gp, bp[l], h[l]);
-                    df_fma(gm, bm[l], h[l]);
-                }
-            const float vp = gp.hi + gp.lo, vm = gm.hi + gm.lo;
-            dz[m] = T(vp);
-            dz[Qz + m] = T(vm);
-            const float w = ld<float>(I.wz, m);
-            df_add_prod(sw, w, vp);
-            df_add_prod(sw, w, vm);
-        }
-        s[2] = I.sumw_z + (double(sw.hi) + double(sw.lo));  // sum over both half ranges
-    } else {
-#pragma unroll 2
-        for (int m = 0; m < Qz; ++m) {
-            const double* h = I.Pz + m * (I.Nzq + 1);
-            double gp = 0.0, gm = 0.0;
-#pragma unroll
-            for (int l = 0; l <= NB; ++l)
-                if (l <= I.Nzq) {
-                    gp += c[l] * h[l];
-                    gm += cm[l] * h[l];
-                }
-            const T vp = T(gp), vm = T(gm);
-            dz[m] = vp;
-            dz[Qz + m] = vm;
-            s[2] += double(ld<T>(I.wz, m)) * ((1.0 + double(vp)) + (1.0 + double(vm)));
-        }
-    }
-    rec[R_SCALE1] = T(nn / (s[0] * s[1] * s[2]) - 1.0);
-    return !bad;
-}
-
-// profiles [14][Nz] and W = (n, u_x, T) of a cell; false if any value is not finite
-static __device__ __forceinline__ bool store_cell(const InstDev& I, int cell, const CellState& c)
-{
-    const int Nz = I.Nz;
-    const double vals[14] = {c.n, c.u[0], c.u[1], c.u[2], c.T, c.q[0], c.q[1], c.q[2],
-                             c.P[0], c.P[1], c.P[2], c.P[3], c.P[4], c.P[5]};
-    bool bad = false;
-#pragma unroll
-    for (int a = 0; a < 14; ++a) {
-        I.prof[(size_t)a * Nz + cell] = vals[a];
-        bad |= !isfinite(vals[a]);
-    }
-    I.Wnew[cell] = c.n;
-    I.Wnew[Nz + cell] = c.u[0];
-    I.Wnew[2 * Nz + cell] = c.T;
-    return !bad;
-}
-
-// The velocity the stage kernel took its moments about: the u of the cell's record of
-// the stage (still in place when the finalisation reads it); 0 for the analysis pass.
-template <typename T>
-__device__ __forceinline__ void moment_origin(const InstDev& I, int cell, int stage, double* ur)
-{
-    const T* rc = static_cast<const T*>(I.rec) + (size_t)cell * I.rec_stride;
-    ur[0] = stage > 0 ? double(rc[R_UX]) : 0.0;
-    ur[1] = stage > 0 ? double(rc[R_UY]) : 0.0;
-    ur[2] = stage > 0 ? double(rc[R_UZ]) : 0.0;
-}
-
-// The macroscopic state from the partials' moments about ur (sums over the deviations
-// d) and the rest state's moments, re-expressed about ur: n, u = ur + the mean of
-// p - ur, P, T and q.
-static __device__ __forceinline__ void state_about(const InstDev& I, double* mom, const double* ur, CellState& st)
-{
-    double rest[kNMom];
-    shift_moments(I.mrest, ur, rest);
-#pragma unroll
-    for (int a = 0; a < kNMom; ++a) mom[a] += rest[a];
-    cell_state(mom, st);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) st.u[a] += ur[a];
-}
-
-// One cell (one thread): the sum of the per-chunk moment partials (written by other
-// CTAs of this launch, hence read past L1; FP32 partials in double-float, FP64 ones in
-// FP64), the macroscopic state, the profiles, W for the residual, and the cell record
-// of the next stage.
-template <typename T, int NB = kMaxN>
-__device__ __noinline__ void finalize_cell(const InstDev& I, int cell, int stage)
-{
-    const int Nz = I.Nz, nch = I.nchunks;
-    typedef typename Acc<T>::type A;
-    const A* part = static_cast<const A*>(I.partial);
-    double mom[kNMom];  // the partials: moments of the deviations about ur
-    // chunks in order, four at a time with every load issued before the adds (the
-    // partials come from L2: one round trip per four chunks instead of per chunk);
-    // FP32 partials summed in double-float (no FP64 instruction per chunk)
-    DF md[kNMom];
-    for (int a = 0; a < kNMom; ++a) {
-        mom[a] = 0.0;
-        md[a] = DF{0.f, 0.f};
-    }
-    for (int c = 0; c < nch; c += 4) {
-        A p[4][kNMom];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int a = 0; a < kNMom; ++a)
-                p[j][a] = c + j < nch ? __ldcg(part + ((size_t)(c + j) * kNMom + a) * Nz + cell) : A(0);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int a = 0; a < kNMom; ++a)
-                if (c + j < nch) {
-                    if constexpr (sizeof(A) == 4) df_add(md[a], p[j][a], 0.f);
-                    else mom[a] += p[j][a];
-                }
-    }
-    if constexpr (sizeof(A) == 4)
-        for (int a = 0; a < kNMom; ++a) mom[a] = double(md[a].hi) + double(md[a].lo);
-    double ur[3];
-    moment_origin<T>(I, cell, stage, ur);
-    CellState st;
-    state_about(I, mom, ur, st);
-    bool bad = !store_cell(I, cell, st);
-    bad |= !write_record<T, NB>(I, cell, st.n, st.in, st.u, st.T, st.q);
-    if (bad) atomicOr(I.status, STATUS_NONFINITE);
-}
-
-// ---- one cell per warp: the same record with its FP64 work spread over the lanes.
-// FP64 instructions issue at a small fraction of the FP32 rate, so with one thread
-// per cell a small batch waits on each cell's long FP64 chain; here lane a sums
-// moment a, the two halves of the warp run the x / y coefficient recurrences and
-// the p_z > 0 / p_z < 0 half-range tables side by side, within a half lane k
-// carries column k of the table J_{l,k} (one shuffle per row instead of the whole
-// triangle in one thread), and the nodes' factors are spread over the lanes.  Large
-// batches keep one thread per cell, where every lane has a cell of its own.
-template <typename T>
-__device__ bool write_record_warp(const InstDev& I, int cell, const CellState& st, int lane)
-{
-    // the half-range recurrence coefficients, loaded ahead of the chain that needs them
-    double al[kMaxN], be[kMaxN];
-#pragma unroll
-    for (int l = 0; l < kMaxN; ++l) {
-        al[l] = I.alpha[l];
-        be[l] = I.beta[l];
-    }
-    bool bad = !(st.n > 0.0) || !(st.T > 0.0) || !isfinite(st.n) || !isfinite(st.T);
-    for (int a = 0; a < 3; ++a) bad |= !isfinite(st.u[a]) || !isfinite(st.q[a]);
-    const double nn = bad ? 1.0 : st.n, inn = bad ? 1.0 : st.in, Tc = bad ? 1.0 : st.T;
-    const double u0 = bad ? 0.0 : st.u[0], u1 = bad ? 0.0 : st.u[1], u2 = bad ? 0.0 : st.u[2];
-    T* rec = static_cast<T*>(I.rec) + (size_t)cell * I.rec_stride;
-    const double iT = 1.0 / Tc;
-    if (lane == 0) {
-        rec[R_N] = T(nn); rec[R_UX] = T(u0); rec[R_UY] = T(u1); rec[R_UZ] = T(u2); rec[R_T] = T(Tc);
-        rec[R_QX] = T(bad ? 0.0 : st.q[0]); rec[R_QY] = T(bad ? 0.0 : st.q[1]); rec[R_QZ] = T(bad ? 0.0 : st.q[2]);
-        rec[R_ITAU] = T(inv_relax_time(I.visc_law, I.iKn, I.visc_param, I.isuth, nn, Tc, iT));
-        rec[R_CS] = T((1.0 - I.Pr) * inn * iT * iT);
-        rec[R_I5T] = T(0.2 * iT);
-    }
-    const int Qx = I.Qx, Qy = I.Qy, Qz = I.Qz;
-    T* dx = rec + R_DX;
-    T* dy = dx + Qx;
-    T* dz = dy + Qy;
-    const int h = lane >> 4, k = lane & 15;  // half of the warp, lane within it
-    // x (h = 0) and y (h = 1) coefficients a_l (Eq. fyz), in every lane of the half
-    double c[kMaxN + 1];
-    const int Nh = h ? I.Ny : I.Nx;
-    full_coeffs(h ? u1 : u0, Tc, Nh, c);
-    // z: half h = 0 the p_z > 0 range (drift u2), h = 1 the p_z < 0 range written in
-    // xi = -p_z >= 0 (drift -u2).  Both share g(0) and one erfc (erfc(x) + erfc(-x) = 2).
-    const int K = I.Nzq;
-    // 1 / sqrt(2T) straight from T, so that the transcendental chain does not wait for
-    // the division 1 / T; with x = |u2| / sqrt(2T): g(0) = exp(-x^2) / sqrt(2 pi T)
-    const double r2T = rsqrt(2.0 * Tc), x = fabs(u2) * r2T;
-    const double g0 = exp(-x * x) * (r2T * (1.0 / sqrt(M_PI)));
-    const double e = erfc_nonneg(x);
-    const double us = h ? -u2 : u2;
-    const double J00 = (u2 >= 0.0) != (h == 1) ? 1.0 - 0.5 * e : 0.5 * e;  // erfc(-us / sqrt(2T)) / 2
-    // J_{0,k}: the half-line Gaussian moments M_k, M_{k+1} = us M_k + k T M_{k-1}
-    double mp = J00, mc = us * J00 + Tc * g0;
-    double Jc = k == 0 ? J00 : (k == 1 ? mc : 0.0);
-#pragma unroll
-    for (int kk = 1; kk < kMaxN; ++kk)
-        if (kk < K) {
-            const double mn = us * mc + kk * Tc * mp;
-            mp = mc;
-            mc = mn;
-            if (k == kk + 1) Jc = mn;
-        }
-    // rows J_{l+1,k} = J_{l,k+1} - alpha_l J_{l,k} - beta_l J_{l-1,k}; b_l = J_{l,0}.
-    // Column k holds a valid entry for k <= K - l; the others never reach column 0.
-    double Jp = 0.0, b[kMaxN + 1];
-    b[0] = Jc;
-#pragma unroll
-    for (int l = 0; l < kMaxN; ++l) {
-        b[l + 1] = 0.0;
-        if (l < K) {
-            const double up = __shfl_down_sync(0xffffffffu, Jc, 1, 16);
-            const double Jn = up - al[l] * Jc - (l > 0 ? be[l] * Jp : 0.0);
-            Jp = Jc;
-            Jc = Jn;
-            b[l + 1] = Jc;
-        }
-    }
-    // column 0 (lanes 0 and 16) holds the two coefficient sets: give them to every lane,
-    // b_0 - 1/2 in place of b_0 (the rest state's coefficient)
-    double bp[kMaxN + 1], bm[kMaxN + 1];
-#pragma unroll
-    for (int l = 0; l <= kMaxN; ++l) {
-        bp[l] = __shfl_sync(0xffffffffu, b[l], 0) - (l == 0 ? 0.5 : 0.0);
-        bm[l] = __shfl_sync(0xffffffffu, b[l], 16) - (l == 0 ? 0.5 : 0.0);
-    }
-    // the nodes' factors: x over the lanes of half 0, y over half 1, z over the warp;
-    // each lane's terms of the R_SCALE sums
-    double sxy = 0.0, sz = 0.0;
-    if (h == 0) {
-        for (int i = k; i < Qx; i += 16) {
-            const double* hb = I.Hx + i * (I.Nx + 1);
-            double g = 0.0;
-#pragma unroll
-            for (int l = 1; l <= kMaxN; ++l)
-                if (l <= I.Nx) g += c[l] * hb[l];
-            const T v = T(g);
-            dx[i] = v;
-            sxy += double(ld<T>(I.wx, i)) * (1.0 + double(v));
-        }
-    } else if (I.reduced) {  // y factors of phi and chi: 1 and T; the mass is phi's alone
-        if (k == 0) {
-            dy[0] = T(0);
-            dy[1] = T(Tc - 1.0);
-            sxy = 1.0;
-        }
-    } else {
-        for (int j = k; j < Qy; j += 16) {
-            const double* hb = I.Hy + j * (I.Ny + 1);
-            double g = 0.0;
-#pragma unroll
-            for (int l = 1; l <= kMaxN; ++l)
-                if (l <= I.Ny) g += c[l] * hb[l];
-            const T v = T(g);
-            dy[j] = v;
-            sxy += double(ld<T>(I.wy, j)) * (1.0 + double(v));
-        }
-    }
-    for (int m = lane; m < Qz; m += 32) {
-        const double* hb = I.Pz + m * (I.Nzq + 1);
-        double gp = 0.0, gm = 0.0;
-#pragma unroll
-        for (int l = 0; l <= kMaxN; ++l)
-            if (l <= K) {
-                gp += bp[l] * hb[l];
-                gm += bm[l] * hb[l];
-            }
-        const T vp = T(gp), vm = T(gm);
-        dz[m] = vp;
-        dz[Qz + m] = vm;
-        sz += double(ld<T>(I.wz, m)) * ((1.0 + double(vp)) + (1.0 + double(vm)));
-    }
-    // R_SCALE = n / (s_x s_y s_z) (see write_record)
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) sxy += __shfl_xor_sync(0xffffffffu, sxy, o, 16);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sz += __shfl_xor_sync(0xffffffffu, sz, o);
-    const double sx = __shfl_sync(0xffffffffu, sxy, 0), sy = __shfl_sync(0xffffffffu, sxy, 16);
-    if (lane == 0) rec[R_SCALE1] = T(nn / (sx * sy * sz) - 1.0);
-    return !bad;
-}
-
-template <typename T>
-__device__ __noinline__ void finalize_cell_warp(const InstDev& I, int cell, int lane, int stage)
-{
-    const int Nz = I.Nz, nch = I.nchunks, am = lane & 15, h = lane >> 4;
-    // moment am: lanes am and 16 + am sum the even and the odd chunks (loads four
-    // chunks ahead), then add the two halves
-    double part = 0.0;
-    if (am < kNMom)
-        for (int c = h; c < nch; c += 8) {
-            double p[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                p[j] = c + 2 * j < nch
-                           ? double(__ldcg(static_cast<const typename Acc<T>::type*>(I.partial) +
-                                           ((size_t)(c + 2 * j) * kNMom + am) * Nz + cell))
-                           : 0.0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (c + 2 * j < nch) part += p[j];
-        }
-    part += __shfl_down_sync(0xffffffffu, part, 16);
-    double mom[kNMom];
-#pragma unroll
-    for (int a = 0; a < kNMom; ++a) mom[a] = __shfl_sync(0xffffffffu, part, a);
-    double ur[3];
-    moment_origin<T>(I, cell, stage, ur);
-    CellState st;
-    state_about(I, mom, ur, st);
-    bool bad = false;
-    if (lane == 0) bad = !store_cell(I, cell, st);
-    bad |= !write_record_warp<T>(I, cell, st, lane);
-    if (bad && lane == 0) atomicOr(I.status, STATUS_NONFINITE);
-}
-
-// One instance (whole CTA): wall densities n_w from the outgoing wall fluxes
-// (zero net mass flux, Appendix); after stage 3 the residual, the step count
-// and retirement; after the analysis pass W_old = W.
-static __device__ __noinline__ void finalize_instance(const InstDev& I, int stage, double* red)
-{
-    // red: kRedSlots doubles.  The wall fluxes and (stage 3) the residual's sums
-    // ||W_new - W_old||^2, ||W_old||^2 for n, u_x, T are reduced together.
-    const int t = threadIdx.x, Nz = I.Nz;
-    double v[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = 0.0;
-    for (int c = t; c < I.nchunks; c += blockDim.x) {
-        v[0] += __ldcg(I.flux_part + 2 * c);
-        v[1] += __ldcg(I.flux_part + 2 * c + 1);
-    }
-    if (stage == 3) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            for (int s = t; s < Nz; s += blockDim.x) {
-                const double wn = __ldcg(I.Wnew + a * Nz + s), wo = I.Wold[a * Nz + s];
-                v[2 + 2 * a] += (wn - wo) * (wn - wo);
-                v[3 + 2 * a] += wo * wo;
-            }
-        block_sum_n<8>(v, red);
-    } else {
-        double w[2] = {v[0], v[1]};
-        block_sum_n<2>(w, red);
-        v[0] = w[0];
-        v[1] = w[1];
-    }
-    if (t == 0) {  // the partials sum w p_z over the deviations: add the rest state's flux
-        I.nw[0] = -(I.frest_bot + v[0]) / I.Dbot;
-        I.nw[1] = -(I.frest_top + v[1]) / I.Dtop;
-        if (!isfinite(I.nw[0]) || !isfinite(I.nw[1])) atomicOr(I.status, STATUS_NONFINITE);
-    }
-    if (stage == 3) {
-        double R = 0.0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)  // the velocity on the wall speed where u_x is smaller
-            R = fmax(R, sqrt(v[2 + 2 * a]) / fmax(sqrt(v[3 + 2 * a]), a == 1 ? I.res_uscale : 1e-30));
-        // every W_old read above is complete (block_sum_n ends with a barrier)
-        for (int e = t; e < 3 * Nz; e += blockDim.x) I.Wold[e] = __ldcg(I.Wnew + e);
-        if (t == 0) {
-            *I.res = R;
-            *I.steps += 1;
-            *I.cur ^= 1;  // the new state was written over the stage-1 increment
-            if (!(R == R)) atomicOr(I.status, STATUS_NONFINITE);
-            if (I.tol > 0.0 && R < I.tol) *I.active = 0;
-        }
-    } else if (stage == 0) {
-        for (int e = t; e < 3 * Nz; e += blockDim.x) I.Wold[e] = __ldcg(I.Wnew + e);
-    }
-}
-
-// records from given macroscopic profiles macro[8][Nz] = n, ux, uy, uz, T, qx, qy, qz
-template <typename T>
-__global__ void records_from_macro(const InstDev* __restrict__ insts, int inst, const double* __restrict__ macro)
-{
-    const InstDev& I = insts[inst];
-    const int Nz = I.Nz, cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= Nz) return;
-    const double u[3] = {macro[Nz + cell], macro[2 * Nz + cell], macro[3 * Nz + cell]};
-    const double q[3] = {macro[5 * Nz + cell], macro[6 * Nz + cell], macro[7 * Nz + cell]};
-    if (!write_record<T>(I, cell, macro[cell], 1.0 / macro[cell], u, macro[4 * Nz + cell], q))
-        atomicOr(I.status, STATUS_NONFINITE);
-}
-
-// The instance descriptor copied into shared memory by the whole block at once: its
-// fields (pointers, orders, wall sums) are then one shared load away instead of an
-// L2 round trip each at first use -- in the stage kernel's prologue (pointer, then
-// table, then value) and inside the finalisation's FP64 chains.
-static __device__ __forceinline__ const InstDev& stage_descriptor(const InstDev* g, InstDev* s)
-{
-    static_assert(sizeof(InstDev) % 8 == 0, "descriptor copied in 8-byte words");
-    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(g);
-    unsigned long long* dst = reinterpret_cast<unsigned long long*>(s);
-    for (int e = threadIdx.x; e < (int)(sizeof(InstDev) / 8); e += blockDim.x) dst[e] = src[e];
-    __syncthreads();
-    return *s;
-}
-
 // ----------------------------------------------------------------------------
 // stage_kernel<T, V, STAGE, RED>: STAGE 1..3 are the RK stages; STAGE 0 only
 // analyses F0 (moments and wall fluxes) without writing F.  RED selects the
@@ -927,7 +320,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     constexpr bool kD = STAGE >= 2;       // the stage input is d + an increment
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
-    __shared__ double wall_red[kRedSlots];
+    __shared__ double wall_red[8 * (kThreads / 32)];
     __shared__ InstDev sI;
     const Tile tile = tiles[blockIdx.x];
     const InstDev& I = stage_descriptor(insts + tile.inst, &sI);
@@ -1622,11 +1015,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    if (I.fin_warp) {
-        for (int c = tid >> 5; c < zn; c += kThreads / 32) finalize_cell_warp<T>(I, z0 + c, tid & 31, STAGE);
-    } else if (tid < zn) {
-        finalize_cell<T>(I, z0 + tid, STAGE);
-    }
+    finalize_tile<T>(I, z0, zn, STAGE, *reinterpret_cast<FinShared<T, 4>*>(smem_raw));  // the rows are done with
     if (tid == 0) I.zcount[tile.zt] = 0;
     __threadfence();
     __syncthreads();

@@ -46,16 +46,16 @@ struct InstDev {
     int nchunks, bulk;            // bulk: rows are 16-byte aligned, stage them with TMA bulk copies
     int nchh;                     // chunks per half range of p_z (chunk c has p_z < 0 iff c >= nchh)
     int half;                     // 1: half channel, bounce-back ghosts below cell 0 (no bottom wall)
-    int fin_warp;                 // finalisation with one warp per cell (small batches) instead of one thread
     int reduced;                  // 1: the phi / chi model (Qy = 2: j = 0 phi, j = 1 chi; p_y unused)
     int visc_law;
     double Kn, visc_param, Pr, dt, tol;
     double res_uscale;            // the residual's velocity scale max(|u_w| sqrt(Nz), 1e-30)
     double iKn, isuth;            // 1 / Kn; Sutherland: 1 / (1 + S)
-    double Dtop, Dbot;            // sum over incoming velocities of w p_z Gw (n_w = 1)
+    double iDtop, iDbot;          // 1 / the sum over incoming velocities of w p_z Gw (n_w = 1)
     int rec_stride;               // values per cell record
     double mrest[kNMom];          // raw moments of the rest state f = w (the stored weights and
                                   // nodes): the partials hold sums over the deviations only
+    float mrest2[kNMom][2];       // the same as FP32 (hi, lo) pairs
     double frest_bot, frest_top;  // outgoing wall flux of the rest state (sum w p_z over the
                                   // velocities leaving through each wall)
     unsigned wait_limit;          // spins of the bounded wait for the bulk copies
@@ -65,8 +65,9 @@ struct InstDev {
     const double *Hx, *Hy, *Pz;   // FP64, [Q_a][N_a + 1] basis values He_l/l!, pi_l/h_l
     const float2 *Hx2, *Hy2, *Pz2;  // the same as FP32 (hi, lo) pairs, hi + lo = the FP64 value
                                     // to 2^-48 (FP32 storage: the records' node sums)
-    double sumw_x, sumw_y, sumw_z;  // sums of the stored weights (z: over both half ranges)
-    const double *alpha, *beta;   // half-range recurrence, [kMaxN + 2]
+    double sumw[3];                 // sums of the stored weights of x, y, z (z: over both half ranges)
+    float sumw2[3][2];              // the same as FP32 (hi, lo) pairs
+    const double* half_poly;        // [kMaxN + 1][kMaxN + 1]: row l the coefficients of the monic pi_l
     // storage-typed tables (float or double)
     const void *px, *py, *xi, *wx, *wy, *wz;
     const void *gwx_top, *gwx_bot, *gwy, *gwz;  // wall equilibria per axis (Q_x, Q_x, Q_y, 2Q_z),
@@ -176,57 +177,6 @@ LBS_HD double erfc_nonneg(double x)
 #pragma unroll
     for (int n = 12; n >= 0; --n) p = fma(p, t, S.c[n]);
     return 1.0 - x * p;
-}
-
-// Both half-range coefficient sets at once: bp for u, bm for -u (the p_z < 0 half
-// range, written in xi = -p_z >= 0).  The two share g(0) and, through
-// erfc(x) + erfc(-x) = 2, one erfc: the one of |x| is evaluated (no cancellation)
-// and the other is 2 minus it (a value in [1, 2], exact to an ulp).
-template <int NB = kMaxN>
-LBS_HD void half_coeffs_pm(double u, double T, double iT, int N, const double* alpha, const double* beta,
-                           double* bp, double* bm)
-{
-    // iT = 1 / T, which the caller has at hand.  Rows J_{l,k} (k <= N - l) of the two
-    // recurrences; only rows l - 1 and l are kept.
-    const int K = N;
-    const double r2T = sqrt(0.5 * iT);
-    const double g0 = exp(-0.5 * u * u * iT) * (r2T * (1.0 / sqrt(M_PI)));
-    const double e = erfc_nonneg(fabs(u) * r2T);  // erfc of the non-negative argument
-    double Pp[kMaxN + 1], Pc[kMaxN + 1], Mp[kMaxN + 1], Mc[kMaxN + 1];
-    Pc[0] = u >= 0.0 ? 1.0 - 0.5 * e : 0.5 * e;  // erfc(-u / sqrt(2T)) / 2
-    Mc[0] = u >= 0.0 ? 0.5 * e : 1.0 - 0.5 * e;  // erfc(u / sqrt(2T)) / 2
-    Pc[1] = u * Pc[0] + T * g0;                  // used only when K >= 1
-    Mc[1] = -u * Mc[0] + T * g0;
-    LBS_UNROLL
-    for (int k = 1; k < NB; ++k)
-        if (k < K) {
-            Pc[k + 1] = u * Pc[k] + k * T * Pc[k - 1];
-            Mc[k + 1] = -u * Mc[k] + k * T * Mc[k - 1];
-        }
-    bp[0] = Pc[0];
-    bm[0] = Mc[0];
-    LBS_UNROLL
-    for (int l = 0; l < NB; ++l) {
-        if (l < N) {
-            const double al = alpha[l], be = l > 0 ? beta[l] : 0.0;
-            double Pn[kMaxN + 1], Mn[kMaxN + 1];
-            LBS_UNROLL
-            for (int k = 0; k + l + 1 <= NB; ++k)
-                if (k + l + 1 <= K) {
-                    Pn[k] = Pc[k + 1] - al * Pc[k] - (l > 0 ? be * Pp[k] : 0.0);
-                    Mn[k] = Mc[k + 1] - al * Mc[k] - (l > 0 ? be * Mp[k] : 0.0);
-                }
-            LBS_UNROLL
-            for (int k = 0; k + l + 1 <= NB; ++k) {
-                Pp[k] = Pc[k];
-                Pc[k] = Pn[k];
-                Mp[k] = Mc[k];
-                Mc[k] = Mn[k];
-            }
-            bp[l + 1] = Pc[0];
-            bm[l + 1] = Mc[0];
-        }
-    }
 }
 
 // Macroscopic state of a cell from its 13 raw moments (FP64): n, u, the central

@@ -363,7 +363,7 @@ class Solver:
         return dict(zip(PROFILE_NAMES, a))
 
     def set_finalize(self, mode):
-        """0 auto, 1 one thread per cell, 2 one warp per cell; returns True if the warp layout is used."""
+        """0 auto, 1 at least eight cells per CTA, 2 four cells; returns True if the four-cell layout is used."""
         w = C.c_int()
         _check(self.lib.lbs_set_finalize(self.h, int(mode), C.byref(w)))
         return bool(w.value)

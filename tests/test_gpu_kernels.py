@@ -37,3 +37,25 @@ def test_fp64_weno_weights_at_vanishing_indicators(pattern):
     s.step(1)
     o.step(1)
     assert rel_err(gpu_f(s, o), o.f[3:3 + o.Nz]) < 1e-13
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("Nz,n", [(9, 1), (4093, 2), (4095, 3), (4093, 7)])
+@pytest.mark.parametrize("reduced", [False, True])
+def test_finalize_cells_per_cta_agree(Nz, n, reduced, prec, tol):
+    """The finalisation at 8, 16 and 32 cells per CTA (batches of 9, 8186, 12285 and 28651
+    cells: ragged last groups) gives the states and profiles of four cells per CTA to
+    rounding (FP64: a few ulps of the third moments; FP32 storage: the records' FP32)."""
+    P = _lbs()
+    from paper_1702_01335_gb300 import Instance, Solver
+    pr = P.LBS_FP64 if prec == "fp64" else P.LBS_FP32
+    inst = [Instance(Qx=3, Qy=0 if reduced else 2, Qz=2 + b % 3, N_eq=3, Nz=Nz - b % 2, Kn=0.2 + 0.1 * b, u_w=0.3,
+                     Pr=2.0 / 3.0, visc_law=b % 2, visc_param=0.75, cfl=0.4) for b in range(n)]
+    a, b = Solver(inst, precision=pr), Solver(inst, precision=pr)
+    assert not a.set_finalize(1) and b.set_finalize(2)
+    a.step(9)
+    b.step(9)
+    for i in range(n):
+        assert rel_err(a.populations(i), b.populations(i)) < tol, i
+        pa, pb = a.profiles(i), b.profiles(i)
+        assert max(np.abs(pa[k] - pb[k]).max() for k in pa) < tol, i
