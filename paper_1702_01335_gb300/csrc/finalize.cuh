@@ -35,6 +35,16 @@ namespace lbs {
 template <typename T> struct Acc { typedef double type; };
 template <> struct Acc<float> { typedef float type; };
 
+// Programmatic dependent launch: the stage and finalisation kernels of a stream start while
+// their predecessor finishes, do what depends on constants only (descriptor, tables,
+// per-velocity values), and wait before they touch anything that a kernel writes.  Every CTA
+// waits, also one that then leaves at once, so that a kernel's completion implies that of
+// all before it.  A kernel releases its successor late (the stage kernel after its march, the
+// finalisation after the cell state): released at the start, the successors of successors
+// pile up on the SMs too and a step of the low-Mach runs takes 172 us instead of 115.
+static __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
+static __device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <typename T>
 __device__ __forceinline__ T ld(const void* p, int i) { return static_cast<const T*>(p)[i]; }
 
@@ -302,36 +312,45 @@ __device__ __forceinline__ void half_line_moments(double u, double T_, int K, do
     for (int k = 1; k < NB; ++k) M[k + 1] = k < K ? fma(u, M[k], (k * T_) * M[k - 1]) : 0.0;
 }
 
-// ---- terms and nodes of the record: cells c0 .. c0 + nc - 1, their state in sm; PROF: also
-// the profiles and W
-template <typename T, int NB, int C, bool PROF>
-__device__ __forceinline__ void record_cells(const InstDev& I, int c0, int nc, FinShared<T, C>& sm, int vt)
-{
-    typedef Real<T> RT;
-    typedef typename RT::type R;
-    typedef typename RT::basis B;
-    constexpr int L = kThreads / C;  // lanes of a cell in the node phase
-    const int warp = vt >> 5, lane = vt & 31;
-    // the nodes of x and y and the node pairs of z; the basis row of this thread's first one
-    // is loaded before the coefficients exist
-    const int Qx = I.Qx, Qy = I.Qy, Qz = I.Qz, G = Qx + Qy + Qz;
-    const int cell = vt / L, j = vt % L;
-    auto load_row = [&](int r, B(&h)[NB + 1], T& w, int& ax) {
+// A node of x or y, or a pair of nodes of z: its basis row, weight and axis
+template <typename T, int NB>
+struct Node {
+    typename Real<T>::basis h[NB + 1];
+    T w;
+    int ax;
+    __device__ __forceinline__ Node() : w(T(0)), ax(0)
+    {
+#pragma unroll
+        for (int l = 0; l <= NB; ++l) h[l] = typename Real<T>::basis();
+    }
+    __device__ __forceinline__ int order(const InstDev& I) const { return ax == 0 ? I.Nx : ax == 1 ? I.Ny : I.Nzq; }
+    __device__ __forceinline__ void load(const InstDev& I, int r)
+    {
+        typedef Real<T> RT;
+        const int Qx = I.Qx, Qy = I.Qy;
+        if (r >= Qx + Qy + I.Qz) return;
         ax = r < Qx ? 0 : r < Qx + Qy ? 1 : 2;
-        const int N = ax == 0 ? I.Nx : ax == 1 ? I.Ny : I.Nzq, k = ax == 0 ? r : ax == 1 ? r - Qx : r - Qx - Qy;
-        const B* row = (ax == 0 ? RT::Hx(I) : ax == 1 ? RT::Hy(I) : RT::Pz(I)) + k * (N + 1);
+        const int N = order(I), k = ax == 0 ? r : ax == 1 ? r - Qx : r - Qx - Qy;
+        const typename RT::basis* row = (ax == 0 ? RT::Hx(I) : ax == 1 ? RT::Hy(I) : RT::Pz(I)) + k * (N + 1);
 #pragma unroll
         for (int l = 0; l <= NB; ++l)
             if (l <= N) h[l] = row[l];
         w = ld<T>(ax == 0 ? I.wx : ax == 1 ? I.wy : I.wz, k);
-    };
-    B h[NB + 1], hn[NB + 1];
-#pragma unroll
-    for (int l = 0; l <= NB; ++l) h[l] = hn[l] = B();
-    T w = T(0), wn = T(0);
-    int ax = 0, axn = 0;
-    if (j < G) load_row(j, h, w, ax);
+    }
+};
 
+// ---- terms and nodes of the record: cells c0 .. c0 + nc - 1, their state in sm; node: this
+// thread's first one, loaded (it does not depend on the state); PROF: also the profiles and W
+template <typename T, int NB, int C, bool PROF>
+__device__ __forceinline__ void record_cells(const InstDev& I, int c0, int nc, FinShared<T, C>& sm, int vt,
+                                             Node<T, NB> node)
+{
+    typedef Real<T> RT;
+    typedef typename RT::type R;
+    constexpr int L = kThreads / C;  // lanes of a cell in the node phase
+    const int warp = vt >> 5, lane = vt & 31;
+    const int Qx = I.Qx, Qz = I.Qz, G = Qx + I.Qy + Qz;
+    const int cell = vt / L, j = vt % L;
     if (warp < 2) {
         // z: with few cells 16 lanes per cell, lane l - 1 of each sign forming row l of the
         // polynomials' coefficients times the moments; else a lane per (cell, sign) and all rows
@@ -424,10 +443,11 @@ __device__ __forceinline__ void record_cells(const InstDev& I, int c0, int nc, F
 #pragma unroll
     for (int a = 0; a < 4; ++a) s[a] = RT::of(T(0));
     PairSum<T> ws;  // of the current axis (a thread's nodes come in axis order)
-    int cur = ax;
+    int cur = node.ax;
     for (int r = j; r < G; r += L) {
-        if (r + L < G) load_row(r + L, hn, wn, axn);
-        const int N = ax == 0 ? I.Nx : ax == 1 ? I.Ny : I.Nzq;
+        Node<T, NB> next;
+        next.load(I, r + L);
+        const int ax = node.ax, N = node.order(I);
         if (ax != cur) {
             (cur == 0 ? s[0] : s[1]) = ws.total();
             ws = PairSum<T>();
@@ -439,18 +459,15 @@ __device__ __forceinline__ void record_cells(const InstDev& I, int c0, int nc, F
         } else {
 #pragma unroll
             for (int l = 0; l <= NB; ++l)
-                if (l <= N) g.term(sm.c[ax][l][cell], h[l]);
+                if (l <= N) g.term(sm.c[ax][l][cell], node.h[l]);
         }
         const auto v = g.value();
         if (live) {
             rec[R_DX + r] = v.x;
             if (ax == 2) rec[R_DX + r + Qz] = v.y;
         }
-        ws.weighted(w, v);
-#pragma unroll
-        for (int l = 0; l <= NB; ++l) h[l] = hn[l];
-        w = wn;
-        ax = axn;
+        ws.weighted(node.w, v);
+        node = next;
     }
     (cur == 0 ? s[0] : cur == 1 ? s[1] : s[2]) = ws.total();
     // the cell's lanes: scatter the four sums over lane pairs L/2 and L/4 apart, then add up
@@ -470,15 +487,18 @@ __device__ __forceinline__ void record_cells(const InstDev& I, int c0, int nc, F
     }
 }
 
+// the thread index with the warps' roles rotated
+static __device__ __forceinline__ int rotated(int rot) { return (threadIdx.x + 32 * rot) & (kThreads - 1); }
+
 // ---- one group of cells c0 .. c0 + nc - 1 (nc <= C), all 128 threads of the CTA -------------
 template <typename T, int NB, int C>
 __device__ __forceinline__ void finalize_group(const InstDev& I, int c0, int nc, int stage, FinShared<T, C>& sm,
-                                               int rot)
+                                               int rot, const Node<T, NB>& node)
 {
     typedef Real<T> RT;
     typedef typename RT::type R;
     typedef typename Acc<T>::type A;
-    const int vt = (threadIdx.x + 32 * rot) & (kThreads - 1);  // thread index with rotated warp roles
+    const int vt = rotated(rot);
     const int Nz = I.Nz, nch = I.nchunks;
     // sums over the chunks, in order within the even and the odd ones (the same order whatever
     // C is); loads past L1: other CTAs wrote the partials
@@ -565,7 +585,8 @@ __device__ __forceinline__ void finalize_group(const InstDev& I, int c0, int nc,
         }
     }
     __syncthreads();
-    record_cells<T, NB, C, true>(I, c0, nc, sm, vt);
+    launch_dependents();
+    record_cells<T, NB, C, true>(I, c0, nc, sm, vt, node);
 }
 
 // the fused finalisation: the cells of a z-tile, four at a time
@@ -574,7 +595,9 @@ __device__ __noinline__ void finalize_tile(const InstDev& I, int z0, int zn, int
 {
     static_assert(sizeof(FinShared<T, 4>) <= 9 * kThreads * sizeof(T), "fits the rows of the smallest z-tile");
     for (int c = 0; c < zn; c += 4) {
-        finalize_group<T, kMaxN, 4>(I, z0 + c, min(4, zn - c), stage, sm, (c >> 2) & 3);
+        Node<T, kMaxN> node;
+        node.load(I, threadIdx.x & 31);  // a cell's 32 lanes; the roles rotate by whole warps
+        finalize_group<T, kMaxN, 4>(I, z0 + c, min(4, zn - c), stage, sm, (c >> 2) & 3, node);
         __syncthreads();
     }
 }
@@ -608,7 +631,9 @@ __global__ void __launch_bounds__(kThreads) records_from_macro(const InstDev* __
         sm.bad[c] = !ok;
     }
     __syncthreads();
-    record_cells<T, kMaxN, 4, false>(I, c0, nc, sm, threadIdx.x);
+    Node<T, kMaxN> node;
+    node.load(I, threadIdx.x & 31);
+    record_cells<T, kMaxN, 4, false>(I, c0, nc, sm, threadIdx.x, node);
 }
 
 // The instance descriptor copied into shared memory by the whole block at once: its

@@ -16,9 +16,12 @@ __global__ void __launch_bounds__(kThreads) finalize_cells(const InstDev* __rest
     __shared__ int last;
     __shared__ InstDev sI;
     const InstDev& I = stage_descriptor(insts + blockIdx.y, &sI);
-    const int nblk = (I.Nz + C - 1) / C, c0 = blockIdx.x * C;
+    const int nblk = (I.Nz + C - 1) / C, c0 = blockIdx.x * C, rot = (blockIdx.x + blockIdx.y) & 3;
+    Node<T, NB> node;
+    node.load(I, rotated(rot) % (kThreads / C));
+    wait_predecessor();
     if (blockIdx.x >= nblk || *I.active == 0) return;
-    finalize_group<T, NB, C>(I, c0, min(C, I.Nz - c0), stage, sm, (blockIdx.x + blockIdx.y) & 3);
+    finalize_group<T, NB, C>(I, c0, min(C, I.Nz - c0), stage, sm, rot, node);
     // the instance's last block to finish (threadfence ticket) forms n_w and, after
     // stage 3, the residual; the counter is reset by its last user
     __threadfence();
@@ -140,16 +143,18 @@ template <typename K>
 static cudaError_t launch_first(K kernel, dim3 g, dim3 b, cudaStream_t st, const InstDev* d_inst, int stage)
 {
     static const int prio = highest_priority();
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributePriority;
     at[0].val.priority = prio;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = g;
     cfg.blockDim = b;
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kernel, d_inst, stage);
 }
 

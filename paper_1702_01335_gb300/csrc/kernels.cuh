@@ -324,8 +324,6 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     __shared__ InstDev sI;
     const Tile tile = tiles[blockIdx.x];
     const InstDev& I = stage_descriptor(insts + tile.inst, &sI);
-    if (*I.active == 0) return;
-    const int cur = *I.cur;  // which of F0 / F1 holds the step's start state
 
     const int Nz = I.Nz, Q = I.Q, Qx = I.Qx, Qy = I.Qy, Qz = I.Qz, QxQy = I.QxQy;
     const int z0 = tile.z0, zn = tile.zn;            // cells z0 .. z0+zn-1 (0-based)
@@ -346,45 +344,29 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     T* idzs = reinterpret_cast<T*>(smem_raw + L.idz);
     A* red = reinterpret_cast<A*>(smem_raw + L.red);  // per-warp moment sums
 
-    // Buffers (Eq. rk3 in increment form, F_l the step's start state d):
-    //   stage 1: d1 = dt L[F_l]                  -> the other of F0 / F1
-    //   stage 2: d2 = (d1 + dt L[F_l + d1]) / 4  -> F2
-    //   stage 3: F_l + 2/3 (d2 + dt L[F_l + d2]) -> the other of F0 / F1 (over d1)
-    const T* Hg = static_cast<const T*>(cur ? I.F1 : I.F0);
-    T* Og = static_cast<T*>(cur ? I.F0 : I.F1);
-    // the stage input's increment (stages 2, 3) is read from global memory through the
-    // read-only path (this launch does not write it), one march step ahead
-    const T* __restrict__ Dg = STAGE == 2 ? Og : static_cast<const T*>(I.F2);
-    T* Fout = STAGE == 2 ? static_cast<T*>(I.F2) : Og;
     const int s_lo = max(0, z0 - 3), s_hi = min(Nz - 1, z0 + zn + 2);
-
-    // ---- 1. stage the input rows and the cell records (TMA bulk copies; plain loads
-    //         if the rows are not 16-byte aligned)
     const T* Rg = static_cast<const T*>(I.rec) + (size_t)z0 * rstride;
     const size_t rec_bytes = (size_t)zn * rstride * sizeof(T);
-    if (I.bulk) {
-        if (tid == 0) {
+
+    // ---- 1. stage the input rows and the cell records by TMA bulk copies: warp 0 waits for
+    //         the predecessor and issues them while the other warps load the constants below
+    //         (all before the wait, 256 x C2 took 1121 us of stage kernels per step instead
+    //         of 1061)
+    if (warp == 0) {
+        wait_predecessor();
+        if (tid == 0 && I.bulk && *I.active != 0) {
+            const T* H = static_cast<const T*>(*I.cur ? I.F1 : I.F0);
             mbar_init(&bar, 1);
             fence_barrier_init();
-        }
-        __syncthreads();
-        if (tid == 0) {
             const uint32_t bytes = kn * sizeof(T);
             uint32_t total = bytes * (s_hi - s_lo + 1);
             if (STAGE > 0) total += rec_bytes;
             mbar_expect_tx(&bar, total);
             for (int s = s_lo; s <= s_hi; ++s)
-                bulk_g2s(Fs + (size_t)(s - z0 + 3) * KC, Hg + (size_t)s * Q + k0, bytes, &bar);
+                bulk_g2s(Fs + (size_t)(s - z0 + 3) * KC, H + (size_t)s * Q + k0, bytes, &bar);
             if (STAGE > 0) bulk_g2s(recs, Rg, rec_bytes, &bar);  // records are 16-byte multiples
         }
-    } else {
-        for (int s = s_lo; s <= s_hi; ++s)
-            for (int kl = tid; kl < kn; kl += kThreads) Fs[(size_t)(s - z0 + 3) * KC + kl] = Hg[(size_t)s * Q + k0 + kl];
-        if (STAGE > 0)
-            for (int e = tid; e < zn * rstride; e += kThreads) recs[e] = Rg[e];
     }
-    if (STAGE > 0)
-        for (int c = tid; c < zn; c += kThreads) idzs[c] = ld<T>(I.inv_dz, z0 + c);
 
     // per-velocity constants: p (and |p_z| for the fluxes), the weight w and |p|^2 for the
     // moments (formed from them per cell: fewer registers than 13 weighted monomials)
@@ -426,6 +408,32 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
             py[v] = jj[v] ? T(-0.4) : T(-0.8);
         }
     }
+    if (STAGE > 0)
+        for (int c = tid; c < zn; c += kThreads) idzs[c] = ld<T>(I.inv_dz, z0 + c);
+    if (warp != 0) wait_predecessor();
+    // from here on: what other kernels write
+    if (*I.active == 0) return;
+    const int cur = *I.cur;  // which of F0 / F1 holds the step's start state
+
+    // Buffers (Eq. rk3 in increment form, F_l the step's start state d):
+    //   stage 1: d1 = dt L[F_l]                  -> the other of F0 / F1
+    //   stage 2: d2 = (d1 + dt L[F_l + d1]) / 4  -> F2
+    //   stage 3: F_l + 2/3 (d2 + dt L[F_l + d2]) -> the other of F0 / F1 (over d1)
+    const T* Hg = static_cast<const T*>(cur ? I.F1 : I.F0);
+    T* Og = static_cast<T*>(cur ? I.F0 : I.F1);
+    // the stage input's increment (stages 2, 3) is read from global memory, one march step
+    // ahead.  Not through the read-only path: the CTA may start while the launch that writes
+    // the increment still runs (wait_predecessor), and only ordinary loads are then coherent.
+    const T* Dg = STAGE == 2 ? Og : static_cast<const T*>(I.F2);
+    T* Fout = STAGE == 2 ? static_cast<T*>(I.F2) : Og;
+    // rows that are not 16-byte aligned: plain loads
+    if (!I.bulk) {
+        for (int s = s_lo; s <= s_hi; ++s)
+            for (int kl = tid; kl < kn; kl += kThreads) Fs[(size_t)(s - z0 + 3) * KC + kl] = Hg[(size_t)s * Q + k0 + kl];
+        if (STAGE > 0)
+            for (int e = tid; e < zn * rstride; e += kThreads) recs[e] = Rg[e];
+    }
+    __syncthreads();  // the barrier's initialisation
 
     // ---- 3. wait for the copies (bounded).  A CTA whose wait runs out flags the
     //         instance (STATUS_TIMEOUT), then waits a further bounded time for its copies
@@ -470,7 +478,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     //          the whole stage-input value d (+ increment); a cell's row holds d.
     const int rbase = 3 - z0;  // smem row of cell s is s + rbase
     auto rowval = [&](int row, int col) -> T {  // the stage input of a cell's row
-        return kD ? Fs[(size_t)row * KC + col] + __ldg(Dg + (size_t)(row - rbase) * Q + k0 + col)
+        return kD ? Fs[(size_t)row * KC + col] + __ldca(Dg + (size_t)(row - rbase) * Q + k0 + col)
                   : Fs[(size_t)row * KC + col];
     };
 #pragma unroll
@@ -538,13 +546,13 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         const float2* rp2 = reinterpret_cast<const float2*>(Fs + (sgc ? (size_t)(zn + 5) * KC : 0)) + tid;
         const int sdir = sgc ? -1 : 1;
         const int zw0 = sgc ? z0 + zn + 2 : z0 - 3;  // the cell of window row 0 at step 0
-        const float* __restrict__ Dgf = reinterpret_cast<const float*>(Dg);
+        const float* Dgf = reinterpret_cast<const float*>(Dg);
         // the increments of the cell of a window row (zero for a ghost row)
         auto inc_row2 = [&](int s, float2(&out)[NP]) {
             const bool in = kD && (unsigned)s < (unsigned)Nz;
             const float2* q = reinterpret_cast<const float2*>(Dgf + (long)s * Q + k0) + tid;
 #pragma unroll
-            for (int p = 0; p < NP; ++p) out[p] = in && ok[2 * p] ? __ldg(q + p * kThreads) : make_float2(0.f, 0.f);
+            for (int p = 0; p < NP; ++p) out[p] = in && ok[2 * p] ? __ldca(q + p * kThreads) : make_float2(0.f, 0.f);
         };
         float2 PX[NP], PY[NP], PZ[NP], NAPZ[NP], WV[NP];  // per pair: p, -|p_z|, weights
 #pragma unroll
@@ -568,20 +576,20 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         inc_row2(sn, DN);
         // the increments' row of cell sn as a running offset in pairs (one add per march
         // step instead of the row's product; a pointer is formed only inside the channel)
-        const float2* __restrict__ dbase = reinterpret_cast<const float2*>(Dgf + k0) + tid;
+        const float2* dbase = reinterpret_cast<const float2*>(Dgf + k0) + tid;
         long doff = (long)sn * (Q / 2);
         const long dstep = sdir * (long)(Q / 2);
         const float2 DT = splat(float(I.dt));
         const long ostep2 = sgc ? -(long)(Q / 2) : (long)(Q / 2);
         const size_t orow0 = (size_t)(sgc ? z0 + zn - 1 : z0) * Q + k0 + tbase;
         float2* outp = reinterpret_cast<float2*>(reinterpret_cast<float*>(Fout) + orow0);
-        const float2* __restrict__ dop = kD ? reinterpret_cast<const float2*>(Dgf + orow0) : nullptr;
+        const float2* dop = kD ? reinterpret_cast<const float2*>(Dgf + orow0) : nullptr;
         unsigned* lop = kLo && STAGE == 3 ? reinterpret_cast<unsigned*>(I.L0 + orow0) : nullptr;
         unsigned LQN[NP];
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             LQN[p] = kLo && STAGE == 3 && ok[2 * p] ? __ldcg(lop + p * kThreads) : 0u;
-            DIN[p] = kD && ok[2 * p] ? __ldg(dop + p * kThreads) : make_float2(0.f, 0.f);
+            DIN[p] = kD && ok[2 * p] ? __ldca(dop + p * kThreads) : make_float2(0.f, 0.f);
         }
         // stage 1 unrolled by two steps (the window's shift halves; 80 vs 86 us on 64 x C2);
         // stages 2 and 3, with their increment and residual streams, lose by unrolling
@@ -594,7 +602,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
                 LQC[p] = LQN[p];
                 if (kLo && STAGE == 3 && ok[2 * p] && c + 1 < zn) LQN[p] = __ldcg(lop + ostep2 + p * kThreads);
                 DIC[p] = DIN[p];
-                if (kD && ok[2 * p] && c + 1 < zn) DIN[p] = __ldg(dop + ostep2 + p * kThreads);
+                if (kD && ok[2 * p] && c + 1 < zn) DIN[p] = __ldca(dop + ostep2 + p * kThreads);
                 DC[p] = DN[p];
             }
             if (kD && c + 1 < zn) {
@@ -603,7 +611,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
                 const bool in = (unsigned)sn < (unsigned)Nz;
 #pragma unroll
                 for (int p = 0; p < NP; ++p)
-                    DN[p] = in && ok[2 * p] ? __ldg(dbase + doff + p * kThreads) : make_float2(0.f, 0.f);
+                    DN[p] = in && ok[2 * p] ? __ldca(dbase + doff + p * kThreads) : make_float2(0.f, 0.f);
             }
             const int cc = sgc ? zn - 1 - c : c;
             const float* sc = reinterpret_cast<const float*>(recs) + (size_t)cc * rstride;
@@ -717,18 +725,18 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     const long rstep = sgc ? -(long)KC : (long)KC;
     const T* rp = Fs + (sgc ? (size_t)(zn + 5) * KC : 0);  // window row d at step c: rp + (c + d) rstep
     // stages 2, 3: the increment of the cell of each window row, read from global memory
-    // through the read-only path (this launch does not write it).  Window row cd at step c
+    // (this launch does not write it).  Window row cd at step c
     // holds cell zw0 + (c + cd) sdir; a ghost row (a cell outside 0 .. Nz-1) takes zero,
     // its shared-memory value being the whole stage input.  Thread-based pointers: the
     // thread's velocity v sits at + voff(v).
     const int sdir = sgc ? -1 : 1;
     const int zw0 = sgc ? z0 + zn + 2 : z0 - 3;
-    const T* __restrict__ dq = Dg + k0 + tbase;
+    const T* dq = Dg + k0 + tbase;
     auto inc_row = [&](int s, T(&out)[V]) {
         const bool in = kD && (unsigned)s < (unsigned)Nz;
         const T* p = dq + (long)s * Q;
 #pragma unroll
-        for (int v = 0; v < V; ++v) out[v] = in && ok[v] ? __ldg(p + voff(v)) : T(0);
+        for (int v = 0; v < V; ++v) out[v] = in && ok[v] ? __ldca(p + voff(v)) : T(0);
     };
     // cm: the WENO correction of the interface behind (its flux is |p_z| (w2 + cm))
     T w[V][6], cm[V], dn[V];
@@ -746,7 +754,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     const long ostep = sgc ? -(long)Q : (long)Q;
     const size_t orow0 = (size_t)(sgc ? z0 + zn - 1 : z0) * Q + k0 + tbase;  // the first cell, thread's column
     T* outp = Fout + orow0;
-    const T* __restrict__ dop = kD ? Dg + orow0 : nullptr;  // the increment of the cell
+    const T* dop = kD ? Dg + orow0 : nullptr;  // the increment of the cell
     unsigned short* lop = kLo && STAGE == 3 ? I.L0 + orow0 : nullptr;
     // stage 3 (FP32): the residuals of the next cell are loaded one march step ahead, so
     // that their global-memory latency overlaps a step's arithmetic
@@ -756,7 +764,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         lqn[v] = kLo && STAGE == 3 && ok[v] ? __ldcg(lop + voff(v)) : 0;
-        din[v] = kD && ok[v] ? __ldg(dop + voff(v)) : T(0);
+        din[v] = kD && ok[v] ? __ldca(dop + voff(v)) : T(0);
     }
     constexpr bool kPack = sizeof(T) == 4 && V % 2 == 0;  // moments of two velocities per packed op
 #pragma unroll 1  // unrolling the z-march only adds instruction-cache misses
@@ -768,7 +776,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
             lqc[v] = lqn[v];
             if (kLo && STAGE == 3 && ok[v] && c + 1 < zn) lqn[v] = __ldcg(lop + ostep + voff(v));
             dic[v] = din[v];
-            if (kD && ok[v] && c + 1 < zn) din[v] = __ldg(dop + ostep + voff(v));
+            if (kD && ok[v] && c + 1 < zn) din[v] = __ldca(dop + ostep + voff(v));
             dc[v] = dn[v];
         }
         if (kD && c + 1 < zn) {
@@ -954,6 +962,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         if (kLo && STAGE == 3) lop += ostep;
     }
     }  // the scalar march
+    launch_dependents();
     __syncthreads();
     // the chunk's partial of each cell: the warps' sums added and stored in the
     // accumulation type (FP32 storage: no FP64 instruction here; the finalisation sums
@@ -1033,10 +1042,21 @@ static cudaError_t launch_stage_t(const InstDev* d_inst, const Tile* d_tiles, in
                                   int fuse, cudaStream_t st)
 {
     auto kfn = stage_kernel<T, V, STAGE, RED>;
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kfn<<<ntiles, kThreads, smem, st>>>(d_inst, d_tiles, fuse);
-    return cudaGetLastError();
+    if (smem > 40 * 1024) {  // with the static arrays above the default limit of 48 KB
+        cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ntiles);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kfn, d_inst, d_tiles, fuse);
 }
 
 template <typename T, int V, bool RED>
