@@ -27,7 +27,7 @@ cudaError_t launch_seed(int fp32, const InstDev* d_inst, int inst, int Nz, const
 cudaError_t launch_seed_free_molecular(int fp32, const InstDev* d_inst, int inst, int Nz, cudaStream_t st);
 cudaError_t launch_gather_moments(const InstDev* d_inst, int ninst, const double* prof_all, double* out,
                                   cudaStream_t st);
-size_t stage_smem_bytes(int fp32, int V, int zn, int G, int stage, int rstride);
+size_t stage_smem_bytes(int fp32, int V, int zn, int Qx, int Qy, int nzm, int rstride);
 }  // namespace lbs
 
 using namespace lbs;
@@ -77,6 +77,7 @@ struct lbs_solver {
     int fp32 = 0, esize = 8, V = 1, ZT = 16, fuse = 1, ninst = 0, maxNz = 0, nb = 0;
     int fin_mode = 0, fin_cells = 4;  // lbs_set_finalize's mode; cells per CTA of the finalisation
     int reduced = 0;                 // the batch runs the phi / chi model (all instances alike)
+    int groupable = 0;               // full model, Qy a multiple of four in every instance
     std::vector<InstHost> ih;
     std::vector<InstDev> idev;
     InstDev* d_inst = nullptr;
@@ -223,6 +224,15 @@ static std::vector<double> rounded(const std::vector<double>& v)
     return r;
 }
 
+// The layout of the stage kernel for the launchers: V, or the grouped form of V = 4 (four
+// adjacent velocities per thread with common x and z nodes), which needs Qy a multiple of four
+// in every instance of a full-model batch and, where it applies, is the faster one (256 x C2
+// 987 us of stage kernels per step against 1061, 16 x C2 in FP64 2365 against 3063).
+static int stage_layout(const lbs_solver* h)
+{
+    return h->V == 4 && h->groupable ? kGroupedV : h->V;
+}
+
 static void build_tiles(lbs_solver* h, std::vector<Tile>& tiles)
 {
     tiles.clear();
@@ -242,17 +252,16 @@ static void build_tiles(lbs_solver* h, std::vector<Tile>& tiles)
             nzm_max = std::max(nzm_max, k1 / (I.Qx * I.Qy) - k0 / (I.Qx * I.Qy) + 1);
         }
         I.nzm_max = nzm_max;
-        const int G = I.Qx + I.Qy + nzm_max;
         const int rs = rec_stride_of(I.Qx, I.Qy, I.Qz);
         // z-tiles of about ZT cells, at least 3 cells each, within the shared-memory budget
         int zt = std::max(3, std::min(h->ZT, kMaxZT));
-        while (zt > 3 && stage_smem_bytes(h->fp32, h->V, zt, G, 3, rs) > kSmemBudget) --zt;
+        while (zt > 3 && stage_smem_bytes(h->fp32, stage_layout(h), zt, I.Qx, I.Qy, nzm_max, rs) > kSmemBudget) --zt;
         int nzt = std::min((I.Nz + zt - 1) / zt, I.Nz / 3);
         nzt = std::max(nzt, 1);
         const int base = I.Nz / nzt, rem = I.Nz % nzt;
         const int zmax = base + (rem ? 1 : 0);
         I.nzt = nzt;
-        smem = std::max(smem, stage_smem_bytes(h->fp32, h->V, zmax, G, 3, rs));
+        smem = std::max(smem, stage_smem_bytes(h->fp32, stage_layout(h), zmax, I.Qx, I.Qy, nzm_max, rs));
         for (int c = 0; c < I.nchunks; ++c) {
             int z0 = 0;
             for (int t = 0; t < nzt; ++t) {
@@ -626,7 +635,7 @@ static const char* const kStageRange[4] = {"lbs analysis", "lbs RK stage 1", "lb
 static lbs_status analyse(lbs_solver* h)
 {
     NvtxRange r(kStageRange[0]);
-    CK(launch_stage(h->fp32, h->reduced, h->V, 0, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->ninst, h->maxNz,
+    CK(launch_stage(h->fp32, h->reduced, stage_layout(h), 0, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->ninst, h->maxNz,
                     h->fin_cells, h->nb, h->stream));
     return LBS_OK;
 }
@@ -652,7 +661,7 @@ static lbs_status enqueue_step(lbs_solver* h)
     if (!split(h)) {
         for (int s = 1; s <= 3; ++s) {
             NvtxRange r(kStageRange[s]);
-            CK(launch_stage(h->fp32, h->reduced, h->V, s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->ninst,
+            CK(launch_stage(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->ninst,
                             h->maxNz, h->fin_cells, h->nb, h->stream));
         }
         return LBS_OK;
@@ -663,9 +672,9 @@ static lbs_status enqueue_step(lbs_solver* h)
     // array, a range of tiles); the finalisation kernels take a range of instances
     for (int s = 1; s <= 3; ++s) {
         NvtxRange r(kStageRange[s]);
-        CK(launch_stage_only(h->fp32, h->reduced, h->V, s, h->d_inst, h->d_tiles, h->ntilesA, h->smem, 0, h->stream));
+        CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntilesA, h->smem, 0, h->stream));
         CK(launch_finalize(h->fp32, s, h->d_inst, h->nA, h->maxNz, h->fin_cells, h->nb, h->stream));
-        CK(launch_stage_only(h->fp32, h->reduced, h->V, s, h->d_inst, h->d_tiles + h->ntilesA, h->ntiles - h->ntilesA, h->smem,
+        CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles + h->ntilesA, h->ntiles - h->ntilesA, h->smem,
                              0, h->stream2));
         CK(launch_finalize(h->fp32, s, h->d_inst + h->nA, h->ninst - h->nA, h->maxNz, h->fin_cells, h->nb, h->stream2));
     }
@@ -844,6 +853,8 @@ lbs_status lbs_batch_create(lbs_handle* out, const lbs_instance_desc* desc, int 
     }
     lbs_solver* h = new lbs_solver();
     h->reduced = desc[0].orders.Qy == 0;
+    h->groupable = !h->reduced;
+    for (int b = 0; b < n; ++b) h->groupable &= desc[b].orders.Qy % 4 == 0;
     if (cudaGetDevice(&h->device) != cudaSuccess) h->device = 0;
     h->fp32 = prec == LBS_FP32_STORE_FP64_ACC;
     h->esize = h->fp32 ? 4 : 8;
@@ -855,8 +866,10 @@ lbs_status lbs_batch_create(lbs_handle* out, const lbs_instance_desc* desc, int 
                 desc[b].orders.Qz_half;
     // untuned default: small batches are latency-bound (short z-tiles, one velocity per
     // thread, more CTAs); large ones take the throughput tiling.  Finalisation apart.
+    // FP64 is bound by the FP64 pipe and takes shorter tiles, which spread more evenly over the
+    // SMs (16 x C2, grouped layout: 2365 us of stage kernels per step at 12 cells, 2004 at 8)
     h->V = work >= (1L << 22) ? 4 : 1;
-    h->ZT = work >= (1L << 22) ? 12 : 4;
+    h->ZT = work < (1L << 22) ? 4 : h->fp32 ? 12 : 8;
     // the FP32 full model with V = 2, 4 takes velocities in pairs (64-bit words), which
     // needs Q / 2 even in every instance; else one velocity per thread
     for (int b = 0; b < n; ++b)
@@ -1051,7 +1064,7 @@ lbs_status lbs_profile_steps(lbs_handle h, long nsteps, double* out_ms)
     for (long it = 0; it < nsteps && st == LBS_OK; ++it) {
         CK(cudaEventRecord(ev[0], h->stream));
         for (int s = 1; s <= 3; ++s) {
-            CK(launch_stage_only(h->fp32, h->reduced, h->V, s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->stream));
+            CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->stream));
             CK(cudaEventRecord(ev[2 * s - 1], h->stream));
             if (!(h->fuse & 1)) CK(launch_finalize(h->fp32, s, h->d_inst, h->ninst, h->maxNz, h->fin_cells, h->nb, h->stream));
             CK(cudaEventRecord(ev[2 * s], h->stream));
@@ -1341,7 +1354,7 @@ lbs_status lbs_set_state(lbs_handle h, int inst, const void* src, int from_host)
         {
             // the same launches as analyse() (the fused finalisation counts per instance)
             NvtxRange ra(kStageRange[0]);
-            CK(launch_stage_only(h->fp32, h->reduced, h->V, 0, h->d_inst, h->d_tiles + h->tile_first[c0],
+            CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), 0, h->d_inst, h->d_tiles + h->tile_first[c0],
                                  h->tile_first[c1] - h->tile_first[c0], h->smem, h->fuse & 1, h->stream2));
             if (!(h->fuse & 1))
                 CK(launch_finalize(h->fp32, 0, h->d_inst + c0, c1 - c0, h->maxNz, h->fin_cells, h->nb, h->stream2));

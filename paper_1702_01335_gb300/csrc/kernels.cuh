@@ -187,6 +187,79 @@ static __device__ __forceinline__ float2 weno5_corr2(float2 v0, float2 v1, float
     return mul2(fma2(w1, e1, fma2(w2, e2, mul2(w3, e3))), inv);
 }
 
+// ---- two velocities of either storage type: float2 by the packed instructions above,
+// double2 component by component (the compiler merges equal components)
+static __device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+static __device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+static __device__ __forceinline__ double2 mul2(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
+static __device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c)
+{
+    return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
+static __device__ __forceinline__ double2 splat(double a) { return make_double2(a, a); }
+template <typename T> struct Two;
+template <> struct Two<float> { typedef float2 type; };
+template <> struct Two<double> { typedef double2 type; };
+
+// WENO-5 correction from differences that the march carries from one interface to the next.
+// With D12 = v2 - v1, D23 = v3 - v2 and the second differences A_j = v_{j-1} - 2 v_j + v_{j+1}
+// (and K A_j^2, K = 13/3) the indicators are 4 sigma_1 = K A_1^2 + (A_1 + 2 D12)^2,
+// 4 sigma_2 = K A_2^2 + (D12 + D23)^2, 4 sigma_3 = K A_3^2 + (A_3 - 2 D23)^2, and the
+// candidates e_1 / 2 = A_1 + 3/2 D12, e_2 / 2 = D23 + D12 / 2, e_3 / 2 = 3/2 D23 - A_3 / 2
+// (e_q as in weno5_corr).  A_1 and A_2 of one interface are A_2 and A_3 of the one before, so
+// a step forms one first and one second difference instead of four differences and six
+// combinations: 12 instructions less.  The weights are those of the two forms above.
+template <typename P>
+struct Carried {
+    P v3, d12, d23, a1, k1, k2, a2;  // v3 the newest cell value; k = K a^2
+};
+static __device__ __forceinline__ float2 carried_weights(float2 s1, float2 s2, float2 s3, float2 e1, float2 e2,
+                                                         float2 e3)
+{
+    const float2 F = splat(kWenoFloor);
+    const float2 q1 = fma2(s1, s1, F), q2 = fma2(s2, s2, F), q3 = fma2(s3, s3, F);
+    const float2 w1 = make_float2(rcp_approx(q1.x), rcp_approx(q1.y));
+    const float2 w2 = make_float2(6.f * rcp_approx(q2.x), 6.f * rcp_approx(q2.y));
+    const float2 w3 = make_float2(3.f * rcp_approx(q3.x), 3.f * rcp_approx(q3.y));
+    const float2 sw = add2(add2(w1, w2), w3);
+    const float2 inv = make_float2(rcp_approx(3.f * sw.x), rcp_approx(3.f * sw.y));
+    return mul2(fma2(w1, e1, fma2(w2, e2, mul2(w3, e3))), inv);
+}
+static __device__ __forceinline__ double carried_weights(double q1, double q2, double q3, double e1, double e2,
+                                                         double e3)
+{
+    const int top = max(__double2hiint(q1), max(__double2hiint(q2), __double2hiint(q3)));  // sigma >= 0
+    const double s = __hiloint2double(0x7FE00000 - (top & 0x7FF00000), 0), floor_ = 0x1p-250;
+    const double s1 = fma(q1, s, floor_), s2 = fma(q2, s, floor_), s3 = fma(q3, s, floor_);
+    const double p1 = s2 * s3, p2 = s1 * s3, p3 = s1 * s2;
+    const double w1 = p1 * p1, w2 = 6.0 * p2 * p2, w3 = 3.0 * p3 * p3;
+    return fma(w1, e1, fma(w2, e2, w3 * e3)) * rcp_newton(fma(3.0, w1, 3.0 * (w2 + w3)));
+}
+static __device__ __forceinline__ double2 carried_weights(double2 s1, double2 s2, double2 s3, double2 e1, double2 e2,
+                                                          double2 e3)
+{
+    return make_double2(carried_weights(s1.x, s2.x, s3.x, e1.x, e2.x, e3.x),
+                        carried_weights(s1.y, s2.y, s3.y, e1.y, e2.y, e3.y));
+}
+// the correction of the interface ahead of v2 for the new value v4; advances the differences
+template <typename T, typename P>
+static __device__ __forceinline__ P carried_corr(Carried<P>& w, P v4)
+{
+    const P d34 = sub2(v4, w.v3), a3 = sub2(d34, w.d23), k3 = mul2(mul2(splat(T(13.0 / 3.0)), a3), a3);
+    const P b1 = fma2(splat(T(2)), w.d12, w.a1), b2 = add2(w.d12, w.d23), b3 = fma2(splat(T(-2)), w.d23, a3);
+    const P e1 = fma2(splat(T(1.5)), w.d12, w.a1), e2 = fma2(splat(T(0.5)), w.d12, w.d23);
+    const P e3 = fma2(splat(T(-0.5)), a3, mul2(splat(T(1.5)), w.d23));
+    const P c = carried_weights(fma2(b1, b1, w.k1), fma2(b2, b2, w.k2), fma2(b3, b3, k3), e1, e2, e3);
+    w.v3 = v4;
+    w.d12 = w.d23;
+    w.d23 = d34;
+    w.a1 = w.a2;
+    w.a2 = a3;
+    w.k1 = w.k2;
+    w.k2 = k3;
+    return c;
+}
+
 template <typename T>
 __device__ __forceinline__ T weno5(T v0, T v1, T v2, T v3, T v4)
 {
@@ -239,23 +312,66 @@ __device__ __forceinline__ A reduce_scatter16(A (&v)[16], int lane)
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
+// The warp totals of 13 FP32 values per lane (q[3].y .. w unused) through 2 KB of shared memory:
+// each lane writes its values as four 16-byte words, then lane 4 s + g sums word g of lanes
+// s, s + 8, s + 16, s + 24 (packed adds) and a reduce-scatter over s finishes.  Word w of lane
+// l sits at w ^ (l / 2 mod 4), which keeps both directions free of bank conflicts.  29
+// instructions instead of the 62 of reduce_scatter16.  Returns the total of value
+// 4 g + 2 b4 + b3 (g = lane mod 4, b = bits of the lane); lanes l, l ^ 4 agree.
+static __device__ __forceinline__ float warp_totals13(const float4 (&q)[4], float4* buf, int lane)
+{
+    float4* row = buf + lane * 4;
+    const int x = (lane >> 1) & 3;
+    __syncwarp();  // the previous cell's reads are done
+#pragma unroll
+    for (int w = 0; w < 4; ++w) row[w ^ x] = q[w];
+    __syncwarp();
+    const int g = lane & 3, s = lane >> 2;
+    const float4* col = buf + s * 4 + (g ^ ((s >> 1) & 3));  // rows s + 8 i have the same swizzle
+    const float4 a = col[0], b = col[32], c = col[64], d = col[96];
+    const float2 t0 = add2(add2(make_float2(a.x, a.y), make_float2(b.x, b.y)),
+                           add2(make_float2(c.x, c.y), make_float2(d.x, d.y)));
+    const float2 t1 = add2(add2(make_float2(a.z, a.w), make_float2(b.z, b.w)),
+                           add2(make_float2(c.z, c.w), make_float2(d.z, d.w)));
+    const bool h4 = lane & 16, h3 = lane & 8;
+    const float2 keep = h4 ? t1 : t0, send = h4 ? t0 : t1;
+    const float2 u = add2(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, 16),
+                                            __shfl_xor_sync(0xffffffffu, send.y, 16)));
+    float v = (h3 ? u.y : u.x) + __shfl_xor_sync(0xffffffffu, h3 ? u.x : u.y, 8);
+    return v + __shfl_xor_sync(0xffffffffu, v, 4);
+}
+
 // shared-memory layout of a stage CTA (offsets in bytes): the staged rows of the
 // step's start state d (cells z0-3 .. z0+zn+2) and the cell records (by bulk copy), the
 // per-axis factors of this chunk's nodes, 1/dz, and the per-warp moment sums.  The stage
 // input's increment (stages 2 and 3) is read from global memory during the march.
 struct StageSmem {
-    size_t fin, rec, g, idz, red, total;
+    size_t fin, rec, g, idz, red, sc, total;
 };
+// values per cell of the factor region: one per node of x, of y and of the chunk's z nodes, or
+// (grouped layout) y's, then x's and z's, FP32 ones twice; a multiple of four either way
+__host__ __device__ inline int factor_stride(int Qx, int Qy, int nzm, bool grouped, int esize)
+{
+    return (Qy + (Qx + nzm) * (grouped && esize == 4 ? 2 : 1) + 3) & ~3;
+}
+// scalars per cell of the grouped layout: u, q, (1 - Pr)/(n T^2), 1/(5T), and -1/tau and 1/dz
+// times the stage's share of dt
+enum { S_UX = 0, S_UY, S_UZ, S_QX, S_QY, S_QZ, S_CS, S_I5T, S_NITAU, S_IDZ, S_COUNT };
 __host__ __device__ inline size_t pad16(size_t b) { return (b + 15) & ~size_t(15); }
-__host__ __device__ inline StageSmem stage_smem(int zn, int KC, int G, int esize, int asize, int rstride)
+__host__ __device__ inline StageSmem stage_smem(int zn, int KC, int G, int esize, int asize, int rstride,
+                                                    bool grouped)
 {
     StageSmem L;
     size_t o = 0;
     L.fin = o; o += (size_t)(zn + 6) * KC * esize;
-    L.rec = o; o += (size_t)zn * rstride * esize;
+    // grouped layout, FP32: the warps' moment scratch takes the records' place after the
+    // factors have been formed from them
+    const size_t scratch = grouped && esize == 4 ? (size_t)kThreads * 16 * 4 : 0, rec = (size_t)zn * rstride * esize;
+    L.rec = o; o += rec > scratch ? rec : scratch;
     L.g = o; o += pad16((size_t)zn * G * esize);
     L.idz = o; o += pad16((size_t)zn * esize);
     L.red = o; o += (size_t)zn * (kThreads / 32) * 16 * asize;
+    L.sc = o; o += grouped ? (size_t)zn * S_COUNT * 8 : 0;  // 80 bytes a cell in either type
     L.total = o;
     return L;
 }
@@ -311,7 +427,9 @@ template <typename T, int V> struct MinBlocks {
     static constexpr int value = V == 1 ? 8 : V == 2 ? 6 : sizeof(T) == 4 ? 4 : 3;
 };
 
-template <typename T, int V, int STAGE, bool RED>
+// GRP (V = 4, full model, Qy a multiple of 4 in every instance): a thread's four velocities
+// are adjacent, so they share the x and the z node.
+template <typename T, int V, int STAGE, bool RED, bool GRP>
 __global__ void __launch_bounds__(kThreads, MinBlocks<T, V>::value)
 stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, int fuse)
 {
@@ -333,16 +451,17 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     const int k0 = sgc * Qh + (tile.chunk - sgc * I.nchh) * KC;
     const int kend = min((sgc + 1) * Qh, k0 + KC), kn = kend - k0;
     const int zm_lo = k0 / QxQy, zm_hi = (kend - 1) / QxQy, nzm = zm_hi - zm_lo + 1;
-    const int G = Qx + Qy + nzm;                     // per-cell factors held in smem
+    const int G = factor_stride(Qx, Qy, nzm, GRP, sizeof(T));  // per-cell factors held in smem
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     const int rstride = I.rec_stride;
-    const StageSmem L = stage_smem(zn, KC, G, sizeof(T), sizeof(A), rstride);
+    const StageSmem L = stage_smem(zn, KC, G, sizeof(T), sizeof(A), rstride, GRP);
     T* Fs = reinterpret_cast<T*>(smem_raw + L.fin);   // d rows: cells z0-3 .. z0+zn+2
     T* recs = reinterpret_cast<T*>(smem_raw + L.rec); // records of cells z0 .. z0+zn-1
     T* gsm = reinterpret_cast<T*>(smem_raw + L.g);
     T* idzs = reinterpret_cast<T*>(smem_raw + L.idz);
     A* red = reinterpret_cast<A*>(smem_raw + L.red);  // per-warp moment sums
+    T* scs = reinterpret_cast<T*>(smem_raw + L.sc);   // grouped layout: the cells' scalars
 
     const int s_lo = max(0, z0 - 3), s_hi = min(Nz - 1, z0 + zn + 2);
     const T* Rg = static_cast<const T*>(I.rec) + (size_t)z0 * rstride;
@@ -354,8 +473,9 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     //         of 1061)
     if (warp == 0) {
         wait_predecessor();
-        if (tid == 0 && I.bulk && *I.active != 0) {
-            const T* H = static_cast<const T*>(*I.cur ? I.F1 : I.F0);
+        const int act = *I.active, c1 = *I.cur;  // both loads in flight
+        if (tid == 0 && I.bulk && act != 0) {
+            const T* H = static_cast<const T*>(c1 ? I.F1 : I.F0);
             mbar_init(&bar, 1);
             fence_barrier_init();
             const uint32_t bytes = kn * sizeof(T);
@@ -374,9 +494,10 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     // 2 tid + 2 kThreads, ...), so that a pair is one 64-bit word in memory and one
     // operand of the packed FP32 instructions; else tid + v kThreads.  voff(v) is v's
     // offset from the thread's first velocity tbase.
+    // Grouped layout: the four velocities 4 tid .. 4 tid + 3.
     constexpr bool kPair = sizeof(T) == 4 && V % 2 == 0;
-    const int tbase = kPair ? 2 * tid : tid;
-    auto voff = [](int v) { return kPair ? (v & 1) + (v >> 1) * 2 * kThreads : v * kThreads; };
+    const int tbase = GRP ? 4 * tid : kPair ? 2 * tid : tid;
+    auto voff = [](int v) { return GRP ? v : kPair ? (v & 1) + (v >> 1) * 2 * kThreads : v * kThreads; };
     int ii[V], jj[V], zz[V], kl[V];
     T px[V], py[V], pz[V], apz[V];
     A wv[V], yv[V], p2v[V], wm[V];  // weight; p_y for the moments; |p|^2; w of the mass flux
@@ -386,13 +507,15 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         kl[v] = tbase + voff(v);
         ok[v] = kl[v] < kn;
         const int kc = ok[v] ? k0 + kl[v] : kend - 1;
-        jj[v] = kc % Qy;
-        ii[v] = (kc / Qy) % Qx;
-        zz[v] = kc / QxQy;
+        // (grouped: kn is a multiple of 4, so v = 0 stands for all four but for the y node; past
+        // the chunk the y nodes still lie inside the table)
+        jj[v] = GRP ? (v ? jj[0] + v : kc % Qy & ~3) : kc % Qy;
+        ii[v] = GRP && v ? ii[0] : (kc / Qy) % Qx;
+        zz[v] = GRP && v ? zz[0] : kc / QxQy;
         const int sg = zz[v] >= Qz, m = zz[v] - sg * Qz;
-        px[v] = ld<T>(I.px, ii[v]);
+        px[v] = GRP && v ? px[0] : ld<T>(I.px, ii[v]);
         py[v] = ld<T>(I.py, jj[v]);
-        const T x = ld<T>(I.xi, m);
+        const T x = GRP && v ? apz[0] : ld<T>(I.xi, m);
         pz[v] = sg ? -x : x;
         apz[v] = x;
         wv[v] = ok[v] ? A(ld<T>(I.wx, ii[v]) * ld<T>(I.wy, jj[v]) * ld<T>(I.wz, m)) : A(0);
@@ -408,12 +531,12 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
             py[v] = jj[v] ? T(-0.4) : T(-0.8);
         }
     }
-    if (STAGE > 0)
+    if (STAGE > 0 && !GRP)
         for (int c = tid; c < zn; c += kThreads) idzs[c] = ld<T>(I.inv_dz, z0 + c);
     if (warp != 0) wait_predecessor();
     // from here on: what other kernels write
-    if (*I.active == 0) return;
-    const int cur = *I.cur;  // which of F0 / F1 holds the step's start state
+    const int act = *I.active, cur = *I.cur;  // cur: which of F0 / F1 holds the step's start state
+    if (act == 0) return;
 
     // Buffers (Eq. rk3 in increment form, F_l the step's start state d):
     //   stage 1: d1 = dt L[F_l]                  -> the other of F0 / F1
@@ -457,7 +580,41 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     // ---- 4a. per-cell factors of the truncated Hermite equilibrium (Sec. III) for this
     //          chunk's nodes, as deviations from 1, from the staged records:
     //          dx[i] with R_SCALE applied (R_SCALE (1 + dx) - 1), dy[j], dz[zm]
-    if (STAGE > 0) {
+    if constexpr (GRP && STAGE > 0) {
+        // [y][x][z], FP32's x and z values twice (a pair register without moves), and the
+        // cell's scalars likewise
+        const T dtc = T(I.dt) * (STAGE == 1 ? T(1) : STAGE == 2 ? T(0.25) : T(2.0 / 3.0));
+        const int nf = Qy + Qx + nzm + S_COUNT;
+        constexpr int dup = sizeof(T) == 4 ? 2 : 1;
+        for (int c = warp; c < zn; c += kThreads / 32)  // a warp per cell
+        for (int r = lane; r < nf; r += 32) {
+            const T* rc = recs + (size_t)c * rstride;
+            T g, *to;
+            if (r < Qy) {
+                gsm[(size_t)c * G + r] = rc[R_DX + Qx + r];  // dy
+                continue;
+            } else if (r < Qy + Qx) {
+                const T s1 = rc[R_SCALE1];
+                g = s1 + (T(1) + s1) * rc[R_DX + r - Qy];
+                to = gsm + (size_t)c * G + Qy + dup * (r - Qy);
+            } else if (r < Qy + Qx + nzm) {
+                g = rc[R_DX + r + zm_lo];  // dz[zm]
+                to = gsm + (size_t)c * G + Qy + dup * (r - Qy);
+            } else {
+                const int q = r - (Qy + Qx + nzm);
+                // the record holds u at R_UX .., q at R_QX .., 1/tau, cS, 1/(5T)
+                g = q < S_QX ? rc[R_UX + q]
+                    : q < S_CS ? rc[R_QX + q - S_QX]
+                    : q == S_CS ? rc[R_CS]
+                    : q == S_I5T ? rc[R_I5T]
+                    : q == S_NITAU ? -rc[R_ITAU] * dtc
+                                   : ld<T>(I.inv_dz, z0 + c) * dtc;
+                to = scs + (c * S_COUNT + q) * dup;
+            }
+            to[0] = g;
+            if (dup == 2) to[1] = g;
+        }
+    } else if (STAGE > 0) {
         for (int e = tid; e < zn * G; e += kThreads) {
             const int c = e / G, r = e - c * G;
             const T* rc = recs + (size_t)c * rstride;
@@ -533,7 +690,243 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
 
     __syncthreads();  // per-cell factors complete
 
-    if constexpr (kPair && !RED) {
+    if constexpr (GRP) {
+        // ---- 5 (grouped layout). The march of the scalar section below with four adjacent
+        // velocities per thread, as two pairs.  They share the x and the z node, so what depends
+        // on those alone -- xi_x, xi_z, their squares, the products with q, the target's x and z
+        // factors, the advection factor -- is formed once per cell, and the moments are the
+        // powers 0 .. 3 of xi_y summed over the four, combined with the shared xi_x and xi_z
+        // afterwards.  A row, an increment, an output of the thread is one 128-bit word (FP64:
+        // two).  The WENO differences are carried (carried_corr), so no window of values shifts.
+        // Measured, stage kernels per step against the pair march (FP32) and the scalar march
+        // (FP64): 256 x C2 1061 -> 987 us, 32 x C3 1049 -> 962, the sweep 405 -> 375; 16 x C2
+        // in FP64 3063 -> 2004 us (2365 at the same 12-cell tiles).  Instructions per update of
+        // the three FP32 stages: 112 / 137 / 155 -> 92 / 109 / 128.
+        typedef typename Two<T>::type P;
+        struct alignas(16) Quad { P p[2]; };
+        auto quad = [](const T* q) -> Quad {  // 16-byte aligned
+            Quad r;
+            if constexpr (sizeof(T) == 4) {
+                const float4 v = *reinterpret_cast<const float4*>(q);
+                r.p[0] = make_float2(v.x, v.y);
+                r.p[1] = make_float2(v.z, v.w);
+            } else {
+                r.p[0] = *reinterpret_cast<const double2*>(q);
+                r.p[1] = *reinterpret_cast<const double2*>(q + 2);
+            }
+            return r;
+        };
+        auto quad_g = [](const T* q) -> Quad {
+            Quad r;
+            if constexpr (sizeof(T) == 4) {
+                const float4 v = __ldca(reinterpret_cast<const float4*>(q));
+                r.p[0] = make_float2(v.x, v.y);
+                r.p[1] = make_float2(v.z, v.w);
+            } else {
+                r.p[0] = __ldca(reinterpret_cast<const double2*>(q));
+                r.p[1] = __ldca(reinterpret_cast<const double2*>(q + 2));
+            }
+            return r;
+        };
+        auto dup = [](const T* q) -> P {  // a value stored for both lanes
+            if constexpr (sizeof(T) == 4) return *reinterpret_cast<const float2*>(q);
+            else return splat(*q);
+        };
+        constexpr int kDup = sizeof(T) == 4 ? 2 : 1;
+        // FP32: two steps per iteration, after which the carried values are back in their
+        // registers (20 moves per step less)
+        constexpr int kUnroll = sizeof(T) == 4 ? 2 : 1;
+        const P zero = splat(T(0));
+        const bool in = ok[0];
+        const P PX = splat(px[0]), PZ = splat(pz[0]), NAPZ = splat(-apz[0]);
+        P PY[2], WV[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            PY[p].x = py[2 * p];
+            PY[p].y = py[2 * p + 1];
+            WV[p].x = wv[2 * p];
+            WV[p].y = wv[2 * p + 1];
+        }
+        const int sdir = sgc ? -1 : 1;
+        const long rstep = sdir * (long)KC, ostep = sdir * (long)Q;
+        const int zw0 = sgc ? z0 + zn + 2 : z0 - 3;  // the cell of march row 0
+        const T* rp = Fs + (sgc ? (size_t)(zn + 5) * KC : 0) + tbase;  // march row r: rp + r rstep
+        const T* dcol = Dg + k0 + tbase;
+        auto inc_row = [&](int s) -> Quad {  // the increments of cell s (zero for a ghost row)
+            Quad q;
+            q.p[0] = q.p[1] = zero;
+            if (kD && in && (unsigned)s < (unsigned)Nz) q = quad_g(dcol + (long)s * Q);
+            return q;
+        };
+        // rows 0 .. 4 (the cell's three upwind neighbours, the cell, the next one) give the
+        // differences and the correction of the interface behind the first cell
+        Carried<P> w[2];
+        P CM[2];
+        {
+            Quad r[5];
+#pragma unroll
+            for (int d = 0; d < 5; ++d) {
+                r[d] = quad(rp + d * rstep);
+                const Quad q = inc_row(zw0 + d * sdir);
+#pragma unroll
+                for (int p = 0; p < 2; ++p) r[d].p[p] = kD ? add2(r[d].p[p], q.p[p]) : r[d].p[p];
+            }
+            const P K = splat(T(13.0 / 3.0));
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const P d0 = sub2(r[1].p[p], r[0].p[p]);
+                w[p].v3 = r[3].p[p];
+                w[p].d12 = sub2(r[2].p[p], r[1].p[p]);
+                w[p].d23 = sub2(r[3].p[p], r[2].p[p]);
+                w[p].a1 = sub2(w[p].d12, d0);
+                w[p].a2 = sub2(w[p].d23, w[p].d12);
+                w[p].k1 = mul2(mul2(K, w[p].a1), w[p].a1);
+                w[p].k2 = mul2(mul2(K, w[p].a2), w[p].a2);
+                CM[p] = carried_corr<T>(w[p], r[4].p[p]);
+            }
+        }
+        // the next row: its shared-memory part is read and its increments are added a step ahead
+        int sn = zw0 + 5 * sdir;
+        Quad NV = quad(rp + 5 * rstep);
+        {
+            const Quad q = inc_row(sn);
+#pragma unroll
+            for (int p = 0; p < 2; ++p) NV.p[p] = kD ? add2(NV.p[p], q.p[p]) : NV.p[p];
+        }
+        sn += sdir;
+        Quad DN = inc_row(sn);
+        const size_t orow0 = (size_t)(sgc ? z0 + zn - 1 : z0) * Q + k0 + tbase;
+        T* outp = Fout + orow0;
+        const T* dop = kD ? Dg + orow0 : nullptr;
+        unsigned short* lop = kLo && STAGE == 3 ? I.L0 + orow0 : nullptr;
+        const T* dnp = dcol + (long)sn * Q;  // increments of the row after the next one
+        Quad DIN;
+        DIN.p[0] = DIN.p[1] = zero;
+        if (kD && in) DIN = quad_g(dop);
+        uint2 LQN = make_uint2(0u, 0u);
+        if (kLo && STAGE == 3 && in) LQN = __ldcg(reinterpret_cast<const uint2*>(lop));
+        const int gy = jj[0], gx = Qy + kDup * ii[0], gz = Qy + kDup * (Qx + zz[0] - zm_lo);
+#pragma unroll(kUnroll)
+        for (int c = 0; c < zn; ++c) {
+            const int cc = sgc ? zn - 1 - c : c;
+            const T* gc = gsm + (size_t)cc * G;
+            const T* sc = scs + cc * (S_COUNT * kDup);
+            const uint2 LQ = LQN;
+            const Quad DI = DIN;
+            const Quad own = quad(Fs + (size_t)(cc + 3) * KC + tbase);  // d of the cell
+            Quad nx = NV;                                               // the row two ahead
+            if (c + 1 < zn) {
+                NV = quad(rp + (c + 6) * rstep);
+#pragma unroll
+                for (int p = 0; p < 2; ++p) NV.p[p] = kD ? add2(NV.p[p], DN.p[p]) : NV.p[p];
+                if (kLo && STAGE == 3 && in) LQN = __ldcg(reinterpret_cast<const uint2*>(lop + ostep));
+                if (kD) {
+                    if (in) DIN = quad_g(dop + ostep);
+                    sn += sdir;
+                    dnp += ostep;
+                    DN.p[0] = DN.p[1] = zero;
+                    if (in && (unsigned)sn < (unsigned)Nz) DN = quad_g(dnp);
+                }
+            }
+            P X = PX, Z = PZ, XZ2, XQ, GXZ, S1, Y[2], out[2];
+            P UY, QY, CS, I5T, NIT;
+            if (STAGE > 0) {
+                X = sub2(PX, dup(sc + kDup * S_UX));
+                Z = sub2(PZ, dup(sc + kDup * S_UZ));
+                UY = dup(sc + kDup * S_UY);
+                QY = dup(sc + kDup * S_QY);
+                CS = dup(sc + kDup * S_CS);
+                I5T = dup(sc + kDup * S_I5T);
+                NIT = dup(sc + kDup * S_NITAU);
+                XQ = fma2(Z, dup(sc + kDup * S_QZ), mul2(X, dup(sc + kDup * S_QX)));
+                S1 = mul2(NAPZ, dup(sc + kDup * S_IDZ));
+                const P DX = dup(gc + gx), DZ = dup(gc + gz);
+                GXZ = fma2(DX, DZ, add2(DX, DZ));
+            }
+            XZ2 = fma2(Z, Z, mul2(X, X));
+            const Quad DY = STAGE > 0 ? quad(gc + gy) : own;
+            Quad st;
+            P A0, A1, A2, A3;  // sums of w f xi_y^a over the thread's velocities, two lanes
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const P h = own.p[p];
+                out[p] = h;
+                Y[p] = PY[p];
+                if (STAGE > 0) {
+                    // the target's deviation from 1, (1 + dx)(1 + dz)(1 + dy)(1 + S) - 1
+                    Y[p] = sub2(PY[p], UY);
+                    const P p2 = fma2(Y[p], Y[p], XZ2), xq = fma2(Y[p], QY, XQ);
+                    const P S = mul2(mul2(CS, fma2(p2, I5T, splat(T(-1)))), xq);
+                    const P b = fma2(GXZ, DY.p[p], add2(GXZ, DY.p[p]));
+                    const P tgt = fma2(b, S, add2(b, S));
+                    // the departure from the target from its parts (see the scalar march)
+                    const P dinc = DI.p[p];
+                    P dep = sub2(h, tgt), lo = zero;
+                    if (STAGE >= 2) dep = add2(dep, dinc);
+                    if constexpr (kLo && STAGE == 3) {
+                        const unsigned q = p ? LQ.y : LQ.x;
+                        lo = make_float2(lo_decode(q, h.x), lo_decode(q >> 16, h.y));
+                        dep = add2(dep, lo);
+                    }
+                    // Eq. (flux) and the relaxation, both scaled by the stage's share of dt
+                    const P d12 = w[p].d12;  // this cell minus the upwind one
+                    const P cp = carried_corr<T>(w[p], nx.p[p]);
+                    const P div = add2(d12, sub2(cp, CM[p]));
+                    CM[p] = cp;
+                    P inc = fma2(dep, NIT, mul2(S1, div));
+                    if (STAGE == 2) inc = fma2(splat(T(0.25)), dinc, inc);
+                    if (STAGE == 3) inc = fma2(splat(T(2.0 / 3.0)), dinc, inc);
+                    if (STAGE < 3) {
+                        st.p[p] = inc;
+                        out[p] = add2(h, inc);
+                    } else if constexpr (kLo) {
+                        const P t = add2(lo, inc), h2 = add2(h, t), lo2 = sub2(t, sub2(h2, h));
+                        if (in) __stcg(reinterpret_cast<unsigned*>(lop) + p, lo_encode2(lo2, h2));
+                        st.p[p] = out[p] = h2;
+                    } else {
+                        st.p[p] = out[p] = add2(h, inc);
+                    }
+                }
+                // w f times the powers of xi_y; columns past the chunk hold no data
+                const P o = in ? mul2(out[p], WV[p]) : zero;
+                const P o1 = mul2(o, Y[p]), o2 = mul2(o1, Y[p]);
+                A0 = p ? add2(A0, o) : o;
+                A1 = p ? add2(A1, o1) : o1;
+                A2 = p ? add2(A2, o2) : o2;
+                A3 = p ? fma2(o2, Y[p], A3) : mul2(o2, Y[p]);
+            }
+            if (STAGE > 0 && in) {
+                if constexpr (sizeof(T) == 4) {
+                    __stcg(reinterpret_cast<float4*>(outp),
+                           make_float4(st.p[0].x, st.p[0].y, st.p[1].x, st.p[1].y));
+                } else {
+                    __stcg(reinterpret_cast<double2*>(outp), st.p[0]);
+                    __stcg(reinterpret_cast<double2*>(outp) + 1, st.p[1]);
+                }
+            }
+            // the 13 moments about the record's u: 1, xi_a, xi_a xi_b, |xi|^2 xi_a
+            const A x = X.x, z = Z.x, xz2 = XZ2.x;
+            const A a0 = A0.x + A0.y, a1 = A1.x + A1.y, a2 = A2.x + A2.y, a3 = A3.x + A3.y;
+            const A m1 = a0 * x, m3 = a0 * z, e = xz2 * a0 + a2;  // e: |xi|^2
+            A* rd = red + ((size_t)cc * (kThreads / 32) + warp) * 16;
+            if constexpr (sizeof(T) == 4) {
+                const float4 q[4] = {make_float4(a0, m1, a1, m3), make_float4(m1 * x, a2, m3 * z, a1 * x),
+                                     make_float4(m3 * x, a1 * z, e * x, xz2 * a1 + a3),
+                                     make_float4(e * z, 0.f, 0.f, 0.f)};
+                const float tot = warp_totals13(q, reinterpret_cast<float4*>(recs) + warp * 128, lane);
+                if ((lane & 4) == 0) rd[4 * (lane & 3) + 2 * (lane >> 4) + ((lane >> 3) & 1)] = tot;
+            } else {
+                A acc[16] = {a0, m1, a1, m3, m1 * x, a2, m3 * z, a1 * x, m3 * x, a1 * z, e * x, xz2 * a1 + a3, e * z,
+                             A(0), A(0), A(0)};
+                const A tot = reduce_scatter16<A>(acc, lane);
+                const int m = (lane >> 4 & 1) * 8 + (lane >> 3 & 1) * 4 + (lane >> 2 & 1) * 2 + (lane >> 1 & 1);
+                if ((lane & 1) == 0) rd[m] = tot;
+            }
+            outp += ostep;
+            if (kD) dop += ostep;
+            if (kLo && STAGE == 3) lop += ostep;
+        }
+    } else if constexpr (kPair && !RED) {
         // ---- 5 (FP32, full model). The march of section 5 below with the thread's
         // velocities as adjacent pairs: the same operations, two velocities per packed
         // FP32 instruction; rows, increments and outputs move as 64-bit pairs and the two
@@ -1037,11 +1430,11 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
 }
 
 // ---- host-side launch of one stage-kernel instantiation ----------------------
-template <typename T, int V, int STAGE, bool RED>
+template <typename T, int V, int STAGE, bool RED, bool GRP>
 static cudaError_t launch_stage_t(const InstDev* d_inst, const Tile* d_tiles, int ntiles, size_t smem,
                                   int fuse, cudaStream_t st)
 {
-    auto kfn = stage_kernel<T, V, STAGE, RED>;
+    auto kfn = stage_kernel<T, V, STAGE, RED, GRP>;
     if (smem > 40 * 1024) {  // with the static arrays above the default limit of 48 KB
         cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1059,15 +1452,15 @@ static cudaError_t launch_stage_t(const InstDev* d_inst, const Tile* d_tiles, in
     return cudaLaunchKernelEx(&cfg, kfn, d_inst, d_tiles, fuse);
 }
 
-template <typename T, int V, bool RED>
+template <typename T, int V, bool RED, bool GRP = false>
 static cudaError_t launch_stage_r(int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
                                   cudaStream_t st)
 {
     switch (stage) {
-        case 0: return launch_stage_t<T, V, 0, RED>(d, t, n, smem, fuse, st);
-        case 1: return launch_stage_t<T, V, 1, RED>(d, t, n, smem, fuse, st);
-        case 2: return launch_stage_t<T, V, 2, RED>(d, t, n, smem, fuse, st);
-        default: return launch_stage_t<T, V, 3, RED>(d, t, n, smem, fuse, st);
+        case 0: return launch_stage_t<T, V, 0, RED, GRP>(d, t, n, smem, fuse, st);
+        case 1: return launch_stage_t<T, V, 1, RED, GRP>(d, t, n, smem, fuse, st);
+        case 2: return launch_stage_t<T, V, 2, RED, GRP>(d, t, n, smem, fuse, st);
+        default: return launch_stage_t<T, V, 3, RED, GRP>(d, t, n, smem, fuse, st);
     }
 }
 
@@ -1075,6 +1468,8 @@ template <typename T, bool RED>
 static cudaError_t launch_stage_m(int V, int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
                                   cudaStream_t st)
 {
+    if constexpr (!RED)
+        if (V == kGroupedV) return launch_stage_r<T, 4, false, true>(stage, d, t, n, smem, fuse, st);
     if (V == 1) return launch_stage_r<T, 1, RED>(stage, d, t, n, smem, fuse, st);
     if (V == 2) return launch_stage_r<T, 2, RED>(stage, d, t, n, smem, fuse, st);
     return launch_stage_r<T, 4, RED>(stage, d, t, n, smem, fuse, st);

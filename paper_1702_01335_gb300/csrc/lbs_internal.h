@@ -24,6 +24,7 @@ constexpr int kNMom = 13;       // raw moments accumulated per cell
 constexpr int kRecHead = 12;    // scalars at the head of a cell record
 constexpr int kThreads = 128;   // threads of a stage CTA
 constexpr int kMaxZT = 64;      // cells of a z-tile
+constexpr int kGroupedV = 64;   // the launchers' V for the grouped layout of V = 4
 
 enum { QUAD_FULL = 0, QUAD_HALF = 1 };
 

@@ -59,3 +59,33 @@ def test_finalize_cells_per_cta_agree(Nz, n, reduced, prec, tol):
         assert rel_err(a.populations(i), b.populations(i)) < tol, i
         pa, pb = a.profiles(i), b.profiles(i)
         assert max(np.abs(pa[k] - pb[k]).max() for k in pa) < tol, i
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("Qx,Qy,Qz,Nz,ZT", [(1, 4, 1, 6, 3), (3, 4, 7, 19, 5), (5, 8, 9, 37, 16), (16, 4, 9, 21, 64),
+                                             (4, 12, 3, 11, 12), (1, 100, 3, 9, 4)])
+@pytest.mark.parametrize("half", [0, 1])
+def test_grouped_layout_matches_one_velocity_per_thread(Qx, Qy, Qz, Nz, ZT, half, prec):
+    """Four adjacent velocities per thread (V = 4 with Qy a multiple of four) against one per
+    thread (V = 1): one or several chunks with ragged last ones (half ranges of 4 to 576
+    velocities, 1, 3 or 25 groups of y), tiles of 3 cells up to the whole channel, one or two
+    walls.  The two layouts differ by rounding: 1e-12 (FP64) and 1e-5 (FP32 storage) of the
+    largest population after 8 steps."""
+    P = _lbs()
+    from paper_1702_01335_gb300 import Instance, Solver
+    pr = P.LBS_FP64 if prec == "fp64" else P.LBS_FP32
+    inst = Instance(Qx=Qx, Qy=Qy, Qz=Qz, N_eq=3, Nz=Nz, A=0.8, half=half, Kn=0.3, u_w=0.4, Pr=2.0 / 3.0, visc_law=1,
+                    visc_param=0.5, cfl=0.4)
+    a, b = Solver(inst, precision=pr), Solver(inst, precision=pr)
+    a.set_tiling(4, ZT, 0)
+    b.set_tiling(1, 4, 0)
+    rng = np.random.default_rng(7)
+    z = np.linspace(-1.0, 1.0, Nz)[:, None]
+    d = (0.1 * np.sin(2 * z) + 0.02 * rng.standard_normal((1, inst.Q))) * (1 + 0.1 * z * z)
+    for s in (a, b):
+        s.set_state(0, d.astype(s.dtype))
+        s.step(8)
+    tol = 1e-12 if prec == "fp64" else 1e-5
+    assert rel_err(a.populations(), b.populations()) < tol
+    pa, pb = a.profiles(), b.profiles()
+    assert max(np.abs(pa[k] - pb[k]).max() for k in pa) < 10 * tol
