@@ -24,7 +24,7 @@ CANDIDATES = tuple((V, ZT, F) for V in (1, 2, 4) for ZT in (4, 6, 8, 12, 16, 24,
 _cache = {}
 
 
-_KERNEL_SOURCES = ("kernels.cuh", "finalize.cuh", "kernels.cu", "lbs_internal.h", "stage_f32_full.cu", "stage_f32_red.cu",
+_KERNEL_SOURCES = ("kernels.cuh", "finalize.cuh", "pdl.cuh", "kernels.cu", "lbs_internal.h", "stage_f32_full.cu", "stage_f32_red.cu",
                    "stage_f64_full.cu", "stage_f64_red.cu")
 
 

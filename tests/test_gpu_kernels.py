@@ -89,3 +89,28 @@ def test_grouped_layout_matches_one_velocity_per_thread(Qx, Qy, Qz, Nz, ZT, half
     assert rel_err(a.populations(), b.populations()) < tol
     pa, pb = a.profiles(), b.profiles()
     assert max(np.abs(pa[k] - pb[k]).max() for k in pa) < 10 * tol
+
+
+@pytest.mark.parametrize("sizes,B", [((1, 1, 1, 1), 1), ((6, 31, 31, 33), 65), ((6, 200, 200, 384), 300),
+                                     ((7, 40, 40, 40), 20000), ((260, 300, 300, 17), 40),
+                                     ((5, 900, 900, 900), 70)])
+def test_network_tiles_at_ragged_sizes(sizes, B):
+    """The network's products where its tiles are ragged: single entries, sizes one below and
+    above a tile, inner sizes above a staged slice of 256, rows that are not 16-byte multiples,
+    a batch past the switch to the large tile; outputs, loss and gradients within the bounds of
+    the BF16 roundings (test_gpu_mlp.error_bounds) against the oracle."""
+    from oracle import mlp as om
+    from tests.test_gpu_mlp import _setup, error_bounds
+    net, pf, x, t, xd, td = _setup(sizes, B, seed=9)
+    E = error_bounds(pf, x, t)
+    y = net.forward(xd).cpu().numpy()
+    y_ora, _ = om.forward(pf, x)
+    floor = 1e-6  # entries whose every term is zero to rounding
+    assert np.all(np.abs(y - y_ora) <= E["y"] + floor)
+    loss, g = net.loss_grad(xd, td, want_grad=True)
+    L_ora, g_ora = om.loss_and_grads(pf, x, t)
+    assert abs(loss / L_ora - 1) < 1e-3
+    gg = net.unpack(g.astype(np.float64))
+    for k in g_ora:
+        assert np.all(np.abs(gg[k] - g_ora[k]) <= E[k] + floor * np.abs(g_ora[k]).max()), k
+    net.close()
