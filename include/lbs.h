@@ -264,7 +264,8 @@ lbs_status lbs_moments_static(lbs_handle h, int inst, const void* f_dev, double*
 lbs_status lbs_profile_steps(lbs_handle h, long nsteps, double* out_ms);
 
 /* Work decomposition of the stage kernel: each CTA of 128 threads updates 128*V
- * velocities (V in {1, 2, 4}) of about ZT consecutive cells (3 <= ZT <= 64).  No
+ * velocities (V in {1, 2, 4}; V = 1 in FP64 32 for a small batch) of about ZT consecutive
+ * cells (3 <= ZT <= 64).  No
  * effect on the arithmetic in FP64 but for the order of operations.  In FP32 the full
  * model with V = 2 or 4 gives each thread adjacent velocity pairs, moved as 64-bit words
  * and updated by packed two-lane FP32 instructions: the same operations up to the
@@ -280,8 +281,7 @@ lbs_status lbs_profile_steps(lbs_handle h, long nsteps, double* out_ms);
  * so that one half's FP64 finalisation overlaps the other half's stage kernel
  * (the step forks from and joins back into the handle's stream; a batch of one
  * instance steps as with fuse = 0).  Used by the tile autotuner.  Without a call
- * a solver starts with V = 1, ZT = 4 below 2^22 cell x velocity updates per step
- * and V = 4, ZT = 12 (FP64: 8) above (V = 1 where the FP32 pair layout does not apply), fuse = 0.  Waits for the handle's stream and
+ * a solver starts with a tiling chosen by its precision and sizes and fuse = 0.  Waits for the handle's stream and
  * recomputes the moment partials of the current state.  LBS_ERR_ARG outside the
  * ranges. */
 lbs_status lbs_set_tiling(lbs_handle h, int V, int ZT, int fuse);

@@ -57,6 +57,8 @@ struct InstHost {
     std::vector<double> xc, xf;  // cell centres (s = -3..Nz+2, 0-based), interfaces
 };
 
+constexpr long kZSplitPairs = 4 * 608;
+
 constexpr size_t kSmemBudget = 200 * 1024;  // dynamic shared memory of a stage CTA
 
 struct Pool {  // bump allocator over one device allocation
@@ -78,6 +80,8 @@ struct lbs_solver {
     int fin_mode = 0, fin_cells = 4;  // lbs_set_finalize's mode; cells per CTA of the finalisation
     int reduced = 0;                 // the batch runs the phi / chi model (all instances alike)
     int groupable = 0;               // full model, Qy a multiple of four in every instance
+    int zsplit = 0;                  // FP64 batch small enough for one velocity and cell per warp lane
+    int min_columns = kThreads;      // velocities of a CTA at V = 1
     std::vector<InstHost> ih;
     std::vector<InstDev> idev;
     InstDev* d_inst = nullptr;
@@ -224,19 +228,94 @@ static std::vector<double> rounded(const std::vector<double>& v)
     return r;
 }
 
-// The layout of the stage kernel for the launchers: V, or the grouped form of V = 4 (four
-// adjacent velocities per thread with common x and z nodes), which needs Qy a multiple of four
-// in every instance of a full-model batch and, where it applies, is the faster one (256 x C2
-// 987 us of stage kernels per step against 1061, 16 x C2 in FP64 2365 against 3063).
+// The layout of the stage kernel for the launchers.
+//  - V = 4: the grouped form (four adjacent velocities per thread with common x and z nodes)
+//    where every instance's Qy is a multiple of four (full model); it is the faster one (256 x
+//    C2 987 us of stage kernels per step against 1061, 16 x C2 in FP64 2365 against 3063).
+//  - V = 1 in FP64: the grouped form too, 128 velocities per CTA, whose warps split the tile's
+//    cells (one C2 channel 225 us per step at 16-cell tiles, four channels 663, against 285 and
+//    776 us with one velocity per thread and four-cell tiles).  In FP32 that form is slower
+//    (one C2 channel 57 us per step against 48: the warps' common start-up outweighs the cells).
+//  - V = 1 in FP64 for a batch of few cells and velocities (zsplit): one velocity per thread,
+//    32 per CTA, the warps splitting the cells, which spreads the FP64 work over the most
+//    schedulers (one C1 channel 102 -> 63 us per step, the low-Mach runs 107 -> 88).
 static int stage_layout(const lbs_solver* h)
 {
-    return h->V == 4 && h->groupable ? kGroupedV : h->V;
+    if (h->V == 4) return h->groupable ? 4 | kGrouped : 4;
+    if (h->V == 1) return h->zsplit ? 1 | kZSplit : h->groupable && !h->fp32 ? 4 | kGrouped | kZSplit : 1;
+    return h->V;
+}
+
+// z-tiles of about zt cells of an instance, at least 3 cells each
+static int z_tiles(int Nz, int zt) { return std::max(1, std::min((Nz + zt - 1) / zt, Nz / 3)); }
+
+// Estimated time of a stage at tiles of zt cells, in march steps: the waves of CTAs (as many
+// per SM as registers and shared memory allow) times a CTA's steps, its start counted as
+// `start` steps more
+static double stage_cost(const lbs_solver* h, int zt, int per_sm, double start)
+{
+    const int layout = stage_layout(h), KC = layout_columns(layout);
+    long ctas = 0, steps = 0;
+    size_t smem = 0;
+    for (const InstHost& I : h->ih) {
+        const int nch = 2 * ((I.Q / 2 + KC - 1) / KC), nzt = z_tiles(I.Nz, zt);
+        const int nzm = std::min((KC - 1) / (I.Qx * I.Qy) + 2, I.Qz);
+        ctas += (long)nch * nzt;
+        steps += (long)nch * I.Nz;
+        smem = std::max(smem, stage_smem_bytes(h->fp32, layout, (I.Nz + nzt - 1) / nzt, I.Qx, I.Qy, nzm,
+                                               rec_stride_of(I.Qx, I.Qy, I.Qz)));
+    }
+    if (smem > kSmemBudget) return 1e300;
+    const long fit = std::max<long>(1, std::min<long>(per_sm, 228 * 1024 / (smem + 1152 + 1024)));
+    const long waves = (ctas + 152 * fit - 1) / (152 * fit);
+    return waves * ((double)steps / ctas + start);
+}
+
+// The tiling a solver starts with.
+//  - FP32, grouped layout: V = 4 once its four-cell tiles are more than one CTA per SM and its
+//    512-velocity chunks at least half full, with the tile length of the least stage_cost (us
+//    per step, C2 replicas at V = 1 four cells / V = 4 four cells / the chosen one: 1 channel
+//    46.6 / 48.2 / 46.6, 4 channels 75 / 56 / 56, 8 channels 119 / 80 / 70 at seven cells, 64
+//    channels 724 / 394 / 311 at twelve; 48 channels of 64 to 256 velocities per half range,
+//    whose chunks are mostly empty, 80 / 93 / 75 at V = 1 and six cells).
+//  - FP32 otherwise: V = 4 from 2^22 velocity-cells (pairs, or the phi / chi model), else V = 1,
+//    the tile length by the same estimate.
+//  - FP64: bound by the FP64 pipe, which short tiles load more evenly (16 x C2 at V = 4: 2365 us
+//    of stage kernels per step at 12 cells, 2004 at 8); V = 1 for less than 2^22
+//    velocity-cells, with tiles of 16 cells in the grouped layout (four per warp).
+static void choose_tiling(lbs_solver* h)
+{
+    long work = 0, chunks4 = 0, full4 = 0;
+    bool pairs = true;  // the pair layout of V = 4 applies
+    for (const InstHost& I : h->ih) {
+        work += (long)I.Nz * I.Q;
+        const int nch = 2 * ((I.Q / 2 + 511) / 512);
+        chunks4 += (long)nch * z_tiles(I.Nz, 4);
+        full4 += (long)I.Nz * nch * 512;
+        pairs = pairs && I.Q / 2 % 2 == 0;
+    }
+    const bool big = work >= (1L << 22);
+    if (!h->fp32) {
+        h->V = big ? 4 : 1;
+        h->ZT = big ? (h->groupable ? 8 : 12) : h->groupable && !h->zsplit ? 16 : 4;
+        return;
+    }
+    const bool grouped = h->groupable && chunks4 > 152 && 2 * work >= full4;
+    h->V = grouped || (big && (h->reduced || pairs)) ? 4 : 1;
+    double best = 1e300;
+    for (int zt = 4; zt <= 16; ++zt) {
+        const double c = h->V == 4 ? stage_cost(h, zt, 4, 4.0) : stage_cost(h, zt, 7, 8.0);
+        if (c < best) {
+            best = c;
+            h->ZT = zt;
+        }
+    }
 }
 
 static void build_tiles(lbs_solver* h, std::vector<Tile>& tiles)
 {
     tiles.clear();
-    const int KC = kThreads * h->V;
+    const int KC = layout_columns(stage_layout(h));
     size_t smem = 0;
     for (int b = 0; b < h->ninst; ++b) {
         InstHost& I = h->ih[b];
@@ -256,8 +335,7 @@ static void build_tiles(lbs_solver* h, std::vector<Tile>& tiles)
         // z-tiles of about ZT cells, at least 3 cells each, within the shared-memory budget
         int zt = std::max(3, std::min(h->ZT, kMaxZT));
         while (zt > 3 && stage_smem_bytes(h->fp32, stage_layout(h), zt, I.Qx, I.Qy, nzm_max, rs) > kSmemBudget) --zt;
-        int nzt = std::min((I.Nz + zt - 1) / zt, I.Nz / 3);
-        nzt = std::max(nzt, 1);
+        const int nzt = z_tiles(I.Nz, zt);
         const int base = I.Nz / nzt, rem = I.Nz % nzt;
         const int zmax = base + (rem ? 1 : 0);
         I.nzt = nzt;
@@ -279,18 +357,10 @@ static void build_tiles(lbs_solver* h, std::vector<Tile>& tiles)
     h->nA = 0;
     h->ntilesA = 0;
     if (h->ninst >= 2) {
-        size_t t = 0;
         int b = 0;
-        while (b < h->ninst - 1) {
-            size_t tb = 0;
-            for (const Tile& x : tiles)
-                if (x.inst == b) ++tb;
-            if (2 * (t + tb) > tiles.size() && b > 0) break;
-            t += tb;
-            ++b;
-        }
+        while (b < h->ninst - 1 && (b == 0 || 2 * (size_t)h->tile_first[b + 1] <= tiles.size())) ++b;
         h->nA = b;
-        h->ntilesA = (int)t;
+        h->ntilesA = h->tile_first[b];
     }
 }
 
@@ -350,6 +420,7 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         h->maxNz = std::max(h->maxNz, I.Nz);
         h->nb = std::max(h->nb, std::max(I.Nx, std::max(I.Ny, I.Nzq)));  // the batch's largest order
     }
+    choose_tiling(h);
     build_tiles(h, tiles);
     for (int b = 0; b < h->ninst; ++b) {
         InstHost& I = h->ih[b];
@@ -441,10 +512,18 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         D.dt = I.dt; D.tol = 0.0;
         D.res_uscale = std::max(std::fabs(d.u_w) * std::sqrt((double)Nz), 1e-30);
         const std::vector<double>& xc = I.xc;  // xc[s + 3]
-        lagrange3(xc[Nz + 3], xc[Nz + 2], xc[Nz + 1], xc[Nz], D.ext_top[0]);
-        lagrange3(xc[Nz + 4], xc[Nz + 3], xc[Nz + 2], xc[Nz + 1], D.ext_top[1]);
-        lagrange3(xc[2], xc[3], xc[4], xc[5], D.ext_bot[0]);
-        lagrange3(xc[1], xc[2], xc[3], xc[4], D.ext_bot[1]);
+        lagrange3(xc[Nz + 3], xc[Nz + 2], xc[Nz + 1], xc[Nz], D.walls.top[0]);
+        lagrange3(xc[Nz + 4], xc[Nz + 3], xc[Nz + 2], xc[Nz + 1], D.walls.top[1]);
+        lagrange3(xc[2], xc[3], xc[4], xc[5], D.walls.bot[0]);
+        lagrange3(xc[1], xc[2], xc[3], xc[4], D.walls.bot[1]);
+        for (int g = 0; g < 2; ++g)
+            for (int e = 0; e < 3; ++e) {
+                D.walls2.top[g][e] = float(D.walls.top[g][e]);
+                D.walls2.bot[g][e] = float(D.walls.bot[g][e]);
+            }
+        auto magic = [](unsigned d) { return d == 1 ? 0u : unsigned(((1ull << 32) + d - 1) / d); };
+        D.mQy = magic(I.Qy);
+        D.mQxQy = magic(I.Qx * I.Qy);
         // D = sum over incoming velocities of w p_z Gw, from the stored (rounded) tables
         // (Gw = 1 + the stored deviation on each axis)
         const std::vector<double> wx = rounded<T>(t.wx), wy = rounded<T>(t.wy), wz = rounded<T>(t.wz);
@@ -499,10 +578,10 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         const size_t nf = (size_t)Nz * I.Q;
         o.F2 = pool.take(nf * es);  // F0, F1, L0: below
         o.rec = pool.take((size_t)Nz * rec_stride_of(I.Qx, I.Qy, I.Qz) * es);
-        const size_t maxch = 2 * ((I.Q / 2 + kThreads - 1) / kThreads);  // chunks at V = 1, the finest tiling
+        const size_t maxch = 2 * ((I.Q / 2 + h->min_columns - 1) / h->min_columns);  // at the finest tiling, V = 1
         o.partial = pool.take(maxch * Nz * kNMom * 8);
         o.flux = pool.take(maxch * 2 * 8);
-        o.nw = pool.take(2 * 8);  // prof: below
+        o.nw = pool.take(sizeof(WallDensity));  // prof: below
         o.Wold = pool.take(3 * (size_t)Nz * 8); o.Wnew = pool.take(3 * (size_t)Nz * 8);
         o.res = pool.take(8); o.steps = pool.take(8); o.active = pool.take(4);  // status: below
         o.zcount = pool.take(4 * (size_t)std::max(1, Nz / 3)); o.icount = pool.take(4);
@@ -545,7 +624,8 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
     const size_t inst_off = pool.take(sizeof(InstDev) * h->ninst);
     size_t max_tiles = 0;  // tiles of the finest tiling (V = 1, 3-cell z-tiles)
     for (int b = 0; b < h->ninst; ++b)
-        max_tiles += (size_t)(2 * ((h->ih[b].Q / 2 + kThreads - 1) / kThreads)) * std::max(1, h->ih[b].Nz / 3);
+        max_tiles += (size_t)(2 * ((h->ih[b].Q / 2 + h->min_columns - 1) / h->min_columns)) *
+                     std::max(1, h->ih[b].Nz / 3);
     h->max_tiles = max_tiles;
     const size_t tile_off = pool.take(sizeof(Tile) * max_tiles);
     const size_t macro_off = pool.take(8 * (size_t)h->maxNz * 8);
@@ -591,7 +671,7 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         D.cur = reinterpret_cast<int*>(P + o.cur);
         D.partial = P + o.partial;
         D.flux_part = reinterpret_cast<double*>(P + o.flux);
-        D.nw = reinterpret_cast<double*>(P + o.nw);
+        D.nw = reinterpret_cast<WallDensity*>(P + o.nw);
         D.prof = reinterpret_cast<double*>(P + o.prof);
         D.Wold = reinterpret_cast<double*>(P + o.Wold);
         D.Wnew = reinterpret_cast<double*>(P + o.Wnew);
@@ -860,22 +940,14 @@ lbs_status lbs_batch_create(lbs_handle* out, const lbs_instance_desc* desc, int 
     h->esize = h->fp32 ? 4 : 8;
     h->ninst = n;
     h->ih.resize(n);
-    long work = 0;
+    // FP64: (cell, 32 velocities of a half range) pairs of the batch; up to four per warp
+    // scheduler (608 of them) each gets a warp of its own
+    long pairs = 0;
     for (int b = 0; b < n; ++b)
-        work += (long)desc[b].grid.Nz * 2 * desc[b].orders.Qx * std::max(desc[b].orders.Qy, 2) *
-                desc[b].orders.Qz_half;
-    // untuned default: small batches are latency-bound (short z-tiles, one velocity per
-    // thread, more CTAs); large ones take the throughput tiling.  Finalisation apart.
-    // FP64 is bound by the FP64 pipe and takes shorter tiles, which spread more evenly over the
-    // SMs (16 x C2, grouped layout: 2365 us of stage kernels per step at 12 cells, 2004 at 8)
-    h->V = work >= (1L << 22) ? 4 : 1;
-    h->ZT = work < (1L << 22) ? 4 : h->fp32 ? 12 : 8;
-    // the FP32 full model with V = 2, 4 takes velocities in pairs (64-bit words), which
-    // needs Q / 2 even in every instance; else one velocity per thread
-    for (int b = 0; b < n; ++b)
-        if (h->fp32 && !h->reduced &&
-            (desc[b].orders.Qx * std::max(desc[b].orders.Qy, 2) * desc[b].orders.Qz_half) % 2)
-            h->V = 1;
+        pairs += (long)desc[b].grid.Nz * 2 *
+                 ((desc[b].orders.Qx * std::max(desc[b].orders.Qy, 2) * desc[b].orders.Qz_half + 31) / 32);
+    h->zsplit = !h->fp32 && pairs <= kZSplitPairs;
+    h->min_columns = h->zsplit ? kThreads / 4 : kThreads;
     h->fuse = 0;
     if (cuda_stream) {
         h->stream = static_cast<cudaStream_t>(cuda_stream);

@@ -715,7 +715,10 @@ static __device__ __noinline__ void finalize_instance(const InstDev& I, int stag
         for (int w = 0; w < kThreads / 32; ++w) x += red[w * 8 + i];
     if (lane < 2) {  // the partials sum w p_z over the deviations: add the rest state's flux
         const double nw = -((lane ? I.frest_top : I.frest_bot) + x) * (lane ? I.iDtop : I.iDbot);
-        I.nw[lane] = nw;
+        I.nw->d[2 * lane] = nw - 1.0;
+        I.nw->d[2 * lane + 1] = nw;
+        I.nw->f[2 * lane] = float(nw - 1.0);
+        I.nw->f[2 * lane + 1] = float(nw);
         if (!isfinite(nw)) atomicOr(I.status, STATUS_NONFINITE);
     }
     if (stage == 3) {

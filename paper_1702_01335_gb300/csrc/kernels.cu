@@ -120,12 +120,13 @@ cudaError_t launch_gather_moments(const InstDev* d_inst, int ninst, const double
 
 size_t stage_smem_bytes(int fp32, int V, int zn, int Qx, int Qy, int nzm, int rstride)
 {
-    const bool grouped = V == kGroupedV;
-    const int KC = kThreads * (grouped ? 4 : V), G = factor_stride(Qx, Qy, nzm, grouped, fp32 ? 4 : 8);
+    const bool grouped = V & kGrouped;
+    const int KC = layout_columns(V), G = factor_stride(Qx, Qy, nzm, grouped, fp32 ? 4 : 8);
     // element and accumulator sizes from the kernel's own types, so that the host's
     // dynamic shared-memory size always covers the kernel's layout
     return stage_smem(zn, KC, G, fp32 ? (int)sizeof(float) : (int)sizeof(double),
-                      fp32 ? (int)sizeof(Acc<float>::type) : (int)sizeof(Acc<double>::type), rstride, grouped)
+                      fp32 ? (int)sizeof(Acc<float>::type) : (int)sizeof(Acc<double>::type), rstride, grouped,
+                      V & kZSplit ? 4 : 1)
         .total;
 }
 

@@ -197,6 +197,24 @@ static __device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c)
     return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
 }
 static __device__ __forceinline__ double2 splat(double a) { return make_double2(a, a); }
+// and single velocities of either type by the same names
+#define LBS_SCALAR(T)                                                                  \
+    static __device__ __forceinline__ T add2(T a, T b) { return a + b; }               \
+    static __device__ __forceinline__ T sub2(T a, T b) { return a - b; }               \
+    static __device__ __forceinline__ T mul2(T a, T b) { return a * b; }               \
+    static __device__ __forceinline__ T fma2(T a, T b, T c) { return fma(a, b, c); }
+LBS_SCALAR(float)
+LBS_SCALAR(double)
+#undef LBS_SCALAR
+template <typename P> struct Constant {
+    static __device__ __forceinline__ P of(double a) { return P(a); }
+};
+template <> struct Constant<float2> {
+    static __device__ __forceinline__ float2 of(double a) { return splat(float(a)); }
+};
+template <> struct Constant<double2> {
+    static __device__ __forceinline__ double2 of(double a) { return splat(a); }
+};
 template <typename T> struct Two;
 template <> struct Two<float> { typedef float2 type; };
 template <> struct Two<double> { typedef double2 type; };
@@ -225,6 +243,13 @@ static __device__ __forceinline__ float2 carried_weights(float2 s1, float2 s2, f
     const float2 inv = make_float2(rcp_approx(3.f * sw.x), rcp_approx(3.f * sw.y));
     return mul2(fma2(w1, e1, fma2(w2, e2, mul2(w3, e3))), inv);
 }
+static __device__ __forceinline__ float carried_weights(float s1, float s2, float s3, float e1, float e2, float e3)
+{
+    const float w1 = rcp_approx(fmaf(s1, s1, kWenoFloor));
+    const float w2 = 6.f * rcp_approx(fmaf(s2, s2, kWenoFloor));
+    const float w3 = 3.f * rcp_approx(fmaf(s3, s3, kWenoFloor));
+    return fmaf(w1, e1, fmaf(w2, e2, w3 * e3)) * rcp_approx(3.f * ((w1 + w2) + w3));
+}
 static __device__ __forceinline__ double carried_weights(double q1, double q2, double q3, double e1, double e2,
                                                          double e3)
 {
@@ -242,13 +267,14 @@ static __device__ __forceinline__ double2 carried_weights(double2 s1, double2 s2
                         carried_weights(s1.y, s2.y, s3.y, e1.y, e2.y, e3.y));
 }
 // the correction of the interface ahead of v2 for the new value v4; advances the differences
-template <typename T, typename P>
+template <typename P>
 static __device__ __forceinline__ P carried_corr(Carried<P>& w, P v4)
 {
-    const P d34 = sub2(v4, w.v3), a3 = sub2(d34, w.d23), k3 = mul2(mul2(splat(T(13.0 / 3.0)), a3), a3);
-    const P b1 = fma2(splat(T(2)), w.d12, w.a1), b2 = add2(w.d12, w.d23), b3 = fma2(splat(T(-2)), w.d23, a3);
-    const P e1 = fma2(splat(T(1.5)), w.d12, w.a1), e2 = fma2(splat(T(0.5)), w.d12, w.d23);
-    const P e3 = fma2(splat(T(-0.5)), a3, mul2(splat(T(1.5)), w.d23));
+    typedef Constant<P> C;
+    const P d34 = sub2(v4, w.v3), a3 = sub2(d34, w.d23), k3 = mul2(mul2(C::of(13.0 / 3.0), a3), a3);
+    const P b1 = fma2(C::of(2.0), w.d12, w.a1), b2 = add2(w.d12, w.d23), b3 = fma2(C::of(-2.0), w.d23, a3);
+    const P e1 = fma2(C::of(1.5), w.d12, w.a1), e2 = fma2(C::of(0.5), w.d12, w.d23);
+    const P e3 = fma2(C::of(-0.5), a3, mul2(C::of(1.5), w.d23));
     const P c = carried_weights(fma2(b1, b1, w.k1), fma2(b2, b2, w.k2), fma2(b3, b3, k3), e1, e2, e3);
     w.v3 = v4;
     w.d12 = w.d23;
@@ -259,6 +285,21 @@ static __device__ __forceinline__ P carried_corr(Carried<P>& w, P v4)
     w.k2 = k3;
     return c;
 }
+// the state before the first of them, from the values v0 .. v3 of its stencil
+template <typename P>
+static __device__ __forceinline__ Carried<P> carried_start(P v0, P v1, P v2, P v3)
+{
+    const P K = Constant<P>::of(13.0 / 3.0);
+    Carried<P> w;
+    w.v3 = v3;
+    w.d12 = sub2(v2, v1);
+    w.d23 = sub2(v3, v2);
+    w.a1 = sub2(w.d12, sub2(v1, v0));
+    w.a2 = sub2(w.d23, w.d12);
+    w.k1 = mul2(mul2(K, w.a1), w.a1);
+    w.k2 = mul2(mul2(K, w.a2), w.a2);
+    return w;
+}
 
 template <typename T>
 __device__ __forceinline__ T weno5(T v0, T v1, T v2, T v3, T v4)
@@ -266,10 +307,18 @@ __device__ __forceinline__ T weno5(T v0, T v1, T v2, T v3, T v4)
     return v2 + weno5_corr<T>(v0, v1, v2, v3, v4);
 }
 
+// The warp's sum of a double-float or FP64 value, in every lane
+template <typename R>
+static __device__ __forceinline__ R warp_sum(R v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = r_add(v, r_shfl_xor(v, o));
+    return v;
+}
 // Block-wide FP64 sum (all threads get the result); deterministic order.
 static __device__ double block_sum(double v, double* red)
 {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    v = warp_sum(v);
     const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     __syncthreads();
     if ((threadIdx.x & 31) == 0) red[w] = v;
@@ -359,7 +408,7 @@ __host__ __device__ inline int factor_stride(int Qx, int Qy, int nzm, bool group
 enum { S_UX = 0, S_UY, S_UZ, S_QX, S_QY, S_QZ, S_CS, S_I5T, S_NITAU, S_IDZ, S_COUNT };
 __host__ __device__ inline size_t pad16(size_t b) { return (b + 15) & ~size_t(15); }
 __host__ __device__ inline StageSmem stage_smem(int zn, int KC, int G, int esize, int asize, int rstride,
-                                                    bool grouped)
+                                                    bool grouped, int zsplit)
 {
     StageSmem L;
     size_t o = 0;
@@ -370,7 +419,7 @@ __host__ __device__ inline StageSmem stage_smem(int zn, int KC, int G, int esize
     L.rec = o; o += rec > scratch ? rec : scratch;
     L.g = o; o += pad16((size_t)zn * G * esize);
     L.idz = o; o += pad16((size_t)zn * esize);
-    L.red = o; o += (size_t)zn * (kThreads / 32) * 16 * asize;
+    L.red = o; o += (size_t)zn * (kThreads / 32 / zsplit) * 16 * asize;
     L.sc = o; o += grouped ? (size_t)zn * S_COUNT * 8 : 0;  // 80 bytes a cell in either type
     L.total = o;
     return L;
@@ -418,19 +467,41 @@ static __device__ __forceinline__ float lo_decode(unsigned q16, float hi)  // q 
 // analyses F0 (moments and wall fluxes) without writing F.  RED selects the
 // phi / chi model (Sec. III, Eqs. boltz_red, sred_def): j = 0 is phi, j = 1 chi.
 // ----------------------------------------------------------------------------
+// n / d for 0 <= n < 2^15 and 2 <= d < 2^14 from m = ceil(2^32 / d) (the error m d - 2^32 < d
+// times n stays below 2^32); m = 0 stands for d = 1
+static __device__ __forceinline__ int div_small(int n, unsigned m) { return m ? __umulhi(n, m) : n; }
+// the walls' extrapolation weights and densities in the storage type
+static __device__ __forceinline__ const Walls<float>& wall_weights(const InstDev& I, float) { return I.walls2; }
+static __device__ __forceinline__ const Walls<double>& wall_weights(const InstDev& I, double) { return I.walls; }
+static __device__ __forceinline__ const float* stored_nw(const InstDev& I, float) { return I.nw->f; }
+static __device__ __forceinline__ const double* stored_nw(const InstDev& I, double) { return I.nw->d; }
+
+template <typename T, bool PACK> struct PackedAs { typedef T type; };
+template <> struct PackedAs<float, true> { typedef float2 type; };
+
 // Minimum resident CTAs per SM requested from the register allocator: the
 // per-velocity register window grows with V; the rarely taken finalisation
 // path may spill instead of lowering occupancy.
-template <typename T, int V> struct MinBlocks {
+template <typename T, int V, int ZW> struct MinBlocks {
     // FP32 at V = 4 fits 128 registers (four CTAs, sixteen warps per SM); FP64 values take
-    // two registers each and keep three
-    static constexpr int value = V == 1 ? 8 : V == 2 ? 6 : sizeof(T) == 4 ? 4 : 3;
+    // two registers each and keep three.  The small batches of ZW = 4 take what registers
+    // they can use.
+    static constexpr int value = ZW == 4 ? (V == 1 ? 4 : 2)
+                                 : V == 1 ? (sizeof(T) == 4 ? 7 : 5)
+                                 : V == 2 ? (sizeof(T) == 4 ? 6 : 4)
+                                          : sizeof(T) == 4 ? 4 : 3;
 };
 
 // GRP (V = 4, full model, Qy a multiple of 4 in every instance): a thread's four velocities
 // are adjacent, so they share the x and the z node.
-template <typename T, int V, int STAGE, bool RED, bool GRP>
-__global__ void __launch_bounds__(kThreads, MinBlocks<T, V>::value)
+// ZW = 4: the CTA's warps share 32 V velocities and split the tile's cells between them, for
+// batches too small to fill the GPU otherwise: a warp marches a quarter of the cells (one of a
+// four-cell tile), so a tile takes a quarter of the steps.  Rows, records and factors are
+// staged once for the four.
+// Measured, us per step: one C1 channel in FP64 102 -> 63, the low-Mach runs 107 -> 88, one C2
+// channel in FP64 285 -> 225.
+template <typename T, int V, int STAGE, bool RED, bool GRP, int ZW>
+__global__ void __launch_bounds__(kThreads, MinBlocks<T, V, ZW>::value)
 stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, int fuse)
 {
     typedef typename Acc<T>::type A;
@@ -440,22 +511,26 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     __shared__ __align__(8) uint64_t bar;
     __shared__ double wall_red[8 * (kThreads / 32)];
     __shared__ InstDev sI;
+    typedef typename Real<T>::type R;
     const Tile tile = tiles[blockIdx.x];
     const InstDev& I = stage_descriptor(insts + tile.inst, &sI);
 
     const int Nz = I.Nz, Q = I.Q, Qx = I.Qx, Qy = I.Qy, Qz = I.Qz, QxQy = I.QxQy;
     const int z0 = tile.z0, zn = tile.zn;            // cells z0 .. z0+zn-1 (0-based)
-    constexpr int KC = kThreads * V;
+    constexpr int NT = kThreads / ZW, KC = NT * V;   // threads along the velocities
     // chunks never straddle p_z = 0: this chunk's velocities share the sign of p_z
     const int Qh = Q >> 1, sgc = tile.chunk >= I.nchh;
     const int k0 = sgc * Qh + (tile.chunk - sgc * I.nchh) * KC;
     const int kend = min((sgc + 1) * Qh, k0 + KC), kn = kend - k0;
-    const int zm_lo = k0 / QxQy, zm_hi = (kend - 1) / QxQy, nzm = zm_hi - zm_lo + 1;
+    const int zm_lo = div_small(k0, I.mQxQy), zm_hi = div_small(kend - 1, I.mQxQy), nzm = zm_hi - zm_lo + 1;
     const int G = factor_stride(Qx, Qy, nzm, GRP, sizeof(T));  // per-cell factors held in smem
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ctid = ZW == 1 ? tid : lane, zw = ZW == 1 ? 0 : warp;
+    // this warp's part of the tile: cells zb .. zb + zc - 1
+    const int zb = zn * zw / ZW, zc = zn * (zw + 1) / ZW - zb;
 
     const int rstride = I.rec_stride;
-    const StageSmem L = stage_smem(zn, KC, G, sizeof(T), sizeof(A), rstride, GRP);
+    const StageSmem L = stage_smem(zn, KC, G, sizeof(T), sizeof(A), rstride, GRP, ZW);
     T* Fs = reinterpret_cast<T*>(smem_raw + L.fin);   // d rows: cells z0-3 .. z0+zn+2
     T* recs = reinterpret_cast<T*>(smem_raw + L.rec); // records of cells z0 .. z0+zn-1
     T* gsm = reinterpret_cast<T*>(smem_raw + L.g);
@@ -496,8 +571,8 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     // offset from the thread's first velocity tbase.
     // Grouped layout: the four velocities 4 tid .. 4 tid + 3.
     constexpr bool kPair = sizeof(T) == 4 && V % 2 == 0;
-    const int tbase = GRP ? 4 * tid : kPair ? 2 * tid : tid;
-    auto voff = [](int v) { return GRP ? v : kPair ? (v & 1) + (v >> 1) * 2 * kThreads : v * kThreads; };
+    const int tbase = GRP ? 4 * ctid : kPair ? 2 * ctid : ctid;
+    auto voff = [](int v) { return GRP ? v : kPair ? (v & 1) + (v >> 1) * 2 * NT : v * NT; };
     int ii[V], jj[V], zz[V], kl[V];
     T px[V], py[V], pz[V], apz[V];
     A wv[V], yv[V], p2v[V], wm[V];  // weight; p_y for the moments; |p|^2; w of the mass flux
@@ -509,9 +584,10 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         const int kc = ok[v] ? k0 + kl[v] : kend - 1;
         // (grouped: kn is a multiple of 4, so v = 0 stands for all four but for the y node; past
         // the chunk the y nodes still lie inside the table)
-        jj[v] = GRP ? (v ? jj[0] + v : kc % Qy & ~3) : kc % Qy;
-        ii[v] = GRP && v ? ii[0] : (kc / Qy) % Qx;
-        zz[v] = GRP && v ? zz[0] : kc / QxQy;
+        const int ky = div_small(kc, I.mQy);  // kc / Qy
+        zz[v] = GRP && v ? zz[0] : div_small(kc, I.mQxQy);
+        ii[v] = GRP && v ? ii[0] : ky - zz[v] * Qx;
+        jj[v] = GRP ? (v ? jj[0] + v : (kc - ky * Qy) & ~3) : kc - ky * Qy;
         const int sg = zz[v] >= Qz, m = zz[v] - sg * Qz;
         px[v] = GRP && v ? px[0] : ld<T>(I.px, ii[v]);
         py[v] = ld<T>(I.py, jj[v]);
@@ -615,32 +691,32 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
             if (dup == 2) to[1] = g;
         }
     } else if (STAGE > 0) {
-        for (int e = tid; e < zn * G; e += kThreads) {
-            const int c = e / G, r = e - c * G;
+        for (int c = warp; c < zn; c += kThreads / 32) {  // a warp per cell
             const T* rc = recs + (size_t)c * rstride;
-            T g;
-            if (r < Qx) {
-                const T s1 = rc[R_SCALE1];
-                g = s1 + (T(1) + s1) * rc[R_DX + r];
-            } else if (r < Qx + Qy) {
-                g = rc[R_DX + r];                               // dy[r - Qx]
-            } else {
-                g = rc[R_DX + Qx + Qy + zm_lo + r - Qx - Qy];   // dz[zm]
+            const T s1 = rc[R_SCALE1];
+            for (int r = lane; r < Qx + Qy + nzm; r += 32) {
+                T g;
+                if (r < Qx) g = s1 + (T(1) + s1) * rc[R_DX + r];
+                else if (r < Qx + Qy) g = rc[R_DX + r];                  // dy[r - Qx]
+                else g = rc[R_DX + Qx + Qy + zm_lo + r - Qx - Qy];       // dz[zm]
+                gsm[c * G + r] = g;
             }
-            gsm[e] = g;
         }
     }
 
     // ---- 4b. ghost rows (each thread fills only its own columns).  A ghost row holds
     //          the whole stage-input value d (+ increment); a cell's row holds d.
     const int rbase = 3 - z0;  // smem row of cell s is s + rbase
+    const auto& ext_top = wall_weights(I, T(0)).top;
+    const auto& ext_bot = wall_weights(I, T(0)).bot;
+    const T* nwt = stored_nw(I, T(0));  // n_w - 1 and n_w of the bottom wall, then of the top one
     auto rowval = [&](int row, int col) -> T {  // the stage input of a cell's row
         return kD ? Fs[(size_t)row * KC + col] + __ldca(Dg + (size_t)(row - rbase) * Q + k0 + col)
                   : Fs[(size_t)row * KC + col];
     };
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        if (!ok[v]) continue;  // columns past the chunk end hold no data
+        if (!ok[v] || zw != 0) continue;  // columns past the chunk end hold no data
         T* col = Fs + kl[v];
         if (z0 < 3 && I.half) {  // bounce-back on the centre line: ghost -1-s holds cell s
             // at the mirrored velocity (p_z, p_x reversed: other half range, node Qx-1-i;
@@ -656,13 +732,13 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
             if (!sgc) {  // incoming at the bottom wall: n_w times the wall equilibrium, minus 1
                 const T ax = ld<T>(I.gwx_bot, ii[v]), ay = ld<T>(I.gwy, jj[v]), az = ld<T>(I.gwz, zz[v]);
                 const T a = ax + ay + ax * ay, b = a + az + a * az;
-                const T g = T(I.nw[0] - 1.0) + T(I.nw[0]) * b;
+                const T g = nwt[0] + nwt[1] * b;
                 for (int s = -3; s <= -1; ++s)
                     if (s + rbase >= 0) col[(size_t)(s + rbase) * KC] = g;
             } else {      // outgoing: quadratic extrapolation (Appendix)
                 const T f1 = rowval(0 + rbase, kl[v]), f2 = rowval(1 + rbase, kl[v]), f3 = rowval(2 + rbase, kl[v]);
-                const T g0 = T(I.ext_bot[0][0]) * f1 + T(I.ext_bot[0][1]) * f2 + T(I.ext_bot[0][2]) * f3;
-                const T g1 = T(I.ext_bot[1][0]) * g0 + T(I.ext_bot[1][1]) * f1 + T(I.ext_bot[1][2]) * f2;
+                const T g0 = ext_bot[0][0] * f1 + ext_bot[0][1] * f2 + ext_bot[0][2] * f3;
+                const T g1 = ext_bot[1][0] * g0 + ext_bot[1][1] * f1 + ext_bot[1][2] * f2;
                 if (-1 + rbase >= 0) col[(size_t)(-1 + rbase) * KC] = g0;
                 if (-2 + rbase >= 0) col[(size_t)(-2 + rbase) * KC] = g1;
                 if (-3 + rbase >= 0) col[(size_t)(-3 + rbase) * KC] = g1;  // never read for p_z < 0
@@ -673,14 +749,14 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
             if (sgc) {
                 const T ax = ld<T>(I.gwx_top, ii[v]), ay = ld<T>(I.gwy, jj[v]), az = ld<T>(I.gwz, zz[v]);
                 const T a = ax + ay + ax * ay, b = a + az + a * az;
-                const T g = T(I.nw[1] - 1.0) + T(I.nw[1]) * b;
+                const T g = nwt[2] + nwt[3] * b;
                 for (int s = Nz; s <= Nz + 2; ++s)
                     if (s <= smax) col[(size_t)(s + rbase) * KC] = g;
             } else {
                 const T f1 = rowval(Nz - 1 + rbase, kl[v]), f2 = rowval(Nz - 2 + rbase, kl[v]),
                         f3 = rowval(Nz - 3 + rbase, kl[v]);
-                const T g0 = T(I.ext_top[0][0]) * f1 + T(I.ext_top[0][1]) * f2 + T(I.ext_top[0][2]) * f3;
-                const T g1 = T(I.ext_top[1][0]) * g0 + T(I.ext_top[1][1]) * f1 + T(I.ext_top[1][2]) * f2;
+                const T g0 = ext_top[0][0] * f1 + ext_top[0][1] * f2 + ext_top[0][2] * f3;
+                const T g1 = ext_top[1][0] * g0 + ext_top[1][1] * f1 + ext_top[1][2] * f2;
                 if (Nz <= smax) col[(size_t)(Nz + rbase) * KC] = g0;
                 if (Nz + 1 <= smax) col[(size_t)(Nz + 1 + rbase) * KC] = g1;
                 if (Nz + 2 <= smax) col[(size_t)(Nz + 2 + rbase) * KC] = g1;  // never read for p_z > 0
@@ -737,7 +813,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         // registers (20 moves per step less)
         constexpr int kUnroll = sizeof(T) == 4 ? 2 : 1;
         const P zero = splat(T(0));
-        const bool in = ok[0];
+        const bool in = ok[0] && zc > 0;  // (ZW = 4: a three-cell tile leaves a warp without cells)
         const P PX = splat(px[0]), PZ = splat(pz[0]), NAPZ = splat(-apz[0]);
         P PY[2], WV[2];
 #pragma unroll
@@ -749,8 +825,8 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         }
         const int sdir = sgc ? -1 : 1;
         const long rstep = sdir * (long)KC, ostep = sdir * (long)Q;
-        const int zw0 = sgc ? z0 + zn + 2 : z0 - 3;  // the cell of march row 0
-        const T* rp = Fs + (sgc ? (size_t)(zn + 5) * KC : 0) + tbase;  // march row r: rp + r rstep
+        const int zw0 = sgc ? z0 + zb + zc + 2 : z0 + zb - 3;  // the cell of march row 0
+        const T* rp = Fs + (size_t)(sgc ? zb + zc + 5 : zb) * KC + tbase;  // march row r: rp + r rstep
         const T* dcol = Dg + k0 + tbase;
         auto inc_row = [&](int s) -> Quad {  // the increments of cell s (zero for a ghost row)
             Quad q;
@@ -771,18 +847,10 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
 #pragma unroll
                 for (int p = 0; p < 2; ++p) r[d].p[p] = kD ? add2(r[d].p[p], q.p[p]) : r[d].p[p];
             }
-            const P K = splat(T(13.0 / 3.0));
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                const P d0 = sub2(r[1].p[p], r[0].p[p]);
-                w[p].v3 = r[3].p[p];
-                w[p].d12 = sub2(r[2].p[p], r[1].p[p]);
-                w[p].d23 = sub2(r[3].p[p], r[2].p[p]);
-                w[p].a1 = sub2(w[p].d12, d0);
-                w[p].a2 = sub2(w[p].d23, w[p].d12);
-                w[p].k1 = mul2(mul2(K, w[p].a1), w[p].a1);
-                w[p].k2 = mul2(mul2(K, w[p].a2), w[p].a2);
-                CM[p] = carried_corr<T>(w[p], r[4].p[p]);
+                w[p] = carried_start(r[0].p[p], r[1].p[p], r[2].p[p], r[3].p[p]);
+                CM[p] = carried_corr(w[p], r[4].p[p]);
             }
         }
         // the next row: its shared-memory part is read and its increments are added a step ahead
@@ -795,7 +863,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         }
         sn += sdir;
         Quad DN = inc_row(sn);
-        const size_t orow0 = (size_t)(sgc ? z0 + zn - 1 : z0) * Q + k0 + tbase;
+        const size_t orow0 = (size_t)(sgc ? z0 + zb + zc - 1 : z0 + zb) * Q + k0 + tbase;
         T* outp = Fout + orow0;
         const T* dop = kD ? Dg + orow0 : nullptr;
         unsigned short* lop = kLo && STAGE == 3 ? I.L0 + orow0 : nullptr;
@@ -807,15 +875,15 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         if (kLo && STAGE == 3 && in) LQN = __ldcg(reinterpret_cast<const uint2*>(lop));
         const int gy = jj[0], gx = Qy + kDup * ii[0], gz = Qy + kDup * (Qx + zz[0] - zm_lo);
 #pragma unroll(kUnroll)
-        for (int c = 0; c < zn; ++c) {
-            const int cc = sgc ? zn - 1 - c : c;
+        for (int c = 0; c < zc; ++c) {
+            const int cc = zb + (sgc ? zc - 1 - c : c);
             const T* gc = gsm + (size_t)cc * G;
             const T* sc = scs + cc * (S_COUNT * kDup);
             const uint2 LQ = LQN;
             const Quad DI = DIN;
             const Quad own = quad(Fs + (size_t)(cc + 3) * KC + tbase);  // d of the cell
             Quad nx = NV;                                               // the row two ahead
-            if (c + 1 < zn) {
+            if (c + 1 < zc) {
                 NV = quad(rp + (c + 6) * rstep);
 #pragma unroll
                 for (int p = 0; p < 2; ++p) NV.p[p] = kD ? add2(NV.p[p], DN.p[p]) : NV.p[p];
@@ -870,7 +938,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
                     }
                     // Eq. (flux) and the relaxation, both scaled by the stage's share of dt
                     const P d12 = w[p].d12;  // this cell minus the upwind one
-                    const P cp = carried_corr<T>(w[p], nx.p[p]);
+                    const P cp = carried_corr(w[p], nx.p[p]);
                     const P div = add2(d12, sub2(cp, CM[p]));
                     CM[p] = cp;
                     P inc = fma2(dep, NIT, mul2(S1, div));
@@ -908,7 +976,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
             const A x = X.x, z = Z.x, xz2 = XZ2.x;
             const A a0 = A0.x + A0.y, a1 = A1.x + A1.y, a2 = A2.x + A2.y, a3 = A3.x + A3.y;
             const A m1 = a0 * x, m3 = a0 * z, e = xz2 * a0 + a2;  // e: |xi|^2
-            A* rd = red + ((size_t)cc * (kThreads / 32) + warp) * 16;
+            A* rd = red + ((size_t)cc * (kThreads / 32 / ZW) + (ZW == 1 ? warp : 0)) * 16;
             if constexpr (sizeof(T) == 4) {
                 const float4 q[4] = {make_float4(a0, m1, a1, m3), make_float4(m1 * x, a2, m3 * z, a1 * x),
                                      make_float4(m3 * x, a1 * z, e * x, xz2 * a1 + a3),
@@ -1113,17 +1181,17 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     // (p_z > 0) from z0, down (p_z < 0) from z0+zn-1.  At march step c the register
     // window holds the cells s-3 .. s+2 seen from upwind (s+3 .. s-2 going down), so
     // both directions use one stencil: the flux through the interface ahead is
-    // |p_z| weno5(w1 .. w5), the one behind was formed at the previous step, and the
+    // |p_z| (w3 + its correction), the one behind was formed at the previous step, and the
     // divergence of Eq. (flux) is (ahead - behind) / dz for the signed p_z either way.
     const long rstep = sgc ? -(long)KC : (long)KC;
-    const T* rp = Fs + (sgc ? (size_t)(zn + 5) * KC : 0);  // window row d at step c: rp + (c + d) rstep
+    const T* rp = Fs + (size_t)(sgc ? zb + zc + 5 : zb) * KC;  // window row d at step c: rp + (c + d) rstep
     // stages 2, 3: the increment of the cell of each window row, read from global memory
     // (this launch does not write it).  Window row cd at step c
     // holds cell zw0 + (c + cd) sdir; a ghost row (a cell outside 0 .. Nz-1) takes zero,
     // its shared-memory value being the whole stage input.  Thread-based pointers: the
     // thread's velocity v sits at + voff(v).
     const int sdir = sgc ? -1 : 1;
-    const int zw0 = sgc ? z0 + zn + 2 : z0 - 3;
+    const int zw0 = sgc ? z0 + zb + zc + 2 : z0 + zb - 3;
     const T* dq = Dg + k0 + tbase;
     auto inc_row = [&](int s, T(&out)[V]) {
         const bool in = kD && (unsigned)s < (unsigned)Nz;
@@ -1131,21 +1199,47 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
 #pragma unroll
         for (int v = 0; v < V; ++v) out[v] = in && ok[v] ? __ldca(p + voff(v)) : T(0);
     };
-    // cm: the WENO correction of the interface behind (its flux is |p_z| (w2 + cm))
-    T w[V][6], cm[V], dn[V];
+    // WENO differences carried from interface to interface (carried_corr), two velocities per
+    // packed instruction where the storage is FP32 and V even.  Window rows 0 .. 4 (the cell's
+    // three upwind neighbours, the cell, the next one) start them and give the correction
+    // behind the first cell (its flux is |p_z| (w2 + cm)); nv is the row two ahead.
+    constexpr bool kPack = sizeof(T) == 4 && V % 2 == 0;
+    constexpr int NP = kPack ? V / 2 : V;
+    typedef typename PackedAs<T, kPack>::type P;
+    auto pack = [](const T(&a)[V], int p) -> P {
+        if constexpr (kPack) return make_float2(a[2 * p], a[2 * p + 1]);
+        else return a[p];
+    };
+    auto lane_of = [](const P(&a)[NP], int v) -> T {
+        if constexpr (kPack) return v & 1 ? a[v >> 1].y : a[v >> 1].x;
+        else return a[v];
+    };
+    Carried<P> w[NP];
+    P cm[NP], nv[NP];
+    T dn[V];
+    {
+        P r[6][NP];
 #pragma unroll
-    for (int d = 0; d < 6; ++d) {
-        inc_row(zw0 + d * sdir, dn);
+        for (int d = 0; d < 6; ++d) {
+            inc_row(zw0 + d * sdir, dn);
+            T x[V];
 #pragma unroll
-        for (int v = 0; v < V; ++v) w[v][d] = rp[d * rstep + kl[v]] + dn[v];
+            for (int v = 0; v < V; ++v) x[v] = kD ? rp[d * rstep + kl[v]] + dn[v] : rp[d * rstep + kl[v]];
+#pragma unroll
+            for (int p = 0; p < NP; ++p) r[d][p] = pack(x, p);
+        }
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            w[p] = carried_start(r[0][p], r[1][p], r[2][p], r[3][p]);
+            cm[p] = carried_corr(w[p], r[4][p]);
+            nv[p] = r[5][p];
+        }
     }
-#pragma unroll
-    for (int v = 0; v < V; ++v) cm[v] = weno5_corr<T>(w[v][0], w[v][1], w[v][2], w[v][3], w[v][4]);
     int sn = zw0 + 6 * sdir;  // the cell of the row the next step loads
     inc_row(sn, dn);
     const T dt = T(I.dt);
     const long ostep = sgc ? -(long)Q : (long)Q;
-    const size_t orow0 = (size_t)(sgc ? z0 + zn - 1 : z0) * Q + k0 + tbase;  // the first cell, thread's column
+    const size_t orow0 = (size_t)(sgc ? z0 + zb + zc - 1 : z0 + zb) * Q + k0 + tbase;  // the first cell, thread's column
     T* outp = Fout + orow0;
     const T* dop = kD ? Dg + orow0 : nullptr;  // the increment of the cell
     unsigned short* lop = kLo && STAGE == 3 ? I.L0 + orow0 : nullptr;
@@ -1156,27 +1250,26 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     T din[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        lqn[v] = kLo && STAGE == 3 && ok[v] ? __ldcg(lop + voff(v)) : 0;
-        din[v] = kD && ok[v] ? __ldca(dop + voff(v)) : T(0);
+        lqn[v] = kLo && STAGE == 3 && ok[v] && zc > 0 ? __ldcg(lop + voff(v)) : 0;
+        din[v] = kD && ok[v] && zc > 0 ? __ldca(dop + voff(v)) : T(0);  // zc = 0: a warp without cells
     }
-    constexpr bool kPack = sizeof(T) == 4 && V % 2 == 0;  // moments of two velocities per packed op
 #pragma unroll 1  // unrolling the z-march only adds instruction-cache misses
-    for (int c = 0; c < zn; ++c) {
+    for (int c = 0; c < zc; ++c) {
         unsigned short lqc[V];
         T dc[V], dic[V];  // increments of the window row this step loads and of the cell
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             lqc[v] = lqn[v];
-            if (kLo && STAGE == 3 && ok[v] && c + 1 < zn) lqn[v] = __ldcg(lop + ostep + voff(v));
+            if (kLo && STAGE == 3 && ok[v] && c + 1 < zc) lqn[v] = __ldcg(lop + ostep + voff(v));
             dic[v] = din[v];
-            if (kD && ok[v] && c + 1 < zn) din[v] = __ldca(dop + ostep + voff(v));
+            if (kD && ok[v] && c + 1 < zc) din[v] = __ldca(dop + ostep + voff(v));
             dc[v] = dn[v];
         }
-        if (kD && c + 1 < zn) {
+        if (kD && c + 1 < zc) {
             sn += sdir;
             inc_row(sn, dn);
         }
-        const int cc = sgc ? zn - 1 - c : c;  // the cell within the tile
+        const int cc = zb + (sgc ? zc - 1 - c : c);  // the cell within the tile
         const T* sc = recs + (size_t)cc * rstride;
         const T* gc = gsm + cc * G;
         const T* rn = rp + (c + 6) * rstep;
@@ -1187,37 +1280,30 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
             qx = sc[R_QX]; qy = sc[R_QY]; qz = sc[R_QZ];
             itau = sc[R_ITAU]; cS = sc[R_CS]; i5T = sc[R_I5T]; idz = idzs[cc];
         }
-        // WENO corrections of the interfaces ahead, two velocities per packed FP32
-        // instruction where the storage is FP32
-        T cpv[V];
-        if (STAGE > 0) {
-            if constexpr (kPack) {
+        // the corrections of the interfaces ahead, the cell minus the upwind one, and the next row
+        P cp2[NP], d12[NP];
 #pragma unroll
-                for (int p2 = 0; p2 < V / 2; ++p2) {
-                    const float2 r = weno5_corr2(make_float2(w[2 * p2][1], w[2 * p2 + 1][1]),
-                                                 make_float2(w[2 * p2][2], w[2 * p2 + 1][2]),
-                                                 make_float2(w[2 * p2][3], w[2 * p2 + 1][3]),
-                                                 make_float2(w[2 * p2][4], w[2 * p2 + 1][4]),
-                                                 make_float2(w[2 * p2][5], w[2 * p2 + 1][5]));
-                    cpv[2 * p2] = r.x;
-                    cpv[2 * p2 + 1] = r.y;
-                }
-            } else {
+        for (int p = 0; p < NP; ++p) {
+            d12[p] = w[p].d12;
+            cp2[p] = STAGE > 0 ? carried_corr(w[p], nv[p]) : cm[p];
+        }
+        {
+            T x[V];
 #pragma unroll
-                for (int v = 0; v < V; ++v) cpv[v] = weno5_corr<T>(w[v][1], w[v][2], w[v][3], w[v][4], w[v][5]);
-            }
+            for (int v = 0; v < V; ++v) x[v] = kD ? rn[kl[v]] + dc[v] : rn[kl[v]];
+#pragma unroll
+            for (int p = 0; p < NP; ++p) nv[p] = pack(x, p);
         }
         // ---- per velocity: the update, its store, and the moment variables
         A ov[V], mx[V], my[V], mz[V], m2[V];  // value; the monomials' factors (p or p - u_r); |.|^2
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             const unsigned short lq = lqc[v];
-            const T wn = rn[kl[v]] + dc[v];
-            T out = w[v][3];  // the value whose moments are taken
+            const T h = own[kl[v]];
+            T out = h;  // the value whose moments are taken
             T ex = 0, ey = 0, ez = 0, xi2 = 0;  // xi = p - u of the cell's record
             if (STAGE > 0) {
-                const T cp = cpv[v];
-                const T f = w[v][3];
+                const T cp = lane_of(cp2, v);
                 // Shakhov target n Gx Gy Gz (1 + S), S = cS (xi^2/(5T) - 1) xi.q; in the
                 // phi / chi model (Eq. sred_def) S = cS ((xi_x^2 + xi_z^2)/(5T) - 4/5 or 2/5) xi.q
                 // with u_y = q_y = 0, and Gy = 1 (phi) or T (chi) from the record
@@ -1240,23 +1326,20 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
                 // (stage 3, FP32) residual separately, (d - tgt) + increment + residual,
                 // so that its rounding is relative to the departure, which in the
                 // collision-dominated regime is much smaller than f itself
-                T h = f, dinc = T(0), lo = T(0);
-                if (STAGE >= 2) {
-                    h = own[kl[v]];
-                    dinc = dic[v];
-                }
+                const T dinc = STAGE >= 2 ? dic[v] : T(0);
+                T lo = T(0);
                 if constexpr (kLo && STAGE == 3) lo = lo_decode(lq, h);
-                const T dep = STAGE >= 2 ? ((h - tgt) + dinc) + lo : f - tgt;
+                const T dep = STAGE >= 2 ? ((h - tgt) + dinc) + lo : h - tgt;
                 // Eq. (flux): (|p_z| (w3 + cp) - |p_z| (w2 + cm)) / dz, formed from the
                 // difference of the two upwind cells and of the two corrections, so that
                 // its rounding is relative to the divergence rather than to d.  The
                 // advection and relaxation increments nearly cancel near a steady state:
                 // combine them first.
-                const T Lv = -apz[v] * ((w[v][3] - w[v][2]) + (cp - cm[v])) * idz - dep * itau;
+                const T Lv = -apz[v] * (lane_of(d12, v) + (cp - lane_of(cm, v))) * idz - dep * itau;
                 T st;  // the value stored
                 if (STAGE == 1) {
                     st = dt * Lv;
-                    out = f + st;
+                    out = h + st;
                 } else if (STAGE == 2) {
                     st = T(0.25) * (dinc + dt * Lv);
                     out = h + st;
@@ -1276,11 +1359,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
                     out = st;
                 }
                 if (ok[v]) __stcg(outp + voff(v), st);
-                cm[v] = cp;
             }
-#pragma unroll
-            for (int d = 0; d < 5; ++d) w[v][d] = w[v][d + 1];
-            w[v][5] = wn;
             // the moments: of psi(p - u_r) about the velocity u_r of the cell's record
             // (stage 0, which has no record: of psi(p)), so that the third moments are
             // close to the heat flux itself instead of its sum with terms of size u |p|^2
@@ -1295,6 +1374,8 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
                 mx[v] = A(px[v]); my[v] = yv[v]; mz[v] = A(pz[v]); m2[v] = p2v[v];
             }
         }
+#pragma unroll
+        for (int p = 0; p < NP; ++p) cm[p] = cp2[p];
         // ---- the 13 weighted monomials summed over the thread's velocities: w f times
         // 1, p_a, p_a p_b, |p|^2 p_a (RED: chi carries the p_y^2 parts: sum chi, sum chi p_x,
         // sum chi p_z)
@@ -1349,7 +1430,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         }
         const A tot = reduce_scatter16<A>(acc, lane);
         const int m = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-        if ((lane & 1) == 0) red[((size_t)cc * (kThreads / 32) + warp) * 16 + m] = tot;
+        if ((lane & 1) == 0) red[((size_t)cc * (kThreads / 32 / ZW) + (ZW == 1 ? warp : 0)) * 16 + m] = tot;
         outp += ostep;
         if (kD) dop += ostep;
         if (kLo && STAGE == 3) lop += ostep;
@@ -1362,47 +1443,58 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
     // the chunks exactly enough in double-float)
     for (int e = tid; e < zn * kNMom; e += kThreads) {
         const int c = e / kNMom, a = e - c * kNMom;
-        A s = red[(size_t)c * (kThreads / 32) * 16 + a];
+        constexpr int nw = kThreads / 32 / ZW;  // warps that share a cell
+        A s = red[(size_t)c * nw * 16 + a];
 #pragma unroll
-        for (int q = 1; q < kThreads / 32; ++q) s += red[((size_t)c * (kThreads / 32) + q) * 16 + a];
+        for (int q = 1; q < nw; ++q) s += red[((size_t)c * nw + q) * 16 + a];
         static_cast<A*>(I.partial)[((size_t)tile.chunk * kNMom + a) * Nz + z0 + c] = s;
     }
 
     // ---- 6. outgoing WENO flux of the stage output through the wall interfaces (for
     // n_w), as a sum over the deviations (the rest state's flux is added by the
-    // finalisation).  Each thread re-reads the outputs it wrote itself: the new d after
+    // finalisation).  The outputs are read back (ZW = 4: other warps wrote some): the new d after
     // stage 3, d + the increment after stages 1 and 2 (STAGE 0: its input rows).
     auto outval = [&](int v, int cell) -> T {
         const T* row = Fs + (size_t)(cell + rbase) * KC;
         if (STAGE == 0) return row[kl[v]];
-        const T o = Fout[(size_t)cell * Q + k0 + kl[v]];
+        const T o = __ldcg(Fout + (size_t)cell * Q + k0 + kl[v]);
         return STAGE == 3 ? o : row[kl[v]] + o;
     };
-    if (z0 == 0) {  // bottom: p_z < 0 leaves through s = -1/2
-        double fl = 0.0;
+    // The sums: exact products (double-float with FP32 storage: no FP64 instruction, which here
+    // held the wall tiles' schedulers for some 2000 cycles; 64 x C2 339 -> 311 us per step), a
+    // warp's and the CTA's sum in the same arithmetic, one FP64 value per chunk.
+    R fl[2] = {Real<T>::of(T(0)), Real<T>::of(T(0))};  // bottom, top
+    if (z0 == 0 && sgc && !I.half && zw == 0) {  // p_z < 0 leaves through s = -1/2; no wall below a half channel
 #pragma unroll
         for (int v = 0; v < V; ++v)
-            if (ok[v] && sgc && !I.half) {  // no wall below a half channel
+            if (ok[v]) {
                 const T f1 = outval(v, 0), f2 = outval(v, 1), f3 = outval(v, 2);
-                const T g0 = T(I.ext_bot[0][0]) * f1 + T(I.ext_bot[0][1]) * f2 + T(I.ext_bot[0][2]) * f3;
-                const T g1 = T(I.ext_bot[1][0]) * g0 + T(I.ext_bot[1][1]) * f1 + T(I.ext_bot[1][2]) * f2;
-                fl += double(wm[v]) * double(pz[v] * weno5<T>(f3, f2, f1, g0, g1));
+                const T g0 = ext_bot[0][0] * f1 + ext_bot[0][1] * f2 + ext_bot[0][2] * f3;
+                const T g1 = ext_bot[1][0] * g0 + ext_bot[1][1] * f1 + ext_bot[1][2] * f2;
+                fl[0] = r_add(fl[0], r_mul(Real<T>::of(T(wm[v])), Real<T>::of(pz[v] * weno5<T>(f3, f2, f1, g0, g1))));
             }
-        fl = block_sum(fl, wall_red);
-        if (tid == 0) I.flux_part[tile.chunk * 2 + 0] = fl;
     }
-    if (z0 + zn == Nz) {  // top: p_z > 0 leaves through s = Nz - 1/2
-        double fl = 0.0;
+    if (z0 + zn == Nz && !sgc && zw == 0) {  // top: p_z > 0 leaves through s = Nz - 1/2
 #pragma unroll
         for (int v = 0; v < V; ++v)
-            if (ok[v] && !sgc) {
+            if (ok[v]) {
                 const T f1 = outval(v, Nz - 1), f2 = outval(v, Nz - 2), f3 = outval(v, Nz - 3);
-                const T g0 = T(I.ext_top[0][0]) * f1 + T(I.ext_top[0][1]) * f2 + T(I.ext_top[0][2]) * f3;
-                const T g1 = T(I.ext_top[1][0]) * g0 + T(I.ext_top[1][1]) * f1 + T(I.ext_top[1][2]) * f2;
-                fl += double(wm[v]) * double(pz[v] * weno5<T>(f3, f2, f1, g0, g1));
+                const T g0 = ext_top[0][0] * f1 + ext_top[0][1] * f2 + ext_top[0][2] * f3;
+                const T g1 = ext_top[1][0] * g0 + ext_top[1][1] * f1 + ext_top[1][2] * f2;
+                fl[1] = r_add(fl[1], r_mul(Real<T>::of(T(wm[v])), Real<T>::of(pz[v] * weno5<T>(f3, f2, f1, g0, g1))));
             }
-        fl = block_sum(fl, wall_red);
-        if (tid == 0) I.flux_part[tile.chunk * 2 + 1] = fl;
+    }
+    if (z0 == 0 || z0 + zn == Nz) {
+        R* fr = reinterpret_cast<R*>(wall_red);
+        const int side = z0 == 0 && (sgc || z0 + zn != Nz) ? 0 : 1;  // the one this chunk can leave through
+        const R s = warp_sum(side ? fl[1] : fl[0]);
+        if (lane == 0) fr[warp] = s;
+        __syncthreads();
+        if (tid == 0) {
+            const double f = r_double(r_add(r_add(fr[0], fr[1]), r_add(fr[2], fr[3])));
+            if (z0 == 0) I.flux_part[tile.chunk * 2 + 0] = side == 0 ? f : 0.0;
+            if (z0 + zn == Nz) I.flux_part[tile.chunk * 2 + 1] = side == 1 ? f : 0.0;
+        }
     }
 
     // ---- 7. (fuse != 0) finalisation without extra launches (threadfence tickets): the CTA
@@ -1430,11 +1522,11 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
 }
 
 // ---- host-side launch of one stage-kernel instantiation ----------------------
-template <typename T, int V, int STAGE, bool RED, bool GRP>
+template <typename T, int V, int STAGE, bool RED, bool GRP, int ZW>
 static cudaError_t launch_stage_t(const InstDev* d_inst, const Tile* d_tiles, int ntiles, size_t smem,
                                   int fuse, cudaStream_t st)
 {
-    auto kfn = stage_kernel<T, V, STAGE, RED, GRP>;
+    auto kfn = stage_kernel<T, V, STAGE, RED, GRP, ZW>;
     if (smem > 40 * 1024) {  // with the static arrays above the default limit of 48 KB
         cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1452,24 +1544,30 @@ static cudaError_t launch_stage_t(const InstDev* d_inst, const Tile* d_tiles, in
     return cudaLaunchKernelEx(&cfg, kfn, d_inst, d_tiles, fuse);
 }
 
-template <typename T, int V, bool RED, bool GRP = false>
+template <typename T, int V, bool RED, bool GRP = false, int ZW = 1>
 static cudaError_t launch_stage_r(int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
                                   cudaStream_t st)
 {
     switch (stage) {
-        case 0: return launch_stage_t<T, V, 0, RED, GRP>(d, t, n, smem, fuse, st);
-        case 1: return launch_stage_t<T, V, 1, RED, GRP>(d, t, n, smem, fuse, st);
-        case 2: return launch_stage_t<T, V, 2, RED, GRP>(d, t, n, smem, fuse, st);
-        default: return launch_stage_t<T, V, 3, RED, GRP>(d, t, n, smem, fuse, st);
+        case 0: return launch_stage_t<T, V, 0, RED, GRP, ZW>(d, t, n, smem, fuse, st);
+        case 1: return launch_stage_t<T, V, 1, RED, GRP, ZW>(d, t, n, smem, fuse, st);
+        case 2: return launch_stage_t<T, V, 2, RED, GRP, ZW>(d, t, n, smem, fuse, st);
+        default: return launch_stage_t<T, V, 3, RED, GRP, ZW>(d, t, n, smem, fuse, st);
     }
 }
 
 template <typename T, bool RED>
-static cudaError_t launch_stage_m(int V, int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
+static cudaError_t launch_stage_m(int V /* a layout: stage_layout in api.cu */, int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
                                   cudaStream_t st)
 {
-    if constexpr (!RED)
-        if (V == kGroupedV) return launch_stage_r<T, 4, false, true>(stage, d, t, n, smem, fuse, st);
+    if constexpr (!RED) {
+        if (V == (4 | kGrouped)) return launch_stage_r<T, 4, false, true>(stage, d, t, n, smem, fuse, st);
+        if constexpr (sizeof(T) == 8)
+            if (V == (4 | kGrouped | kZSplit))
+                return launch_stage_r<T, 4, false, true, 4>(stage, d, t, n, smem, fuse, st);
+    }
+    if constexpr (sizeof(T) == 8)
+        if (V == (1 | kZSplit)) return launch_stage_r<T, 1, RED, false, 4>(stage, d, t, n, smem, fuse, st);
     if (V == 1) return launch_stage_r<T, 1, RED>(stage, d, t, n, smem, fuse, st);
     if (V == 2) return launch_stage_r<T, 2, RED>(stage, d, t, n, smem, fuse, st);
     return launch_stage_r<T, 4, RED>(stage, d, t, n, smem, fuse, st);

@@ -24,7 +24,10 @@ constexpr int kNMom = 13;       // raw moments accumulated per cell
 constexpr int kRecHead = 12;    // scalars at the head of a cell record
 constexpr int kThreads = 128;   // threads of a stage CTA
 constexpr int kMaxZT = 64;      // cells of a z-tile
-constexpr int kGroupedV = 64;   // the launchers' V for the grouped layout of V = 4
+// flags of the launchers' layout next to its velocities per thread (1, 2, 4)
+constexpr int kGrouped = 8;     // four adjacent velocities of one x and z node per thread
+constexpr int kZSplit = 16;     // the CTA's warps split the tile's cells
+inline int layout_columns(int layout) { return (layout & 7) * (layout & kZSplit ? kThreads / 4 : kThreads); }
 
 enum { QUAD_FULL = 0, QUAD_HALF = 1 };
 
@@ -39,6 +42,18 @@ enum { R_N = 0, R_UX, R_UY, R_UZ, R_T, R_QX, R_QY, R_QZ, R_ITAU, R_CS, R_I5T, R_
 constexpr int R_DX = kRecHead;
 // record length of an instance, rounded up to 16 bytes in either storage type
 inline int rec_stride_of(int Qx, int Qy, int Qz) { return (kRecHead + Qx + Qy + 2 * Qz + 3) & ~3; }
+
+// Weights of the ghost values' extrapolation: ghost Nz+1 <- (Nz, Nz-1, Nz-2), Nz+2 <-
+// (Nz+1, Nz, Nz-1) above, ghost 0 <- (1, 2, 3), -1 <- (0, 1, 2) below
+template <typename T>
+struct Walls {
+    T top[2][3], bot[2][3];
+};
+// n_w - 1 and n_w of the bottom wall, then of the top one, in FP64 and rounded to FP32
+struct WallDensity {
+    double d[4];
+    float f[4];
+};
 
 // Everything a kernel needs to know about one instance (lives in device memory).
 struct InstDev {
@@ -60,8 +75,9 @@ struct InstDev {
     double frest_bot, frest_top;  // outgoing wall flux of the rest state (sum w p_z over the
                                   // velocities leaving through each wall)
     unsigned wait_limit;          // spins of the bounded wait for the bulk copies
-    double ext_top[2][3];         // ghost Nz+1 <- (Nz, Nz-1, Nz-2); Nz+2 <- (Nz+1, Nz, Nz-1)
-    double ext_bot[2][3];         // ghost 0 <- (1, 2, 3); ghost -1 <- (0, 1, 2)
+    Walls<double> walls;
+    Walls<float> walls2;          // the same rounded to FP32
+    unsigned mQy, mQxQy;          // ceil(2^32 / d) for div_small, 0 for d = 1
     // tables
     const double *Hx, *Hy, *Pz;   // FP64, [Q_a][N_a + 1] basis values He_l/l!, pi_l/h_l
     const float2 *Hx2, *Hy2, *Pz2;  // the same as FP32 (hi, lo) pairs, hi + lo = the FP64 value
@@ -87,7 +103,7 @@ struct InstDev {
     void *rec;                    // [Nz][rec_stride]
     void *partial;                // [nchunks][kNMom][Nz] in the accumulation type (FP32 sums of FP32 storage)
     double *flux_part;            // [nchunks][2]: bottom, top outgoing flux
-    double *nw;                   // [2]: bottom, top wall density
+    WallDensity *nw;              // [1]
     double *prof;                 // [14][Nz]
     double *Wold, *Wnew;          // [3][Nz]: n, u_x, T
     double *res;                  // [1]

@@ -114,3 +114,43 @@ def test_network_tiles_at_ragged_sizes(sizes, B):
     for k in g_ora:
         assert np.all(np.abs(gg[k] - g_ora[k]) <= E[k] + floor * np.abs(g_ora[k]).max()), k
     net.close()
+
+
+@pytest.mark.parametrize("Qx,Qy,Qz,Nz", [(8, 8, 8, 81), (7, 7, 11, 73), (9, 0, 31, 70), (2, 0, 4, 64), (4, 4, 4, 23)])
+@pytest.mark.parametrize("ZT", [3, 5, 16])
+@pytest.mark.parametrize("half", [0, 1])
+def test_fp64_one_velocity_layouts_agree(Qx, Qy, Qz, Nz, ZT, half):
+    """V = 1 in FP64 (warps that split a tile's cells, in the grouped form or, for the small
+    batches, with one velocity per thread; tiles of 3 and 5 cells leave them unevenly filled)
+    against V = 2, which marches whole tiles: 1e-12 of the largest population after 6 steps."""
+    P = _lbs()
+    from paper_1702_01335_gb300 import Instance, Solver
+    inst = Instance(Qx=Qx, Qy=Qy, Qz=Qz, N_eq=3, Nz=Nz, A=0.7, half=half, Kn=0.4, u_w=0.5, Pr=2.0 / 3.0, cfl=0.4)
+    a, b = Solver(inst), Solver(inst)
+    a.set_tiling(1, ZT, 0)
+    b.set_tiling(2, 7, 0)
+    z = np.linspace(-1.0, 1.0, Nz)[:, None]
+    d = 0.1 * np.sin(2 * z) + 0.02 * np.random.default_rng(3).standard_normal((1, inst.Q)) * (1 - 0.2 * z)
+    for s in (a, b):
+        s.set_state(0, d)
+        s.step(6)
+    assert rel_err(a.populations(), b.populations()) < 1e-12
+    pa, pb = a.profiles(), b.profiles()
+    assert max(np.abs(pa[k] - pb[k]).max() for k in pa) < 1e-11
+
+
+def test_default_tiling_follows_the_batch():
+    """The tiling a solver starts with: V = 1 for one small channel and for mostly empty
+    512-velocity chunks, V = 4 for several channels of full ones, V = 1 for an odd half range."""
+    P = _lbs()
+    def tiling(p, n, prec):
+        s = solver_of([p] * n, 0.0, prec)
+        t = s.tiling()
+        s.close()
+        return t["V"], t["fuse"]
+    assert tiling(W.C2, 1, P.LBS_FP32) == (1, 0)
+    assert tiling(W.C2, 8, P.LBS_FP32) == (4, 0)
+    assert tiling(dict(W.C1, Nz=128), 64, P.LBS_FP32) == (1, 0)
+    assert tiling(dict(W.C2, Qx=9, Qy=9, Qz=9), 64, P.LBS_FP32) == (1, 0)
+    assert tiling(W.C2, 1, P.LBS_FP64) == (1, 0)
+    assert tiling(W.C2, 16, P.LBS_FP64) == (4, 0)
