@@ -146,7 +146,7 @@ lbs_status lbs_step(lbs_handle h, long nsteps);
  * Each instance stops (retires) in the step where its R first drops below tol;
  * steps_out[n] (may be NULL) receives the steps each instance took.  R is
  * checked on the device every step; the host polls every check_every steps
- * (CUDA-graph launches of check_every steps).  Returns LBS_ERR_NO_CONVERGENCE
+ * (CUDA-graph launches of check_every steps or a divisor of it).  Returns LBS_ERR_NO_CONVERGENCE
  * if some instance did not converge. */
 lbs_status lbs_run_to_steady(lbs_handle h, double tol, long max_steps, int check_every,
                              long* steps_out);

@@ -27,6 +27,8 @@ cudaError_t launch_seed(int fp32, const InstDev* d_inst, int inst, int Nz, const
 cudaError_t launch_seed_free_molecular(int fp32, const InstDev* d_inst, int inst, int Nz, cudaStream_t st);
 cudaError_t launch_gather_moments(const InstDev* d_inst, int ninst, const double* prof_all, double* out,
                                   cudaStream_t st);
+cudaError_t launch_gather_states(const InstDev* d_inst, int b0, int n, void* dst, size_t d_total, int esize,
+                                 cudaStream_t st);
 size_t stage_smem_bytes(int fp32, int V, int zn, int Qx, int Qy, int nzm, int rstride);
 }  // namespace lbs
 
@@ -98,6 +100,8 @@ struct lbs_solver {
     double* mom_all = nullptr;  // [8][Nz] per instance: lbs_moments' rows, gathered for one copy
     int* status_all = nullptr;
     int* cur_all = nullptr;  // per instance: which of F0 / F1 holds the state
+    int* active_all = nullptr;         // per instance: the active flag, the step counter
+    long long* steps_all = nullptr;
     cudaGraphExec_t gexec = nullptr;
     int gsteps = 0;
     // split stepping (fuse = 2): instances [0, nA) on stream, [nA, ninst) on stream2
@@ -583,7 +587,7 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         o.flux = pool.take(maxch * 2 * 8);
         o.nw = pool.take(sizeof(WallDensity));  // prof: below
         o.Wold = pool.take(3 * (size_t)Nz * 8); o.Wnew = pool.take(3 * (size_t)Nz * 8);
-        o.res = pool.take(8); o.steps = pool.take(8); o.active = pool.take(4);  // status: below
+        o.res = pool.take(8);  // steps, active, status: below
         o.zcount = pool.take(4 * (size_t)std::max(1, Nz / 3)); o.icount = pool.take(4);
     }
     // The two state buffers F0 and F1 of every instance back to back (one region each),
@@ -592,7 +596,7 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
     // multiple of 256 bytes, such as C2's 1 MiB), a whole-batch lbs_get_state /
     // lbs_set_state is one copy per region.  Profiles, status words and the state
     // selectors are packed.
-    size_t prof_base = 0, status_base = 0, cur_base = 0;
+    size_t prof_base = 0, status_base = 0, cur_base = 0, active_base = 0, steps_base = 0;
     {
         size_t f0_total = 0, l0_total = 0, prof_total = 0;
         for (int b = 0; b < h->ninst; ++b) {
@@ -606,8 +610,10 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         prof_base = pool.take(prof_total * 8);
         status_base = pool.take(4 * (size_t)h->ninst);
         cur_base = pool.take(4 * (size_t)h->ninst);
+        active_base = pool.take(4 * (size_t)h->ninst);
+        steps_base = pool.take(8 * (size_t)h->ninst);
         h->prof_all_n = prof_total;
-        size_t fo = 0, lo = 0, po = 0;
+        size_t fo = 0, lo = 0, po = 0, values = 0;
         for (int b = 0; b < h->ninst; ++b) {
             const size_t nf = (size_t)h->ih[b].Nz * h->ih[b].Q;
             off[b].F0 = f0_base + fo;
@@ -619,6 +625,10 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
             po += 14 * (size_t)h->ih[b].Nz;
             off[b].status = status_base + 4 * (size_t)b;
             off[b].cur = cur_base + 4 * (size_t)b;
+            off[b].active = active_base + 4 * (size_t)b;
+            off[b].steps = steps_base + 8 * (size_t)b;
+            h->idev[b].state_at = (long)values;
+            values += nf;
         }
     }
     const size_t inst_off = pool.take(sizeof(InstDev) * h->ninst);
@@ -694,6 +704,8 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
     h->mom_all = reinterpret_cast<double*>(P + mom_off);
     h->status_all = reinterpret_cast<int*>(P + status_base);
     h->cur_all = reinterpret_cast<int*>(P + cur_base);
+    h->active_all = reinterpret_cast<int*>(P + active_base);
+    h->steps_all = reinterpret_cast<long long*>(P + steps_base);
     h->ntiles = (int)tiles.size();
     CK(cudaMemcpyAsync(P, img.data(), pool.bytes, cudaMemcpyHostToDevice, h->stream));
     CK(cudaStreamSynchronize(h->stream));
@@ -1053,18 +1065,24 @@ lbs_status lbs_run_to_steady(lbs_handle h, double tol, long max_steps, int check
     CK(cudaMemcpyAsync(h->d_inst, h->idev.data(), sizeof(InstDev) * h->ninst, cudaMemcpyHostToDevice, h->stream));
     std::vector<long long> st0(h->ninst), st(h->ninst);
     std::vector<int> act(h->ninst);
-    for (int b = 0; b < h->ninst; ++b)
-        CK(cudaMemcpyAsync(&st0[b], h->idev[b].steps, 8, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(st0.data(), h->steps_all, 8 * (size_t)h->ninst, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    lbs_status s = get_graph(h, check_every);
+    // The graph holds the largest divisor of check_every up to 16 and is launched as often as
+    // needed: it is captured and instantiated again for each shorter tile list, a cost per step
+    // in it (48 sweep instances to R < 1e-5 with checks every 50 steps: 105 -> 89 ms, together
+    // with one copy of all active flags per check instead of one each)
+    int gsteps = 1;
+    for (int g = 2; g <= 16; ++g)
+        if (check_every % g == 0) gsteps = g;
+    if (gsteps < 4) gsteps = check_every;  // no useful divisor
+    lbs_status s = get_graph(h, gsteps);
     long done = 0;
     bool all = false;
     while (s == LBS_OK && done < max_steps && !all) {
-        CK(cudaGraphLaunch(h->gexec, h->stream));
+        for (int g = 0; g < check_every; g += gsteps) CK(cudaGraphLaunch(h->gexec, h->stream));
         done += check_every;
         all = true;
-        for (int b = 0; b < h->ninst; ++b)
-            CK(cudaMemcpyAsync(&act[b], h->idev[b].active, 4, cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaMemcpyAsync(act.data(), h->active_all, 4 * (size_t)h->ninst, cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
         for (int b = 0; b < h->ninst; ++b) all &= act[b] == 0;
         // once a quarter of the launched tiles belong to retired instances, launch only
@@ -1085,18 +1103,16 @@ lbs_status lbs_run_to_steady(lbs_handle h, double tol, long max_steps, int check
             drop_graph(h);
             regraph = true;
         }
-        if (regraph && s == LBS_OK) s = get_graph(h, check_every);
+        if (regraph && s == LBS_OK) s = get_graph(h, gsteps);
     }
     // disarm and reactivate every instance, with every tile and the batch's own
     // finalisation layout
     choose_finalize(h);
     for (int b = 0; b < h->ninst; ++b) h->idev[b].tol = 0.0;
     CK(cudaMemcpyAsync(h->d_inst, h->idev.data(), sizeof(InstDev) * h->ninst, cudaMemcpyHostToDevice, h->stream));
-    const int one = 1;
-    for (int b = 0; b < h->ninst; ++b) {
-        CK(cudaMemcpyAsync(&st[b], h->idev[b].steps, 8, cudaMemcpyDeviceToHost, h->stream));
-        CK(cudaMemcpyAsync(h->idev[b].active, &one, 4, cudaMemcpyHostToDevice, h->stream));
-    }
+    const std::vector<int> ones(h->ninst, 1);
+    CK(cudaMemcpyAsync(st.data(), h->steps_all, 8 * (size_t)h->ninst, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(h->active_all, ones.data(), 4 * (size_t)h->ninst, cudaMemcpyHostToDevice, h->stream));
     const lbs_status su = upload_tiles(h, nullptr);
     if (s == LBS_OK) s = su;
     CK(cudaStreamSynchronize(h->stream));
@@ -1365,6 +1381,16 @@ lbs_status lbs_get_state(lbs_handle h, int inst, void* dst, int to_host)
     if (!h || inst < -1 || inst >= h->ninst) return fail(LBS_ERR_ARG, "invalid handle or instance index");
     if (!dst) return fail(LBS_ERR_ARG, "null destination");
     const int b0 = inst < 0 ? 0 : inst, b1 = inst < 0 ? h->ninst : inst + 1;
+    // Up to 48 MB to device memory: one launch that finds the buffers itself instead of a read
+    // of the selectors and a copy or two per instance (20 table runs 167 -> 14 us, one C1
+    // channel 22 -> 12, the 64-instance sweep, 50 MB, 68 -> 70; 256 x C2, 384 MB, 147 -> 242:
+    // larger states keep the copies, as does a destination at an odd address)
+    const size_t d_total = state_d_bytes(h, b0, b1);
+    if (!to_host && d_total <= (size_t(48) << 20) && reinterpret_cast<uintptr_t>(dst) % 2 == 0 && b1 - b0 <= 65535) {
+        CK(launch_gather_states(h->d_inst, b0, b1 - b0, dst, d_total, h->esize, h->stream));
+        CK(cudaStreamSynchronize(h->stream));
+        return LBS_OK;
+    }
     std::vector<int> cur(h->ninst);
     CK(cudaMemcpyAsync(cur.data(), h->cur_all, 4 * (size_t)h->ninst, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));

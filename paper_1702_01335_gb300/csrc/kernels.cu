@@ -110,7 +110,54 @@ __global__ void __launch_bounds__(128) gather_moment_rows(const InstDev* __restr
     for (int c = threadIdx.x; c < I.Nz; c += blockDim.x) dst[c] = src[c];
 }
 
+// bytes from src to dst by the whole grid row (blockIdx.x of gridDim.x): 16 at a time where
+// both allow, else 2 (every state is a whole number of 16-bit units)
+static __device__ __forceinline__ void copy_bytes(unsigned char* dst, const unsigned char* src, size_t n)
+{
+    const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    if (((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) == 0) {
+        const uint4* s = reinterpret_cast<const uint4*>(src);
+        uint4* d = reinterpret_cast<uint4*>(dst);
+        const size_t words = n / 16;
+        size_t e = t;
+        for (; e + 3 * step < words; e += 4 * step) {
+            const uint4 a = __ldcs(s + e), b = __ldcs(s + e + step), c = __ldcs(s + e + 2 * step),
+                        x = __ldcs(s + e + 3 * step);
+            __stcs(d + e, a);
+            __stcs(d + e + step, b);
+            __stcs(d + e + 2 * step, c);
+            __stcs(d + e + 3 * step, x);
+        }
+        for (; e < words; e += step) __stcs(d + e, __ldcs(s + e));
+        for (size_t q = words * 8 + t; q < n / 2; q += step)
+            reinterpret_cast<unsigned short*>(dst)[q] = reinterpret_cast<const unsigned short*>(src)[q];
+    } else {
+        for (size_t q = t; q < n / 2; q += step)
+            reinterpret_cast<unsigned short*>(dst)[q] = reinterpret_cast<const unsigned short*>(src)[q];
+    }
+}
+
+// The state of instances b0 .. b0 + gridDim.y - 1 to device memory in lbs_get_state's layout:
+// every d, then (FP32) every residual; each instance's buffer is found on the device.
+__global__ void __launch_bounds__(256) gather_states(const InstDev* __restrict__ insts, int b0, unsigned char* dst,
+                                                     size_t d_total, int esize)
+{
+    const InstDev& I = insts[b0 + blockIdx.y];
+    const size_t n = (size_t)I.Nz * I.Q, at = I.state_at - insts[b0].state_at;
+    copy_bytes(dst + at * esize, static_cast<const unsigned char*>(*I.cur ? I.F1 : I.F0), n * esize);
+    if (I.L0) copy_bytes(dst + d_total + at * 2, reinterpret_cast<const unsigned char*>(I.L0), n * 2);
+}
+
 // ---- host launchers ---------------------------------------------------------
+cudaError_t launch_gather_states(const InstDev* d_inst, int b0, int n, void* dst, size_t d_total, int esize,
+                                 cudaStream_t st)
+{
+    // about 8 KB of state per block in the mean, at least one and at most 1024 blocks an instance
+    const size_t per = d_total / n / 8192 + 1;
+    gather_states<<<dim3((unsigned)(per < 1024 ? per : 1024), n), 256, 0, st>>>(
+        d_inst, b0, static_cast<unsigned char*>(dst), d_total, esize);
+    return cudaGetLastError();
+}
 cudaError_t launch_gather_moments(const InstDev* d_inst, int ninst, const double* prof_all, double* out,
                                   cudaStream_t st)
 {

@@ -100,6 +100,7 @@ struct InstDev {
     void *F0, *F1, *F2;
     unsigned short *L0;           // [Nz][Q], FP32 storage only
     int *cur;                     // [1]
+    long state_at;                // values of the instances before this one (whole-batch states)
     void *rec;                    // [Nz][rec_stride]
     void *partial;                // [nchunks][kNMom][Nz] in the accumulation type (FP32 sums of FP32 storage)
     double *flux_part;            // [nchunks][2]: bottom, top outgoing flux

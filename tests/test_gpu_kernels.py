@@ -154,3 +154,33 @@ def test_default_tiling_follows_the_batch():
     assert tiling(dict(W.C2, Qx=9, Qy=9, Qz=9), 64, P.LBS_FP32) == (1, 0)
     assert tiling(W.C2, 1, P.LBS_FP64) == (1, 0)
     assert tiling(W.C2, 16, P.LBS_FP64) == (4, 0)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("offset", [0, 2, 8])
+def test_checkpoint_to_device_memory_equals_the_host_copy(prec, offset):
+    """lbs_get_state to device memory (one gathering launch) gives the bytes of the copy to
+    host memory: ragged instances whose buffers are not adjacent, whole batch and single
+    instance, destinations that are not 16-byte aligned, states in either buffer."""
+    import torch
+    P = _lbs()
+    pr = P.LBS_FP64 if prec == "fp64" else P.LBS_FP32
+    ps = [dict(W.C1, Nz=11), dict(W.C1, Qx=3, Qy=1, Qz=5, Nz=19), dict(W.C2, Nz=30), dict(W.C1, Qx=3, Qy=3, Nz=7)]
+    s = solver_of(ps, 1e-3, pr)
+    for steps in (0, 1, 3):
+        s.step(steps)
+        n = s.state_bytes()
+        host = np.zeros(n, np.uint8)
+        s.get_state_all_ptr(host.ctypes.data)
+        dev = torch.full((n + 16,), 7, dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        s.get_state_all_ptr(dev.data_ptr() + offset, to_host=False)
+        got = dev.cpu().numpy()
+        assert np.array_equal(got[offset:offset + n], host)
+        assert np.all(got[:offset] == 7) and np.all(got[offset + n:] == 7)
+        st = s.get_state(1)
+        one = st.d.view(np.uint8).ravel() if st.r is None else np.concatenate(
+            [st.d.view(np.uint8).ravel(), st.r.view(np.uint8).ravel()])
+        s.get_state_device(1, dev.data_ptr() + offset)
+        assert np.array_equal(dev.cpu().numpy()[offset:offset + one.size], one)
+    s.close()
