@@ -1376,6 +1376,18 @@ static size_t state_d_bytes(const lbs_solver* h, int b0, int b1)
     return n;
 }
 
+// dst is memory of the solver's own device (anything else is left to the copies, which take or
+// refuse it)
+static bool on_device(const lbs_solver* h, const void* dst)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == h->device;
+}
+
 lbs_status lbs_get_state(lbs_handle h, int inst, void* dst, int to_host)
 {
     if (!h || inst < -1 || inst >= h->ninst) return fail(LBS_ERR_ARG, "invalid handle or instance index");
@@ -1384,9 +1396,10 @@ lbs_status lbs_get_state(lbs_handle h, int inst, void* dst, int to_host)
     // Up to 48 MB to device memory: one launch that finds the buffers itself instead of a read
     // of the selectors and a copy or two per instance (20 table runs 167 -> 14 us, one C1
     // channel 22 -> 12, the 64-instance sweep, 50 MB, 68 -> 70; 256 x C2, 384 MB, 147 -> 242:
-    // larger states keep the copies, as does a destination at an odd address)
+    // larger states keep the copies, as does a destination at an odd address or elsewhere)
     const size_t d_total = state_d_bytes(h, b0, b1);
-    if (!to_host && d_total <= (size_t(48) << 20) && reinterpret_cast<uintptr_t>(dst) % 2 == 0 && b1 - b0 <= 65535) {
+    if (!to_host && d_total <= (size_t(48) << 20) && reinterpret_cast<uintptr_t>(dst) % 2 == 0 && b1 - b0 <= 65535 &&
+        on_device(h, dst)) {
         CK(launch_gather_states(h->d_inst, b0, b1 - b0, dst, d_total, h->esize, h->stream));
         CK(cudaStreamSynchronize(h->stream));
         return LBS_OK;
