@@ -61,6 +61,10 @@ struct InstHost {
 
 constexpr long kZSplitPairs = 4 * 608;
 
+// FP32 batches whose three state-sized buffers and residuals (14 bytes a value) exceed this, about
+// the L2's size, prefetch their increments (stage_kernel, where both sides' times stand)
+constexpr size_t kPrefetchBytes = size_t(120) << 20;
+
 constexpr size_t kSmemBudget = 200 * 1024;  // dynamic shared memory of a stage CTA
 
 struct Pool {  // bump allocator over one device allocation
@@ -424,6 +428,8 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         h->maxNz = std::max(h->maxNz, I.Nz);
         h->nb = std::max(h->nb, std::max(I.Nx, std::max(I.Ny, I.Nzq)));  // the batch's largest order
     }
+    long values = 0;  // of a state, all instances
+    for (const InstHost& I : h->ih) values += (long)I.Nz * I.Q;
     choose_tiling(h);
     build_tiles(h, tiles);
     for (int b = 0; b < h->ninst; ++b) {
@@ -510,6 +516,7 @@ static lbs_status setup(lbs_solver* h, const lbs_instance_desc* desc)
         D.reduced = I.reduced;
         // every row segment (row s, chunk start k0 in either half) starts on 16 bytes
         D.bulk = ((size_t)(I.Q / 2) * sizeof(T)) % 16 == 0;
+        D.prefetch = D.bulk && h->fp32 && 14 * (size_t)values > kPrefetchBytes;
         D.visc_law = d.visc.law; D.Kn = d.Kn; D.visc_param = d.visc.omega_or_S; D.Pr = d.Pr;
         D.iKn = 1.0 / d.Kn;
         D.isuth = d.visc.law == 1 ? 1.0 / (1.0 + d.visc.omega_or_S) : 0.0;

@@ -78,6 +78,7 @@ struct InstDev {
     Walls<double> walls;
     Walls<float> walls2;          // the same rounded to FP32
     unsigned mQy, mQxQy;          // ceil(2^32 / d) for div_small, 0 for d = 1
+    int prefetch;                 // the batch's buffers exceed the L2: tiles fetch their increments ahead
     // tables
     const double *Hx, *Hy, *Pz;   // FP64, [Q_a][N_a + 1] basis values He_l/l!, pi_l/h_l
     const float2 *Hx2, *Hy2, *Pz2;  // the same as FP32 (hi, lo) pairs, hi + lo = the FP64 value

@@ -184,3 +184,27 @@ def test_checkpoint_to_device_memory_equals_the_host_copy(prec, offset):
         s.get_state_device(1, dev.data_ptr() + offset)
         assert np.array_equal(dev.cpu().numpy()[offset:offset + one.size], one)
     s.close()
+
+
+@pytest.mark.parametrize("Qx,Qy,Qz,Nz,half", [(8, 8, 16, 64, 0), (6, 6, 17, 71, 1), (16, 0, 60, 75, 0)])
+def test_large_batch_steps_as_a_single_channel(Qx, Qy, Qz, Nz, half):
+    """A batch larger than L2, whose tiles fetch their increments ahead (rows of residuals that are
+    16-byte multiples and ones that are not, both walls or the centre line), gives every instance
+    the bytes that a solver of that instance alone computes with the same layouts."""
+    P = _lbs()
+    from paper_1702_01335_gb300 import Instance, Solver
+    inst = Instance(Qx=Qx, Qy=Qy, Qz=Qz, N_eq=3, Nz=Nz, A=0.8, half=half, Kn=0.3, u_w=0.4, Pr=2.0 / 3.0, cfl=0.4)
+    n = int(9.2e6 / (Nz * inst.Q)) + 1
+    a, b = Solver([inst] * n, precision=P.LBS_FP32), Solver(inst, precision=P.LBS_FP32)
+    z = np.linspace(-1.0, 1.0, Nz)[:, None]
+    d = 0.1 * np.sin(2 * z) + 0.02 * np.random.default_rng(5).standard_normal((1, inst.Q)) * (1 + 0.1 * z)
+    for s, which in ((a, (0, n - 1)), (b, (0,))):
+        s.set_tiling(4, 12, 0)
+        s.set_finalize(2)
+        for i in which:
+            s.set_state(i, d.astype(np.float32))
+        s.step(5)
+    one = b.get_state(0)
+    for i in (0, n - 1):
+        st = a.get_state(i)
+        assert np.array_equal(st.d, one.d) and np.array_equal(st.r, one.r)
