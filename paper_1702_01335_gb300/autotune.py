@@ -98,7 +98,7 @@ def autotune(solver, candidates=CANDIDATES, steps=3, cache_file=None, verbose=Fa
     if not table:
         raise ValueError("no valid tiling among the candidates")
     best = min(table, key=lambda r: r["ms_per_step"])
-    # then the finalisation layout (one thread or one warp per cell) for that tiling
+    # then the finalisation layout (at least eight cells per CTA, or four) for that tiling
     fin_times = {}
     scratch = Solver(solver.instances, precision=solver.precision)
     try:
