@@ -250,7 +250,7 @@ def run_small(a):
     st = s.torch_stream()
     upd_step = sum(i.Nz * i.Q for i in inst)
     s.step(a.warmup)
-    barrier()
+    torch.cuda.synchronize()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     with Clocks(local) as clk:
         e0.record(st)
