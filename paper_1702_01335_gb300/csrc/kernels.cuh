@@ -805,8 +805,10 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         // two).  The WENO differences are carried (carried_corr), so no window of values shifts.
         // Measured, stage kernels per step against the pair march (FP32) and the scalar march
         // (FP64): 256 x C2 1061 -> 987 us, 32 x C3 1049 -> 962, the sweep 405 -> 375; 16 x C2
-        // in FP64 3063 -> 2004 us (2365 at the same 12-cell tiles).  Instructions per update of
-        // the three FP32 stages: 112 / 137 / 155 -> 92 / 109 / 128.
+        // in FP64 3063 -> 2004 us (2365 at the same 12-cell tiles); now 944, 926, 357 and 1914
+        // with the weights of carried_weights and the prefetch above.  Instructions per update of
+        // the three FP32 stages: 112 / 137 / 155 -> 85 / 99 / 120; bound by latency at four CTAs
+        // per SM (2.0 to 2.2 instructions per cycle of 4), then issue.
         typedef typename Two<T>::type P;
         struct alignas(16) Quad { P p[2]; };
         auto quad = [](const T* q) -> Quad {  // 16-byte aligned
