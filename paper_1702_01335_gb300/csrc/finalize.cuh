@@ -580,11 +580,11 @@ __device__ __forceinline__ void finalize_group(const InstDev& I, int c0, int nc,
     record_cells<T, NB, C, true>(I, c0, nc, sm, vt, node);
 }
 
-// the fused finalisation: the cells of a z-tile, four at a time
+// the fused finalisation: the cells of a z-tile, four at a time; sm is the stage CTA's dynamic
+// shared memory, which stage_smem makes at least this large
 template <typename T>
 __device__ __noinline__ void finalize_tile(const InstDev& I, int z0, int zn, int stage, FinShared<T, 4>& sm)
 {
-    static_assert(sizeof(FinShared<T, 4>) <= 9 * kThreads * sizeof(T), "fits the rows of the smallest z-tile");
     for (int c = 0; c < zn; c += 4) {
         Node<T, kMaxN> node;
         node.load(I, threadIdx.x & 31);  // a cell's 32 lanes; the roles rotate by whole warps

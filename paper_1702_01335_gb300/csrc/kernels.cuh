@@ -433,7 +433,10 @@ __host__ __device__ inline StageSmem stage_smem(int zn, int KC, int G, int esize
     L.idz = o; o += pad16((size_t)zn * esize);
     L.red = o; o += (size_t)zn * (kThreads / 32 / zsplit) * 16 * asize;
     L.sc = o; o += grouped ? (size_t)zn * S_COUNT * 8 : 0;  // 80 bytes a cell in either type
-    L.total = o;
+    // the folded-in finalisation's cell group lies over all of it: the 32 columns of a three-cell
+    // FP64 tile at two to four velocities are shorter (3200 bytes against 3312)
+    const size_t fin = esize == 4 ? sizeof(FinShared<float, 4>) : sizeof(FinShared<double, 4>);
+    L.total = o > fin ? o : fin;
     return L;
 }
 

@@ -208,3 +208,43 @@ def test_large_batch_steps_as_a_single_channel(Qx, Qy, Qz, Nz, half):
     for i in (0, n - 1):
         st = a.get_state(i)
         assert np.array_equal(st.d, one.d) and np.array_equal(st.r, one.r)
+
+
+# (precision, Qx, Qy, Qz, Nz, V, ZT): three-cell z-split tiles at the smallest velocity sets (one
+# and two nodes per sign of p_z, phi / chi too), longer z-split tiles, the grouped march with
+# whole-tile and split warps, ragged chunks and tiles
+FOLDED = [("fp64", 1, 1, 1, 6, 1, 3), ("fp64", 1, 1, 2, 9, 1, 3), ("fp64", 1, 2, 1, 6, 1, 4), ("fp64", 2, 1, 1, 6, 1, 4),
+          ("fp64", 1, 0, 1, 9, 1, 3), ("fp64", 2, 2, 2, 7, 1, 3), ("fp64", 7, 7, 11, 23, 1, 5), ("fp64", 8, 8, 16, 41, 1, 16),
+          ("fp64", 8, 8, 16, 41, 4, 8), ("fp64", 3, 4, 7, 19, 4, 3), ("fp64", 1, 4, 1, 6, 4, 3),
+          ("fp32", 1, 4, 1, 6, 4, 3), ("fp32", 8, 8, 16, 41, 4, 13), ("fp32", 5, 8, 9, 23, 4, 5), ("fp32", 1, 1, 1, 6, 1, 3)]
+
+
+@pytest.mark.parametrize("fuse", [1, 2])
+@pytest.mark.parametrize("prec,Qx,Qy,Qz,Nz,V,ZT", FOLDED)
+def test_folded_and_split_finalisation_agree_with_separate_launches(prec, Qx, Qy, Qz, Nz, V, ZT, fuse):
+    """The finalisation folded into the stage kernel (fuse = 1) and split stepping (fuse = 2) against
+    separate launches, same layout.  Folded, the cells are grouped by z-tile, so only the choice
+    between the small-drift series and erfc can differ: 1e-12 (FP64) and 1e-5 (FP32 storage) of the
+    largest population after 9 steps, as between layouts."""
+    P = _lbs()
+    from paper_1702_01335_gb300 import Instance, Solver
+    pr = P.LBS_FP64 if prec == "fp64" else P.LBS_FP32
+    inst = [Instance(Qx=Qx, Qy=Qy, Qz=Qz, N_eq=3, Nz=Nz, A=0.8, half=b % 2, Kn=0.3 + 0.1 * b, u_w=0.4, Pr=2.0 / 3.0,
+                     visc_law=1, visc_param=0.5, cfl=0.1) for b in range(3)]
+    a, b = Solver(inst, precision=pr), Solver(inst, precision=pr)
+    a.set_tiling(V, ZT, 0)
+    b.set_tiling(V, ZT, fuse)
+    rng = np.random.default_rng(7)
+    z = np.linspace(-1.0, 1.0, Nz)[:, None]
+    for i in range(3):
+        d = (0.1 * np.sin(2 * z) + 0.02 * rng.standard_normal((1, inst[i].Q))) * (1 + 0.1 * z * z)
+        for s in (a, b):
+            s.set_state(i, d.astype(s.dtype))
+    for s in (a, b):
+        s.step(9)
+    tol = 1e-12 if prec == "fp64" else 1e-5
+    for i in range(3):
+        assert rel_err(b.populations(i), a.populations(i)) < tol, i
+        pa, pb = a.profiles(i), b.profiles(i)
+        assert max(np.abs(pa[k] - pb[k]).max() for k in pa) < 10 * tol, i
+        assert abs(a.residual(i) - b.residual(i)) <= 100 * tol * max(a.residual(i), 1e-2), i
