@@ -1383,16 +1383,17 @@ static size_t state_d_bytes(const lbs_solver* h, int b0, int b1)
     return n;
 }
 
-// dst is memory of the solver's own device (anything else is left to the copies, which take or
-// refuse it)
-static bool on_device(const lbs_solver* h, const void* dst)
+// what gather_allowed asks about dst; a query that fails leaves it to the copies
+static GatherTarget gather_target(const void* dst)
 {
+    GatherTarget t;
     cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess || cudaGetDevice(&t.current) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return t;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == h->device;
+    if (at.type == cudaMemoryTypeDevice) t.device = at.device;
+    return t;
 }
 
 lbs_status lbs_get_state(lbs_handle h, int inst, void* dst, int to_host)
@@ -1406,7 +1407,7 @@ lbs_status lbs_get_state(lbs_handle h, int inst, void* dst, int to_host)
     // larger states keep the copies, as does a destination at an odd address or elsewhere)
     const size_t d_total = state_d_bytes(h, b0, b1);
     if (!to_host && d_total <= (size_t(48) << 20) && reinterpret_cast<uintptr_t>(dst) % 2 == 0 && b1 - b0 <= 65535 &&
-        on_device(h, dst)) {
+        gather_allowed(gather_target(dst), h->device)) {
         CK(launch_gather_states(h->d_inst, b0, b1 - b0, dst, d_total, h->esize, h->stream));
         CK(cudaStreamSynchronize(h->stream));
         return LBS_OK;

@@ -273,6 +273,20 @@ LBS_HD double relax_time(int law, double Kn, double param, double n, double T)
     return Kn * sqrt(T) * (1.0 + param) / (n * (T + param));
 }
 
+// ---- the destination of lbs_get_state's gathering launch ----
+// A kernel needs the solver's device to be the current one and writes wherever it is told; a
+// copy runs whatever device is current and refuses what is not memory.  So the launch takes
+// memory of the solver's own device while that is current, and everything else goes through
+// the copies.
+struct GatherTarget {
+    int device = -1;   // the device whose memory it is, -1 otherwise (host, managed, unknown)
+    int current = -1;  // the calling thread's device
+};
+inline bool gather_allowed(const GatherTarget& t, int solver_device)
+{
+    return t.device == solver_device && t.current == solver_device;
+}
+
 // ---- access to a handle for entry points defined outside api.cu ----
 struct HandleView {
     const InstDev* d_inst;   // device array of descriptors
