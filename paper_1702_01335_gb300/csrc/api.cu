@@ -1386,13 +1386,28 @@ static size_t state_d_bytes(const lbs_solver* h, int b0, int b1)
 // what gather_allowed asks about dst; a query that fails leaves it to the copies
 static GatherTarget gather_target(const void* dst)
 {
+    // the extent of an allocation is known to the driver alone, whose library is not linked
+    typedef int (*AddressRange)(unsigned long long*, size_t*, unsigned long long);
+    static const AddressRange address_range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        const cudaError_t e =
+            cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found);
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? reinterpret_cast<AddressRange>(f) : nullptr;
+    }();
     GatherTarget t;
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, dst) != cudaSuccess || cudaGetDevice(&t.current) != cudaSuccess) {
         cudaGetLastError();
         return t;
     }
-    if (at.type == cudaMemoryTypeDevice) t.device = at.device;
+    if (at.type != cudaMemoryTypeDevice || !address_range) return t;
+    const unsigned long long p = reinterpret_cast<uintptr_t>(dst);
+    unsigned long long base = 0;
+    size_t size = 0;
+    if (address_range(&base, &size, p) != 0) return t;
+    t.device = at.device;
+    t.bytes = size - (size_t)(p - base);
     return t;
 }
 
@@ -1405,9 +1420,9 @@ lbs_status lbs_get_state(lbs_handle h, int inst, void* dst, int to_host)
     // of the selectors and a copy or two per instance (20 table runs 167 -> 14 us, one C1
     // channel 22 -> 12, the 64-instance sweep, 50 MB, 68 -> 70; 256 x C2, 384 MB, 147 -> 242:
     // larger states keep the copies, as does a destination at an odd address or elsewhere)
-    const size_t d_total = state_d_bytes(h, b0, b1);
+    const size_t d_total = state_d_bytes(h, b0, b1), bytes = d_total + (h->fp32 ? d_total / 2 : 0);
     if (!to_host && d_total <= (size_t(48) << 20) && reinterpret_cast<uintptr_t>(dst) % 2 == 0 && b1 - b0 <= 65535 &&
-        gather_allowed(gather_target(dst), h->device)) {
+        gather_allowed(gather_target(dst), h->device, bytes)) {
         CK(launch_gather_states(h->d_inst, b0, b1 - b0, dst, d_total, h->esize, h->stream));
         CK(cudaStreamSynchronize(h->stream));
         return LBS_OK;

@@ -8,6 +8,7 @@ struct float2;  // host code built without the CUDA headers holds only pointers 
 #endif
 
 #include <cmath>
+#include <cstddef>
 #include <vector>
 
 #if defined(__CUDACC__)
@@ -276,15 +277,16 @@ LBS_HD double relax_time(int law, double Kn, double param, double n, double T)
 // ---- the destination of lbs_get_state's gathering launch ----
 // A kernel needs the solver's device to be the current one and writes wherever it is told; a
 // copy runs whatever device is current and refuses what is not memory.  So the launch takes
-// memory of the solver's own device while that is current, and everything else goes through
-// the copies.
+// memory of the solver's own device while that is current, in an allocation that holds the
+// whole state, and everything else goes through the copies.
 struct GatherTarget {
     int device = -1;   // the device whose memory it is, -1 otherwise (host, managed, unknown)
     int current = -1;  // the calling thread's device
+    size_t bytes = 0;  // from the destination to the end of its allocation
 };
-inline bool gather_allowed(const GatherTarget& t, int solver_device)
+inline bool gather_allowed(const GatherTarget& t, int solver_device, size_t state_bytes)
 {
-    return t.device == solver_device && t.current == solver_device;
+    return t.device == solver_device && t.current == solver_device && state_bytes <= t.bytes;
 }
 
 // ---- access to a handle for entry points defined outside api.cu ----

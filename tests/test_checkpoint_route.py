@@ -26,7 +26,22 @@ def test_gathering_launch_needs_the_solvers_device_to_be_current(tmp_path):
                 GatherTarget t;
                 t.device = device;
                 t.current = current;
-                std::printf("%d ", gather_allowed(t, solver));
+                t.bytes = 1 << 20;
+                std::printf("%d ", gather_allowed(t, solver, 1 << 20));
             }""")
     want = [d == s and c == s for s in (0, 1) for d in (-1, 0, 1) for c in (-1, 0, 1)]
     assert [g == "1" for g in got] == want and sum(want) == 2
+
+
+def test_gathering_launch_needs_an_allocation_that_holds_the_state(tmp_path):
+    """A destination whose allocation ends before the state does is left to the copies, which
+    refuse it; the kernel would write past it.  Nothing is known of memory that a query failed for."""
+    got = answers(tmp_path, """
+    for (size_t bytes : {size_t(0), size_t(599), size_t(600), size_t(601), size_t(1) << 40}) {
+        GatherTarget t;
+        t.device = t.current = 0;
+        t.bytes = bytes;
+        std::printf("%d ", gather_allowed(t, 0, 600));
+    }
+    std::printf("%d ", gather_allowed(GatherTarget(), 0, 0));""")
+    assert got == ["0", "0", "1", "1", "1", "0"]

@@ -248,3 +248,44 @@ def test_folded_and_split_finalisation_agree_with_separate_launches(prec, Qx, Qy
         pa, pb = a.profiles(i), b.profiles(i)
         assert max(np.abs(pa[k] - pb[k]).max() for k in pa) < 10 * tol, i
         assert abs(a.residual(i) - b.residual(i)) <= 100 * tol * max(a.residual(i), 1e-2), i
+
+
+def _drop_cuda_error():
+    """A refused copy stays the CUDA runtime's last error; torch's next check takes and reports it."""
+    import torch
+    try:
+        torch.zeros(1, device="cuda")
+    except RuntimeError:
+        pass
+    torch.zeros(1, device="cuda")
+
+
+def _short_allocation(nbytes):
+    """A device allocation of its own (driver API) of nbytes: address, release."""
+    import ctypes
+
+    import torch
+    torch.zeros(1, device="cuda")
+    cu, p = ctypes.CDLL("libcuda.so.1"), ctypes.c_uint64()
+    assert cu.cuMemAlloc_v2(ctypes.byref(p), ctypes.c_size_t(nbytes)) == 0
+    return p.value, lambda: cu.cuMemFree_v2(p)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_checkpoint_to_a_short_allocation_is_refused(prec):
+    """A device allocation of its own that ends before the state does: refused as by a copy, and the
+    solver is as before.  (It lies in a mapped page much larger than the state, so that nothing
+    could fault in any case.)"""
+    P = _lbs()
+    s = solver_of(dict(W.C1, Nz=11), 1e-3, P.LBS_FP64 if prec == "fp64" else P.LBS_FP32)
+    assert s.state_bytes() < 1 << 17
+    p, release = _short_allocation(s.state_bytes() // 2)
+    s.step(2)
+    before = s.get_state(0)
+    with pytest.raises(P.LbsError):
+        s.get_state_all_ptr(p, to_host=False)
+    release()
+    _drop_cuda_error()
+    after = s.get_state(0)
+    assert np.array_equal(before.d, after.d) and (before.r is None or np.array_equal(before.r, after.r))
+    s.close()
