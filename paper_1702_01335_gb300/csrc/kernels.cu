@@ -154,9 +154,12 @@ cudaError_t launch_gather_states(const InstDev* d_inst, int b0, int n, void* dst
 {
     // about 8 KB of state per block in the mean, at least one and at most 1024 blocks an instance
     const size_t per = d_total / n / 8192 + 1;
-    gather_states<<<dim3((unsigned)(per < 1024 ? per : 1024), n), 256, 0, st>>>(
-        d_inst, b0, static_cast<unsigned char*>(dst), d_total, esize);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(per < 1024 ? per : 1024), n);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    // the launch's own status: the last error may be an earlier call's (a refused copy's)
+    return cudaLaunchKernelEx(&cfg, gather_states, d_inst, b0, static_cast<unsigned char*>(dst), d_total, esize);
 }
 cudaError_t launch_gather_moments(const InstDev* d_inst, int ninst, const double* prof_all, double* out,
                                   cudaStream_t st)

@@ -289,3 +289,24 @@ def test_checkpoint_to_a_short_allocation_is_refused(prec):
     after = s.get_state(0)
     assert np.array_equal(before.d, after.d) and (before.r is None or np.array_equal(before.r, after.r))
     s.close()
+
+
+def test_checkpoint_after_another_calls_error():
+    """A CUDA error that an earlier call left behind (here a refused checkpoint) is not taken for the
+    next checkpoint's own."""
+    import torch
+    P = _lbs()
+    s = solver_of(dict(W.C1, Nz=11), 1e-3, P.LBS_FP32)
+    n = s.state_bytes()
+    host, dev = np.zeros(n, np.uint8), torch.zeros(n, dtype=torch.uint8, device="cuda")
+    p, release = _short_allocation(n // 2)
+    s.step(2)
+    s.get_state_all_ptr(host.ctypes.data)
+    torch.cuda.synchronize()
+    with pytest.raises(P.LbsError):
+        s.get_state_all_ptr(p, to_host=False)
+    s.get_state_all_ptr(dev.data_ptr(), to_host=False)
+    release()
+    _drop_cuda_error()
+    assert np.array_equal(dev.cpu().numpy(), host)
+    s.close()
