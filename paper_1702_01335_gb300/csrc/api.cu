@@ -27,7 +27,7 @@ cudaError_t launch_seed(int fp32, const InstDev* d_inst, int inst, int Nz, const
 cudaError_t launch_seed_free_molecular(int fp32, const InstDev* d_inst, int inst, int Nz, cudaStream_t st);
 cudaError_t launch_gather_moments(const InstDev* d_inst, int ninst, const double* prof_all, double* out,
                                   cudaStream_t st);
-cudaError_t launch_gather_states(const InstDev* d_inst, int b0, int n, void* dst, size_t d_total, int esize,
+cudaError_t launch_gather_states(const InstDev* d_inst, int b0, int n, long at, long total, void* dst, int esize,
                                  cudaStream_t st);
 size_t stage_smem_bytes(int fp32, int V, int zn, int Qx, int Qy, int nzm, int rstride);
 }  // namespace lbs
@@ -1418,12 +1418,14 @@ lbs_status lbs_get_state(lbs_handle h, int inst, void* dst, int to_host)
     const int b0 = inst < 0 ? 0 : inst, b1 = inst < 0 ? h->ninst : inst + 1;
     // Up to 48 MB to device memory: one launch that finds the buffers itself instead of a read
     // of the selectors and a copy or two per instance (20 table runs 167 -> 14 us, one C1
-    // channel 22 -> 12, the 64-instance sweep, 50 MB, 68 -> 70; 256 x C2, 384 MB, 147 -> 242:
-    // larger states keep the copies, as does a destination at an odd address or elsewhere)
+    // channel 22 -> 12, one state of 47 MB 47 -> 36; the 256 x C2 batch, 384 MB, took 147 us by
+    // copies and 242 by an earlier form of the launch: larger states keep the copies, as does a
+    // destination at an odd address or elsewhere)
     const size_t d_total = state_d_bytes(h, b0, b1), bytes = d_total + (h->fp32 ? d_total / 2 : 0);
-    if (!to_host && d_total <= (size_t(48) << 20) && reinterpret_cast<uintptr_t>(dst) % 2 == 0 && b1 - b0 <= 65535 &&
+    if (!to_host && d_total <= (size_t(48) << 20) && reinterpret_cast<uintptr_t>(dst) % 2 == 0 &&
         gather_allowed(gather_target(dst), h->device, bytes)) {
-        CK(launch_gather_states(h->d_inst, b0, b1 - b0, dst, d_total, h->esize, h->stream));
+        CK(launch_gather_states(h->d_inst, b0, b1 - b0, h->idev[b0].state_at, (long)(d_total / h->esize), dst, h->esize,
+                                h->stream));
         CK(cudaStreamSynchronize(h->stream));
         return LBS_OK;
     }

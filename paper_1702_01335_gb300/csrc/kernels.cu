@@ -110,56 +110,100 @@ __global__ void __launch_bounds__(128) gather_moment_rows(const InstDev* __restr
     for (int c = threadIdx.x; c < I.Nz; c += blockDim.x) dst[c] = src[c];
 }
 
-// bytes from src to dst by the whole grid row (blockIdx.x of gridDim.x): 16 at a time where
-// both allow, else 2 (every state is a whole number of 16-bit units)
-static __device__ __forceinline__ void copy_bytes(unsigned char* dst, const unsigned char* src, size_t n)
+// 16 bytes at an even address from the two aligned words that hold them: m the offset into a
+static __device__ __forceinline__ uint4 word_at(const uint4& a, const uint4& b, int m)
 {
-    const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
-    if (((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) == 0) {
-        const uint4* s = reinterpret_cast<const uint4*>(src);
-        uint4* d = reinterpret_cast<uint4*>(dst);
-        const size_t words = n / 16;
-        size_t e = t;
-        for (; e + 3 * step < words; e += 4 * step) {
-            const uint4 a = __ldcs(s + e), b = __ldcs(s + e + step), c = __ldcs(s + e + 2 * step),
-                        x = __ldcs(s + e + 3 * step);
-            __stcs(d + e, a);
-            __stcs(d + e + step, b);
-            __stcs(d + e + 2 * step, c);
-            __stcs(d + e + 3 * step, x);
-        }
-        for (; e < words; e += step) __stcs(d + e, __ldcs(s + e));
-        for (size_t q = words * 8 + t; q < n / 2; q += step)
-            reinterpret_cast<unsigned short*>(dst)[q] = reinterpret_cast<const unsigned short*>(src)[q];
-    } else {
-        for (size_t q = t; q < n / 2; q += step)
-            reinterpret_cast<unsigned short*>(dst)[q] = reinterpret_cast<const unsigned short*>(src)[q];
+    const unsigned r = (m & 2) * 8;
+    auto four = [r](unsigned x0, unsigned x1, unsigned x2, unsigned x3, unsigned x4) {
+        return make_uint4(__funnelshift_r(x0, x1, r), __funnelshift_r(x1, x2, r), __funnelshift_r(x2, x3, r),
+                          __funnelshift_r(x3, x4, r));
+    };
+    switch (m >> 2) {
+        case 0: return four(a.x, a.y, a.z, a.w, b.x);
+        case 1: return four(a.y, a.z, a.w, b.x, b.y);
+        case 2: return four(a.z, a.w, b.x, b.y, b.z);
+        default: return four(a.w, b.x, b.y, b.z, b.w);
+    }
+}
+// n bytes from src to dst by a warp, all even.  Aligned 16-byte stores; where src and dst lie
+// differently in their words, a word is put together from the two of the source that hold it.
+// Both hold bytes of the copy, so nothing is read outside the source's 16-byte words.
+static __device__ __forceinline__ void copy_bytes(unsigned char* dst, const unsigned char* src, size_t n, int lane)
+{
+    const size_t to_word = (16 - (reinterpret_cast<uintptr_t>(dst) & 15)) & 15, head = to_word < n ? to_word : n;
+    const size_t words = (n - head) / 16, tail = head + 16 * words;
+    auto two_bytes = [&](size_t at) {
+        *reinterpret_cast<unsigned short*>(dst + at) = *reinterpret_cast<const unsigned short*>(src + at);
+    };
+    if (2 * lane < head) two_bytes(2 * lane);
+    if (tail + 2 * lane < n) two_bytes(tail + 2 * lane);
+    uint4* d = reinterpret_cast<uint4*>(dst + head);
+    const int m = reinterpret_cast<uintptr_t>(src + head) & 15;
+    const uint4* s = reinterpret_cast<const uint4*>(src + head - m);
+    for (size_t w = lane; w < words; w += 128) {
+        uint4 a[4], b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (w + 32 * i < words) {
+                a[i] = __ldcs(s + w + 32 * i);
+                if (m) b[i] = __ldcs(s + w + 32 * i + 1);
+            }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (w + 32 * i < words) __stcs(d + w + 32 * i, m ? word_at(a[i], b[i], m) : a[i]);
     }
 }
 
-// The state of instances b0 .. b0 + gridDim.y - 1 to device memory in lbs_get_state's layout:
-// every d, then (FP32) every residual; each instance's buffer is found on the device.
-__global__ void __launch_bounds__(256) gather_states(const InstDev* __restrict__ insts, int b0, unsigned char* dst,
-                                                     size_t d_total, int esize)
+// The state of instances b0 .. b0 + n - 1 (at: values before b0, total: theirs) to device memory in
+// lbs_get_state's layout: every d, then (FP32) every residual.  Each warp takes `per` values of
+// the whole, whatever the instances' sizes, and finds the instance they begin in and its
+// buffers on the device.  Bound by memory from some 10 MB on, by latency below.
+// Measured, host call in us, against blocks shared out by instance with 2-byte units off 16 bytes
+// (and against copies): FP32, one 39 MB instance and 99 small ones 66 -> 34 (45), the same to an
+// address 8 off 16 bytes 817 -> 41 (53), one 47 MB state 8 off 188 -> 44 (54), one of odd size 2 off
+// 194 -> 44 (78), four of 11 MB and odd size 77 -> 35 (103); FP64, 12 MB 8 off 35 -> 19 (29).
+__global__ void __launch_bounds__(256) gather_states(const InstDev* __restrict__ insts, int b0, int n, long at,
+                                                     long total, long per, unsigned char* dst, int esize)
 {
-    const InstDev& I = insts[b0 + blockIdx.y];
-    const size_t n = (size_t)I.Nz * I.Q, at = I.state_at - insts[b0].state_at;
-    copy_bytes(dst + at * esize, static_cast<const unsigned char*>(*I.cur ? I.F1 : I.F0), n * esize);
-    if (I.L0) copy_bytes(dst + d_total + at * 2, reinterpret_cast<const unsigned char*>(I.L0), n * 2);
+    const int lane = threadIdx.x & 31;
+    long v = (blockIdx.x * (long)(blockDim.x / 32) + threadIdx.x / 32) * per;
+    const long end = v + per < total ? v + per : total;
+    if (v >= end) return;
+    // the last instance that begins at or before v: 32 candidates per step
+    int b = 0;
+    for (int len = n; len > 1;) {
+        const int step = (len + 31) / 32, c = lane * step;
+        const bool before = c < len && insts[b0 + b + c].state_at - at <= v;
+        const int k = __popc(__ballot_sync(0xffffffffu, before)) - 1;  // candidate 0 always is
+        b += k * step;
+        len = len - k * step < step ? len - k * step : step;
+    }
+    for (; v < end; ++b) {
+        const InstDev& I = insts[b0 + b];
+        const long i0 = I.state_at - at, i1 = i0 + (long)I.Nz * I.Q, e = end < i1 ? end : i1;
+        const unsigned char* F = static_cast<const unsigned char*>(*I.cur ? I.F1 : I.F0);
+        copy_bytes(dst + v * esize, F + (v - i0) * esize, (size_t)(e - v) * esize, lane);
+        if (I.L0)
+            copy_bytes(dst + total * esize + v * 2, reinterpret_cast<const unsigned char*>(I.L0 + (v - i0)),
+                       (size_t)(e - v) * 2, lane);
+        v = e;
+    }
 }
 
 // ---- host launchers ---------------------------------------------------------
-cudaError_t launch_gather_states(const InstDev* d_inst, int b0, int n, void* dst, size_t d_total, int esize,
+cudaError_t launch_gather_states(const InstDev* d_inst, int b0, int n, long at, long total, void* dst, int esize,
                                  cudaStream_t st)
 {
-    // about 8 KB of state per block in the mean, at least one and at most 1024 blocks an instance
-    const size_t per = d_total / n / 8192 + 1;
+    // 512 values a warp (four 16-byte words per lane in FP32), or more so that one wave of 64 warps
+    // per SM takes them all
+    const long per = 512 * ((total - 1) / (512L * 64 * 152) + 1), warps = (total + per - 1) / per;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(per < 1024 ? per : 1024), n);
+    cfg.gridDim = dim3((unsigned)((warps + 7) / 8));
     cfg.blockDim = dim3(256);
     cfg.stream = st;
     // the launch's own status: the last error may be an earlier call's (a refused copy's)
-    return cudaLaunchKernelEx(&cfg, gather_states, d_inst, b0, static_cast<unsigned char*>(dst), d_total, esize);
+    return cudaLaunchKernelEx(&cfg, gather_states, d_inst, b0, n, at, total, per, static_cast<unsigned char*>(dst),
+                              esize);
 }
 cudaError_t launch_gather_moments(const InstDev* d_inst, int ninst, const double* prof_all, double* out,
                                   cudaStream_t st)

@@ -310,3 +310,38 @@ def test_checkpoint_after_another_calls_error():
     _drop_cuda_error()
     assert np.array_equal(dev.cpu().numpy(), host)
     s.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("sizes", [[(7, 7, 11, 65 + 2 * b) for b in range(5)], [(1, 1, 1, 6)],
+                                   [(9, 9, 31, 151)] + [(3, 1, 1 + b % 2, 6 + b % 5) for b in range(39)],
+                                   [(1, 1 + b % 2, 1, 6 + b % 3) for b in range(1030)]],
+                         ids=["odd", "smallest", "uneven", "many"])
+def test_checkpoint_at_every_alignment(sizes, prec):
+    """A checkpoint to device memory at every even offset from 16 bytes equals the copy to host
+    memory: states that are not whole 16-byte words, one large instance among small ones, states
+    shorter than a warp's share, more than 32 and more than 1024 instances; nothing beside it is
+    written."""
+    import torch
+    P = _lbs()
+    from paper_1702_01335_gb300 import Instance, Solver
+    s = Solver([Instance(Qx=x, Qy=y, Qz=z, N_eq=3, Nz=Nz, A=0.5, Kn=0.3, u_w=0.4, Pr=2.0 / 3.0, dt=1e-3)
+                for x, y, z, Nz in sizes], precision=P.LBS_FP64 if prec == "fp64" else P.LBS_FP32)
+    n = s.state_bytes()
+    rng = np.random.default_rng(3)
+    host, out = rng.integers(0, 256, n, dtype=np.uint8), np.zeros(n, np.uint8)
+    nd = n if prec == "fp64" else n // 6 * 4
+    host[:nd] = (0.1 * rng.standard_normal(nd // 8 if prec == "fp64" else nd // 4)).astype(s.dtype).view(np.uint8)
+    s.set_state_all_ptr(host.ctypes.data)
+    for steps in (0, 1):  # the state in either buffer
+        s.step(steps)
+        s.get_state_all_ptr(out.ctypes.data)
+        assert steps or np.array_equal(out, host)
+        for offset in range(0, 16, 2):
+            dev = torch.full((n + 64,), 7, dtype=torch.uint8, device="cuda")
+            torch.cuda.synchronize()
+            s.get_state_all_ptr(dev.data_ptr() + 16 + offset, to_host=False)
+            got = dev.cpu().numpy()
+            assert np.array_equal(got[16 + offset:16 + offset + n], out)
+            assert np.all(got[:16 + offset] == 7) and np.all(got[16 + offset + n:] == 7)
+    s.close()
