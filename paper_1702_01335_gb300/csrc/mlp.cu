@@ -326,8 +326,10 @@ __global__ void __launch_bounds__(kThreadsMlp) backward_gemm(Operand<float> dzT,
     }
 }
 
-// Adam (bias corrected) on the FP32 masters, then refresh the BF16 weight copies
-__global__ void adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
+// Adam (bias corrected) on the FP32 masters, then refresh the BF16 weight copies.  g is no
+// __restrict__: the kernel starts while its predecessor still writes the gradients, and loads of
+// memory promised constant could go through the read-only path or above the wait.
+__global__ void adam(float* __restrict__ p, const float* g, float* __restrict__ m,
                      float* __restrict__ v, long n, float lr, float b1, float b2, float eps, float c1, float c2,
                      __nv_bfloat16* __restrict__ pb, const unsigned char* __restrict__ is_w)
 {
