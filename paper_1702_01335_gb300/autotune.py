@@ -50,10 +50,12 @@ def device_tag():
 
 def signature(solver):
     """Kernel hash, precision, the GPU, and the (Nz, Q) of the batch's instances with
-    the velocity model (r: the reduced phi / chi model, which runs other kernels) and
+    the velocity model (r: the reduced phi / chi model, n: a full one whose Qy is not a
+    multiple of four, which rules the grouped march out; both run other kernels) and
     the channel (h: a half channel), run-length encoded ("256*128x2048")."""
     def tag(i):
-        return "%dx%d%s%s" % (i.Nz, i.Q, "r" if i.Qy == 0 else "", "h" if i.half else "")
+        model = "r" if i.Qy == 0 else "n" if i.Qy % 4 else ""
+        return "%dx%d%s%s" % (i.Nz, i.Q, model, "h" if i.half else "")
     runs = [(k, len(list(g))) for k, g in itertools.groupby(tag(i) for i in solver.instances)]
     return "%s:p%d:%s:" % (kernel_hash(), solver.precision, device_tag()) + ",".join(
         ("%d*%s" % (n, k)) if n > 1 else k for k, n in runs)

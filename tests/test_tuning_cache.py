@@ -1,0 +1,20 @@
+"""Host-side checks of the tuning cache's key (autotune.py)."""
+from types import SimpleNamespace
+
+from paper_1702_01335_gb300 import autotune as AT
+from paper_1702_01335_gb300 import lbs as L
+
+
+def key(*instances):
+    return AT.signature(SimpleNamespace(instances=list(instances), precision=1))
+
+
+def test_signature_tells_the_marches_apart():
+    """V = 4 (and V = 1 in FP64) runs the grouped march where every Qy is a multiple of four, another
+    one elsewhere: batches of the same (Nz, Q) on either side have keys of their own."""
+    a, b = L.Instance(Qx=8, Qy=8, Qz=16, Nz=64), L.Instance(Qx=16, Qy=2, Qz=32, Nz=64)
+    assert a.Q == b.Q and key(a) != key(b) and key(a, a) != key(a, b)
+    c = L.Instance(Qx=16, Qy=4, Qz=16, Nz=64)  # grouped too
+    assert c.Q == a.Q and key(a) == key(c)
+    r = L.Instance(Qx=16, Qy=0, Qz=32, Nz=64)
+    assert r.Q == a.Q and len({key(a), key(b), key(r)}) == 3
