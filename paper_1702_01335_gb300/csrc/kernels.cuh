@@ -1416,51 +1416,25 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
         A acc[16];
 #pragma unroll
         for (int a = kNMom; a < 16; ++a) acc[a] = A(0);
-        if constexpr (kPack && !RED) {
-            float2 s2[kNMom];
 #pragma unroll
-            for (int p2 = 0; p2 < V / 2; ++p2) {
-                const int v0 = 2 * p2, v1 = v0 + 1;
-                const float2 o = make_float2(ov[v0], ov[v1]), X = make_float2(mx[v0], mx[v1]),
-                             Y = make_float2(my[v0], my[v1]), Z = make_float2(mz[v0], mz[v1]),
-                             P = make_float2(m2[v0], m2[v1]);
-                const float2 oX = mul2(o, X), oY = mul2(o, Y), oZ = mul2(o, Z), oP = mul2(o, P);
-                if (p2 == 0) {
-                    s2[0] = o; s2[1] = oX; s2[2] = oY; s2[3] = oZ;
-                    s2[4] = mul2(oX, X); s2[5] = mul2(oY, Y); s2[6] = mul2(oZ, Z);
-                    s2[7] = mul2(oX, Y); s2[8] = mul2(oX, Z); s2[9] = mul2(oY, Z);
-                    s2[10] = mul2(oP, X); s2[11] = mul2(oP, Y); s2[12] = mul2(oP, Z);
-                } else {
-                    s2[0] = add2(s2[0], o); s2[1] = add2(s2[1], oX); s2[2] = add2(s2[2], oY);
-                    s2[3] = add2(s2[3], oZ);
-                    s2[4] = fma2(oX, X, s2[4]); s2[5] = fma2(oY, Y, s2[5]); s2[6] = fma2(oZ, Z, s2[6]);
-                    s2[7] = fma2(oX, Y, s2[7]); s2[8] = fma2(oX, Z, s2[8]); s2[9] = fma2(oY, Z, s2[9]);
-                    s2[10] = fma2(oP, X, s2[10]); s2[11] = fma2(oP, Y, s2[11]); s2[12] = fma2(oP, Z, s2[12]);
-                }
+        for (int v = 0; v < V; ++v) {
+            A t[kNMom];
+            const A o = ov[v], X = mx[v], Y = my[v], Z = mz[v], P = m2[v];
+            if (RED) {  // phi: p_y = 0; chi: the p_y^2 parts
+                const A oc = chi[v] ? o : A(0), op = o - oc;
+                const A oX = op * X, oZ = op * Z, r3 = op * P + oc;
+                t[0] = op; t[1] = oX; t[2] = A(0); t[3] = oZ;
+                t[4] = oX * X; t[5] = oc; t[6] = oZ * Z; t[7] = A(0); t[8] = oX * Z;
+                t[9] = A(0); t[10] = r3 * X; t[11] = A(0); t[12] = r3 * Z;
+            } else {
+                const A oX = o * X, oY = o * Y, oZ = o * Z, oP = o * P;
+                t[0] = o; t[1] = oX; t[2] = oY; t[3] = oZ;
+                t[4] = oX * X; t[5] = oY * Y; t[6] = oZ * Z;
+                t[7] = oX * Y; t[8] = oX * Z; t[9] = oY * Z;
+                t[10] = oP * X; t[11] = oP * Y; t[12] = oP * Z;
             }
 #pragma unroll
-            for (int a = 0; a < kNMom; ++a) acc[a] = s2[a].x + s2[a].y;
-        } else {
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                A t[kNMom];
-                const A o = ov[v], X = mx[v], Y = my[v], Z = mz[v], P = m2[v];
-                if (RED) {  // phi: p_y = 0; chi: the p_y^2 parts
-                    const A oc = chi[v] ? o : A(0), op = o - oc;
-                    const A oX = op * X, oZ = op * Z, r3 = op * P + oc;
-                    t[0] = op; t[1] = oX; t[2] = A(0); t[3] = oZ;
-                    t[4] = oX * X; t[5] = oc; t[6] = oZ * Z; t[7] = A(0); t[8] = oX * Z;
-                    t[9] = A(0); t[10] = r3 * X; t[11] = A(0); t[12] = r3 * Z;
-                } else {
-                    const A oX = o * X, oY = o * Y, oZ = o * Z, oP = o * P;
-                    t[0] = o; t[1] = oX; t[2] = oY; t[3] = oZ;
-                    t[4] = oX * X; t[5] = oY * Y; t[6] = oZ * Z;
-                    t[7] = oX * Y; t[8] = oX * Z; t[9] = oY * Z;
-                    t[10] = oP * X; t[11] = oP * Y; t[12] = oP * Z;
-                }
-#pragma unroll
-                for (int a = 0; a < kNMom; ++a) acc[a] = v == 0 ? t[a] : acc[a] + t[a];
-            }
+            for (int a = 0; a < kNMom; ++a) acc[a] = v == 0 ? t[a] : acc[a] + t[a];
         }
         const A tot = reduce_scatter16<A>(acc, lane);
         const int m = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);

@@ -125,28 +125,15 @@ constexpr unsigned kDrainLimit = 1u << 28;  // spins granted to copies still in 
 
 struct Tile { int inst, z0, zn, chunk, zt; };
 
-// ---- equilibrium coefficients (shared by host set-up and device finalise) ----
+// ---- equilibrium coefficients of the walls, at set-up ----
 
 // a_l = int g(p; u, T) He_l(p) dp: a_0 = 1, a_1 = u, a_{l+1} = u a_l + l (T - 1) a_{l-1}
 // (from int g p He_l = u a_l + T l a_{l-1} and He_{l+1} = p He_l - l He_{l-1}).
-// Loops below run to a bound NB on the order (the largest order kMaxN by default;
-// device code instantiates smaller bounds for batches of low order) and test the
-// actual order inside, so that, unrolled, every array index is a constant and device
-// code keeps the arrays in registers instead of local memory.
-#if defined(__CUDACC__)
-#define LBS_UNROLL _Pragma("unroll")
-#else
-#define LBS_UNROLL
-#endif
-
-template <int NB = kMaxN>
-LBS_HD void full_coeffs(double u, double T, int N, double* a)
+inline void full_coeffs(double u, double T, int N, double* a)
 {
     a[0] = 1.0;
     a[1] = u;  // read only when N >= 1
-    LBS_UNROLL
-    for (int l = 1; l < NB; ++l)
-        if (l < N) a[l + 1] = u * a[l] + l * (T - 1.0) * a[l - 1];
+    for (int l = 1; l < N; ++l) a[l + 1] = u * a[l] + l * (T - 1.0) * a[l - 1];
 }
 
 // b_l = int_0^inf g(p; u, T) pi_l(p) dp for the monic half-range polynomials,
@@ -224,29 +211,6 @@ LBS_HD void cell_state(const double* mom, CellState& c)
     for (int a = 0; a < 3; ++a) {
         const double uM2 = u[0] * M2[0][a] + u[1] * M2[1][a] + u[2] * M2[2][a];
         c.q[a] = 0.5 * (mom[10 + a] - u[a] * tr - 2.0 * uM2 + 2.0 * u[a] * um + uu * mom[1 + a] - uu * u[a] * n);
-    }
-}
-
-// The 13 raw moments m (order of cell_state: 1, p_a, p_a p_b (xx yy zz xy xz yz),
-// |p|^2 p_a) of a distribution re-expressed about the velocity u: the moments of
-// psi(p - u).  |p - u|^2 (p_a - u_a) = |p|^2 p_a - u_a |p|^2 - 2 (p.u) p_a + 2 u_a (p.u)
-// + |u|^2 p_a - |u|^2 u_a.
-LBS_HD void shift_moments(const double* m, const double* u, double* out)
-{
-    const double m0 = m[0], m1[3] = {m[1], m[2], m[3]};
-    const double M2[3][3] = {{m[4], m[7], m[8]}, {m[7], m[5], m[9]}, {m[8], m[9], m[6]}};
-    out[0] = m0;
-    for (int a = 0; a < 3; ++a) out[1 + a] = m1[a] - u[a] * m0;
-    const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
-    for (int e = 0; e < 6; ++e) {
-        const int a = ia[e], b = ib[e];
-        out[4 + e] = M2[a][b] - u[a] * m1[b] - u[b] * m1[a] + u[a] * u[b] * m0;
-    }
-    const double tr = m[4] + m[5] + m[6], uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const double um = u[0] * m1[0] + u[1] * m1[1] + u[2] * m1[2];
-    for (int a = 0; a < 3; ++a) {
-        const double uM2 = u[0] * M2[0][a] + u[1] * M2[1][a] + u[2] * M2[2][a];
-        out[10 + a] = m[10 + a] - u[a] * tr - 2.0 * uM2 + 2.0 * u[a] * um + uu * m1[a] - uu * u[a] * m0;
     }
 }
 
