@@ -75,11 +75,18 @@ typedef enum { LBS_VISC_POWER = 0, LBS_VISC_SUTHERLAND = 1 } lbs_visc_law;
  * (without it the state stalls about eps_32 / (lambda dt) short of the steady
  * state, lambda the decay rate of the slowest mode).  The RK stages hold their
  * increments over the step's start state, not stage values, for the same reason.
- * Moment sums: with FP32 storage, in FP32 within a CTA's velocity chunk and in
- * double-float (an FP32 pair, about 48 significant bits) across chunks; with FP64
- * storage, in FP64.  From those sums the cell state (n, u, P, T, q) is formed in the same
- * arithmetic (double-float or FP64) and rounded to FP64; the half-range coefficients of the
- * equilibrium, the wall flux balance and the residual are FP64 in both modes. */
+ * FP64 storage: FP64 throughout.  FP32 storage, behind the FP32 update:
+ *  - moment sums: FP32 within a CTA's velocity chunk, double-float (an FP32 pair, about
+ *    48 significant bits) across chunks;
+ *  - cell state (n, u, P, T, q), x and y expansion coefficients, per-node factors and their
+ *    weighted sums: double-float; the profiles are that state as FP64 numbers;
+ *  - outgoing wall flux: FP32 terms, their weighted products and sums within a chunk
+ *    double-float, FP64 across chunks;
+ *  - half-range coefficients, relaxation time, n_w and the residual: FP64.
+ * The FP32 partial sums carry about 24 bits, so the double-float parts cost no accuracy: with
+ * all of them in FP64 instead, the errors of profiles and states against a 64-bit solution
+ * are the same to four digits (61 batches of all sizes and both models; the profiles differ by
+ * 2e-15). */
 typedef enum { LBS_FP64 = 0, LBS_FP32_STORE_FP64_ACC = 1 } lbs_precision;
 
 /* Velocity-set orders.  N_eq is the order of the truncated Hermite expansion

@@ -291,6 +291,9 @@ static double stage_cost(const lbs_solver* h, int zt, int per_sm, double start)
 //  - FP64: bound by the FP64 pipe, which short tiles load more evenly (16 x C2 at V = 4: 2365 us
 //    of stage kernels per step at 12 cells, 2004 at 8); V = 1 for less than 2^22
 //    velocity-cells, with tiles of 16 cells in the grouped layout (four per warp).
+// Every solver starts unsplit: stepping the halves on two streams is faster in FP64 (us per step,
+// 16 x C2 1947 -> 1878, 8 x C2 1149 -> 1033), mixed in FP32 (256 x C2 1045 -> 1023, 32 x C2 179 ->
+// 186), and needs a second stream and halves alike in tiles, so lbs_set_tiling turns it on.
 static void choose_tiling(lbs_solver* h)
 {
     long work = 0, chunks4 = 0, full4 = 0;
@@ -381,6 +384,9 @@ static void build_tiles(lbs_solver* h, std::vector<Tile>& tiles)
 // 76, 8192 cells 111 / 71 / 73 / 94, 16384 cells 177 / 117 / 90 / 108, 32768 cells 297 / 190 /
 // 152 / 139; 8192 cells of C3 129 / 92 / 104 / 145, the 11792-cell sweep 182 / 124 / 116 / 137;
 // FP64 storage: 2048 cells 68 / 60 / 69 / 92, 8192 cells 165 / 101 / 97 / 115.
+// The lines are FP32's (8 against 16 cells: even between 8192 cells of C2 and the sweep) and serve
+// FP64 too, where 16 cells take over earlier: at 8192 cells it loses 4% of the finalisation by
+// them, under 1% of the step.
 static int finalize_cells_rule(long cells)
 {
     return cells <= 1216 ? 4 : cells <= 10240 ? 8 : cells <= 24576 ? 16 : 32;

@@ -18,7 +18,10 @@
 // the FP64-heavy ones do not meet on one scheduler.  With FP32 storage everything but the
 // half-range coefficients (they cancel by up to 1e7 at order 6) and the scalars of warp 3 is
 // double-float arithmetic: FP32 pairs of about 48 bits, a few cycles per instruction, far
-// below the FP32 rounding of the partials that enter.
+// below the FP32 rounding of the partials that enter.  Against the same code in FP64 (and the
+// wall flux of the stage kernel, which is double-float too) the errors of profiles and states
+// against 64 bits are equal to four digits on each of 61 batches (both models, 3 to 64 nodes per
+// half range, orders 3 to 6, Kn 0.02 to 100); the profiles differ by 2e-15.
 // Measured, us per step (three launches; before: one thread per cell, or one warp per cell up
 // to 608 cells, all but the node sums in FP64): one C2 channel 88 -> 43, the 20 table runs 98
 // -> 47, 64 x C2 157 -> 71, 256 x C2 190 -> 139, 32 x C3 282 -> 92, the sweep 240 -> 116, the
@@ -39,9 +42,11 @@ template <> struct Acc<float> { typedef float type; };
 template <typename T>
 __device__ __forceinline__ T ld(const void* p, int i) { return static_cast<const T*>(p)[i]; }
 
-// 1 / x in FP64 for a finite normal x: the hardware's approximate reciprocal (relative error
-// below 2^-23) and two Newton steps r <- r + r (1 - x r), each squaring the relative error:
-// correct to an ulp in four FMAs, where the IEEE division takes about ten FP64 instructions.
+// 1 / x in FP64 for a finite normal x: the hardware's approximate reciprocal, which reads the
+// upper 32 bits of x and sets those of the result (20 bits of mantissa each: a relative error
+// of some 2^-20), and two Newton steps r <- r + r (1 - x r), each squaring the relative error:
+// about 2^-40, then below the rounding; correct to an ulp in four FMAs, where the IEEE division
+// takes about ten FP64 instructions.
 static __device__ __forceinline__ double rcp_newton(double x)
 {
     double r;
@@ -49,7 +54,8 @@ static __device__ __forceinline__ double rcp_newton(double x)
     r = fma(r, fma(-x, r, 1.0), r);
     return fma(r, fma(-x, r, 1.0), r);
 }
-// 1 / sqrt(x) likewise: r <- r + r (1 - x r^2) / 2
+// 1 / sqrt(x) likewise (a start of some 2^-20 too): r <- r + r (1 - x r^2) / 2, the relative error e
+// becomes 3/2 e^2
 static __device__ __forceinline__ double rsqrt_newton(double x)
 {
     double r;

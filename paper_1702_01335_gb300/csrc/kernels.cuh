@@ -16,15 +16,18 @@
 //                    Appendix, incoming ones as n_w times the wall equilibrium;
 //                    below a half channel's centre line, cells 0..2 at the
 //                    mirrored velocity (bounce-back, Appendix).
-//                    Each thread marches up the z-range for its V velocities
-//                    with a register window: WENO-5 interface fluxes (Eqs.
+//                    Each thread marches through the z-range in the upwind
+//                    direction of its V velocities, carrying the differences of
+//                    the WENO-5 stencil from one interface to the next (the pair
+//                    layout keeps a window of six values): interface fluxes (Eqs.
 //                    weno5_flux - weno_sigma, Table weno), the divergence of
 //                    Eq. (flux), relaxation to n G_x G_y G_z (1 + S) and the
 //                    Shu-Osher combine; it stores F_out and accumulates the raw
 //                    moments of F_out (in FP32 within the CTA and stored per
 //                    chunk in FP32 in FP32 mode; in FP64 in FP64 mode).  Tiles
 //                    that end at a wall also reduce the outgoing WENO flux of
-//                    F_out through the wall.
+//                    F_out through the wall (double-float within the chunk in FP32
+//                    mode).
 //   finalisation     (finalize.cuh) per cell: the sum of the chunks' partials, n, u, P, T, q
 //                    (Eq. qdef), tau, and the cell record of the next stage; per
 //                    instance: the wall densities n_w (zero net mass
@@ -495,7 +498,7 @@ template <typename T, bool PACK> struct PackedAs { typedef T type; };
 template <> struct PackedAs<float, true> { typedef float2 type; };
 
 // Minimum resident CTAs per SM requested from the register allocator: the
-// per-velocity register window grows with V; the rarely taken finalisation
+// per-velocity registers grow with V; the rarely taken finalisation
 // path may spill instead of lowering occupancy.
 template <typename T, int V, int ZW> struct MinBlocks {
     // FP32 at V = 4 fits 128 registers (four CTAs, sixteen warps per SM); FP64 values take

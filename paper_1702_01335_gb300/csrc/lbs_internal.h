@@ -37,8 +37,9 @@ enum { QUAD_FULL = 0, QUAD_HALF = 1 };
 // the per-axis factors); then the per-node factors of the truncated equilibrium as
 // deviations from the rest state's factor 1 (the populations are stored as deviations
 // from the rest state too): dx[Qx] = Gx / w - 1 (before R_SCALE), dy[Qy], dz[2 Qz]
-// (p_z > 0 nodes, then p_z < 0).  They are summed in FP64 in the finalisation and
-// rounded once to the storage type.  Records are rec_stride values apart.
+// (p_z > 0 nodes, then p_z < 0).  The finalisation sums them in FP64 (FP64 storage) or
+// double-float (FP32 storage) and rounds once to the storage type.  Records are rec_stride
+// values apart.
 enum { R_N = 0, R_UX, R_UY, R_UZ, R_T, R_QX, R_QY, R_QZ, R_ITAU, R_CS, R_I5T, R_SCALE1 };
 constexpr int R_DX = kRecHead;
 // record length of an instance, rounded up to 16 bytes in either storage type

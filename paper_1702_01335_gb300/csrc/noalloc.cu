@@ -89,7 +89,7 @@ __global__ void static_profiles(const InstDev* __restrict__ insts, int inst, int
         for (int c = 0; c < nchunks; ++c) s += partial[((size_t)c * Nz + cell) * kNMom + a];
         mom[a] = s;
     }
-    CellState c;  // the solver's own raw -> central moment map (NaN profiles if n = 0)
+    CellState c;  // raw moments about rest -> central ones (NaN profiles if n = 0)
     cell_state(mom, c);
     const double vals[14] = {c.n, c.u[0], c.u[1], c.u[2], c.T, c.q[0], c.q[1], c.q[2],
                              c.P[0], c.P[1], c.P[2], c.P[3], c.P[4], c.P[5]};
