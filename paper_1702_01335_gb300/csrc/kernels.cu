@@ -194,9 +194,12 @@ __global__ void __launch_bounds__(256) gather_states(const InstDev* __restrict__
 cudaError_t launch_gather_states(const InstDev* d_inst, int b0, int n, long at, long total, void* dst, int esize,
                                  cudaStream_t st)
 {
-    // 512 values a warp (four 16-byte words per lane in FP32), or more so that one wave of 64 warps
-    // per SM takes them all
-    const long per = 512 * ((total - 1) / (512L * 64 * 152) + 1), warps = (total + per - 1) / per;
+    // values of a warp: 128 (an FP32 word per lane), up to 512 while eight warps per SM take them all,
+    // then as many more as one wave of 64 warps per SM needs.  Host call in us at 512 / 128 from the
+    // start: one C1 channel in FP64 12.3 / 11.6, the low-Mach runs 13.2 / 12.1, 20 table runs
+    // 13.6 / 14.8, eight C2 channels 15.3 / 17.9.
+    const long few = (total - 1) / (128L * 8 * 152) + 1, many = (total - 1) / (512L * 64 * 152) + 1;
+    const long per = few < 4 ? 128 * few : 512 * many, warps = (total + per - 1) / per;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((warps + 7) / 8));
     cfg.blockDim = dim3(256);
