@@ -16,10 +16,11 @@
 
 namespace lbs {
 cudaError_t launch_stage(int fp32, int red, int V, int stage, const InstDev* d_inst, const Tile* d_tiles,
-                         int ntiles, size_t smem, int fuse, int ninst, int maxNz, int fin_cells, int nb,
+                         int ntiles, size_t smem, int fuse, bool early, int ninst, int maxNz, int fin_cells, int nb,
                          cudaStream_t st);
 cudaError_t launch_stage_only(int fp32, int red, int V, int stage, const InstDev* d_inst, const Tile* d_tiles,
-                              int ntiles, size_t smem, int fuse, cudaStream_t st);
+                              int ntiles, size_t smem, int fuse, bool early, cudaStream_t st);
+int stage_min_ctas(int fp32, int layout);
 cudaError_t launch_finalize(int fp32, int stage, const InstDev* d_inst, int ninst, int maxNz, int fin_cells,
                             int nb, cudaStream_t st);
 cudaError_t launch_seed(int fp32, const InstDev* d_inst, int inst, int Nz, const double* d_macro,
@@ -66,6 +67,8 @@ constexpr long kZSplitPairs = 4 * 608;
 constexpr size_t kPrefetchBytes = size_t(120) << 20;
 
 constexpr size_t kSmemBudget = 200 * 1024;  // dynamic shared memory of a stage CTA
+// shared memory of an SM; what a stage CTA holds beside the dynamic part (its arrays, 1 KB reserved)
+constexpr size_t kSmemPerSM = 228 * 1024, kSmemPerCTA = 1152 + 1024;
 
 struct Pool {  // bump allocator over one device allocation
     size_t bytes = 0;
@@ -274,7 +277,7 @@ static double stage_cost(const lbs_solver* h, int zt, int per_sm, double start)
                                                rec_stride_of(I.Qx, I.Qy, I.Qz)));
     }
     if (smem > kSmemBudget) return 1e300;
-    const long fit = std::max<long>(1, std::min<long>(per_sm, 228 * 1024 / (smem + 1152 + 1024)));
+    const long fit = std::max<long>(1, std::min<long>(per_sm, kSmemPerSM / (smem + kSmemPerCTA)));
     const long waves = (ctas + 152 * fit - 1) / (152 * fit);
     return waves * ((double)steps / ctas + start);
 }
@@ -740,7 +743,7 @@ static const char* const kStageRange[4] = {"lbs analysis", "lbs RK stage 1", "lb
 static lbs_status analyse(lbs_solver* h)
 {
     NvtxRange r(kStageRange[0]);
-    CK(launch_stage(h->fp32, h->reduced, stage_layout(h), 0, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->ninst, h->maxNz,
+    CK(launch_stage(h->fp32, h->reduced, stage_layout(h), 0, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, true, h->ninst, h->maxNz,
                     h->fin_cells, h->nb, h->stream));
     return LBS_OK;
 }
@@ -761,12 +764,25 @@ static lbs_status ensure_stream2(lbs_solver* h)
     return LBS_OK;
 }
 
+// the stage kernel of a step as a programmatic dependent of the finalisation before it
+// (stage_starts_early; the tiles launched now, both halves of a split batch)
+static bool starts_early(const lbs_solver* h)
+{
+    if (h->fuse & 1) return true;  // no finalisation launches between
+    // small batches whose warps split the cells: the low-Mach runs take 91 us per step instead of 93
+    if (h->zsplit && h->V == 1) return true;
+    const long fit = std::min<long>(stage_min_ctas(h->fp32, stage_layout(h)), kSmemPerSM / (h->smem + kSmemPerCTA));
+    const long fin_blocks = (long)h->ninst * ((h->maxNz + h->fin_cells - 1) / h->fin_cells);
+    return stage_starts_early(h->fp32, h->ntiles, std::max(1L, fit), fin_blocks);
+}
+
 static lbs_status enqueue_step(lbs_solver* h)
 {
+    const bool early = starts_early(h);
     if (!split(h)) {
         for (int s = 1; s <= 3; ++s) {
             NvtxRange r(kStageRange[s]);
-            CK(launch_stage(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->ninst,
+            CK(launch_stage(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, early, h->ninst,
                             h->maxNz, h->fin_cells, h->nb, h->stream));
         }
         return LBS_OK;
@@ -777,10 +793,10 @@ static lbs_status enqueue_step(lbs_solver* h)
     // array, a range of tiles); the finalisation kernels take a range of instances
     for (int s = 1; s <= 3; ++s) {
         NvtxRange r(kStageRange[s]);
-        CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntilesA, h->smem, 0, h->stream));
+        CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntilesA, h->smem, 0, early, h->stream));
         CK(launch_finalize(h->fp32, s, h->d_inst, h->nA, h->maxNz, h->fin_cells, h->nb, h->stream));
         CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles + h->ntilesA, h->ntiles - h->ntilesA, h->smem,
-                             0, h->stream2));
+                             0, early, h->stream2));
         CK(launch_finalize(h->fp32, s, h->d_inst + h->nA, h->ninst - h->nA, h->maxNz, h->fin_cells, h->nb, h->stream2));
     }
     CK(cudaEventRecord(h->ev_join, h->stream2));
@@ -1165,7 +1181,7 @@ lbs_status lbs_profile_steps(lbs_handle h, long nsteps, double* out_ms)
     for (long it = 0; it < nsteps && st == LBS_OK; ++it) {
         CK(cudaEventRecord(ev[0], h->stream));
         for (int s = 1; s <= 3; ++s) {
-            CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, h->stream));
+            CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, starts_early(h), h->stream));
             CK(cudaEventRecord(ev[2 * s - 1], h->stream));
             if (!(h->fuse & 1)) CK(launch_finalize(h->fp32, s, h->d_inst, h->ninst, h->maxNz, h->fin_cells, h->nb, h->stream));
             CK(cudaEventRecord(ev[2 * s], h->stream));
@@ -1497,7 +1513,7 @@ lbs_status lbs_set_state(lbs_handle h, int inst, const void* src, int from_host)
             // the same launches as analyse() (the fused finalisation counts per instance)
             NvtxRange ra(kStageRange[0]);
             CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), 0, h->d_inst, h->d_tiles + h->tile_first[c0],
-                                 h->tile_first[c1] - h->tile_first[c0], h->smem, h->fuse & 1, h->stream2));
+                                 h->tile_first[c1] - h->tile_first[c0], h->smem, h->fuse & 1, true, h->stream2));
             if (!(h->fuse & 1))
                 CK(launch_finalize(h->fp32, 0, h->d_inst + c0, c1 - c0, h->maxNz, h->fin_cells, h->nb, h->stream2));
         }

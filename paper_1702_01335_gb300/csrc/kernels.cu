@@ -227,6 +227,15 @@ size_t stage_smem_bytes(int fp32, int V, int zn, int Qx, int Qy, int nzm, int rs
         .total;
 }
 
+// stage CTAs per SM that the register allocator is asked for (shared memory may allow fewer)
+int stage_min_ctas(int fp32, int layout)
+{
+    const int v = layout & 7;
+    if (layout & kZSplit) return v == 1 ? MinBlocks<double, 1, 4>::value : MinBlocks<double, 4, 4>::value;
+    if (fp32) return v == 1 ? MinBlocks<float, 1, 1>::value : v == 2 ? MinBlocks<float, 2, 1>::value : MinBlocks<float, 4, 1>::value;
+    return v == 1 ? MinBlocks<double, 1, 1>::value : v == 2 ? MinBlocks<double, 2, 1>::value : MinBlocks<double, 4, 1>::value;
+}
+
 // Finalisation launches carry the device's highest priority: when the batch's halves step
 // on two streams, the block scheduler then dispatches one half's finalisation blocks as soon
 // as the other half's stage CTAs free room on an SM, instead of after all of them.  (The
@@ -275,14 +284,14 @@ static cudaError_t launch_finalize_c(int fp32, int stage, const InstDev* d_inst,
 
 // the stage kernel alone
 cudaError_t launch_stage_only(int fp32, int red, int V, int stage, const InstDev* d_inst, const Tile* d_tiles,
-                              int ntiles, size_t smem, int fuse, cudaStream_t st)
+                              int ntiles, size_t smem, int fuse, bool early, cudaStream_t st)
 {
     if (ntiles <= 0) return cudaSuccess;  // a split half whose instances have all retired
     if (fp32)
-        return red ? launch_stage_f32_red(V, stage, d_inst, d_tiles, ntiles, smem, fuse, st)
-                   : launch_stage_f32_full(V, stage, d_inst, d_tiles, ntiles, smem, fuse, st);
-    return red ? launch_stage_f64_red(V, stage, d_inst, d_tiles, ntiles, smem, fuse, st)
-               : launch_stage_f64_full(V, stage, d_inst, d_tiles, ntiles, smem, fuse, st);
+        return red ? launch_stage_f32_red(V, stage, d_inst, d_tiles, ntiles, smem, fuse, early, st)
+                   : launch_stage_f32_full(V, stage, d_inst, d_tiles, ntiles, smem, fuse, early, st);
+    return red ? launch_stage_f64_red(V, stage, d_inst, d_tiles, ntiles, smem, fuse, early, st)
+               : launch_stage_f64_full(V, stage, d_inst, d_tiles, ntiles, smem, fuse, early, st);
 }
 
 // the separate finalisation launches of an unfused stage
@@ -300,10 +309,10 @@ cudaError_t launch_finalize(int fp32, int stage, const InstDev* d_inst, int nins
 // one RK stage (stage 1..3) or the analysis pass (stage 0); without fusion the
 // finalisation follows as two more launches
 cudaError_t launch_stage(int fp32, int red, int V, int stage, const InstDev* d_inst, const Tile* d_tiles,
-                         int ntiles, size_t smem, int fuse, int ninst, int maxNz, int fin_cells, int nb,
+                         int ntiles, size_t smem, int fuse, bool early, int ninst, int maxNz, int fin_cells, int nb,
                          cudaStream_t st)
 {
-    cudaError_t e = launch_stage_only(fp32, red, V, stage, d_inst, d_tiles, ntiles, smem, fuse, st);
+    cudaError_t e = launch_stage_only(fp32, red, V, stage, d_inst, d_tiles, ntiles, smem, fuse, early, st);
     if (e != cudaSuccess || fuse) return e;
     return launch_finalize(fp32, stage, d_inst, ninst, maxNz, fin_cells, nb, st);
 }

@@ -1535,7 +1535,7 @@ stage_kernel(const InstDev* __restrict__ insts, const Tile* __restrict__ tiles, 
 // ---- host-side launch of one stage-kernel instantiation ----------------------
 template <typename T, int V, int STAGE, bool RED, bool GRP, int ZW>
 static cudaError_t launch_stage_t(const InstDev* d_inst, const Tile* d_tiles, int ntiles, size_t smem,
-                                  int fuse, cudaStream_t st)
+                                  int fuse, bool early, cudaStream_t st)
 {
     auto kfn = stage_kernel<T, V, STAGE, RED, GRP, ZW>;
     if (smem > 40 * 1024) {  // with the static arrays above the default limit of 48 KB
@@ -1551,47 +1551,47 @@ static cudaError_t launch_stage_t(const InstDev* d_inst, const Tile* d_tiles, in
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;  // stage_starts_early
     return cudaLaunchKernelEx(&cfg, kfn, d_inst, d_tiles, fuse);
 }
 
 template <typename T, int V, bool RED, bool GRP = false, int ZW = 1>
 static cudaError_t launch_stage_r(int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
-                                  cudaStream_t st)
+                                  bool early, cudaStream_t st)
 {
     switch (stage) {
-        case 0: return launch_stage_t<T, V, 0, RED, GRP, ZW>(d, t, n, smem, fuse, st);
-        case 1: return launch_stage_t<T, V, 1, RED, GRP, ZW>(d, t, n, smem, fuse, st);
-        case 2: return launch_stage_t<T, V, 2, RED, GRP, ZW>(d, t, n, smem, fuse, st);
-        default: return launch_stage_t<T, V, 3, RED, GRP, ZW>(d, t, n, smem, fuse, st);
+        case 0: return launch_stage_t<T, V, 0, RED, GRP, ZW>(d, t, n, smem, fuse, early, st);
+        case 1: return launch_stage_t<T, V, 1, RED, GRP, ZW>(d, t, n, smem, fuse, early, st);
+        case 2: return launch_stage_t<T, V, 2, RED, GRP, ZW>(d, t, n, smem, fuse, early, st);
+        default: return launch_stage_t<T, V, 3, RED, GRP, ZW>(d, t, n, smem, fuse, early, st);
     }
 }
 
 template <typename T, bool RED>
 static cudaError_t launch_stage_m(int V /* a layout: stage_layout in api.cu */, int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
-                                  cudaStream_t st)
+                                  bool early, cudaStream_t st)
 {
     if constexpr (!RED) {
-        if (V == (4 | kGrouped)) return launch_stage_r<T, 4, false, true>(stage, d, t, n, smem, fuse, st);
+        if (V == (4 | kGrouped)) return launch_stage_r<T, 4, false, true>(stage, d, t, n, smem, fuse, early, st);
         if constexpr (sizeof(T) == 8)
             if (V == (4 | kGrouped | kZSplit))
-                return launch_stage_r<T, 4, false, true, 4>(stage, d, t, n, smem, fuse, st);
+                return launch_stage_r<T, 4, false, true, 4>(stage, d, t, n, smem, fuse, early, st);
     }
     if constexpr (sizeof(T) == 8)
-        if (V == (1 | kZSplit)) return launch_stage_r<T, 1, RED, false, 4>(stage, d, t, n, smem, fuse, st);
-    if (V == 1) return launch_stage_r<T, 1, RED>(stage, d, t, n, smem, fuse, st);
-    if (V == 2) return launch_stage_r<T, 2, RED>(stage, d, t, n, smem, fuse, st);
-    return launch_stage_r<T, 4, RED>(stage, d, t, n, smem, fuse, st);
+        if (V == (1 | kZSplit)) return launch_stage_r<T, 1, RED, false, 4>(stage, d, t, n, smem, fuse, early, st);
+    if (V == 1) return launch_stage_r<T, 1, RED>(stage, d, t, n, smem, fuse, early, st);
+    if (V == 2) return launch_stage_r<T, 2, RED>(stage, d, t, n, smem, fuse, early, st);
+    return launch_stage_r<T, 4, RED>(stage, d, t, n, smem, fuse, early, st);
 }
 
 // per (storage type, model) launchers of the stage kernel, one translation unit each
 cudaError_t launch_stage_f32_full(int V, int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
-                                  cudaStream_t st);
+                                  bool early, cudaStream_t st);
 cudaError_t launch_stage_f32_red(int V, int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
-                                 cudaStream_t st);
+                                 bool early, cudaStream_t st);
 cudaError_t launch_stage_f64_full(int V, int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
-                                  cudaStream_t st);
+                                  bool early, cudaStream_t st);
 cudaError_t launch_stage_f64_red(int V, int stage, const InstDev* d, const Tile* t, int n, size_t smem, int fuse,
-                                 cudaStream_t st);
+                                 bool early, cudaStream_t st);
 
 }  // namespace lbs

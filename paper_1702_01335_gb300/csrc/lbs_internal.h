@@ -239,6 +239,23 @@ LBS_HD double relax_time(int law, double Kn, double param, double n, double T)
     return Kn * sqrt(T) * (1.0 + param) / (n * (T + param));
 }
 
+// ---- whether a stage kernel starts while the finalisation before it still runs ----
+// Started early (as a programmatic dependent), the stage kernel saves 1 us, but its CTAs go to the
+// SMs that the finalisation's blocks have left room on and stay there.  Where the batch is one
+// wave, the finalisation sits on many SMs and an SM can take more CTAs than its even share, they
+// pile up, and in FP64, which is bound by an SM's FP64 units, the fullest SM sets the time: ten
+// half channels of 5 x 3 x 11 nodes and 45 cells at V = 4 and eight cells 668 us per step before
+// there were early starts, 1009 with one, 404 without.  Hence, in FP64, none where the finalisation
+// holds a quarter of the 152 SMs, both together outnumber the SMs, and an SM could take a third
+// more than its share.  Of 510 measured FP64 tilings (17 batches, V = 1, 2, 4, 3 to 64 cells, split
+// or not) none is slower by the rule than with early starts throughout, 63 are faster by 3% to 65%.
+// FP32, bound by latency, gains by early starts (one C2 channel 53 -> 48 us per step).
+inline bool stage_starts_early(bool fp32, long ctas, long fit, long fin_blocks)
+{
+    const long share = (ctas + 151) / 152;
+    return fp32 || 4 * fin_blocks < 152 || ctas + fin_blocks <= 152 || 4 * share > 3 * fit;
+}
+
 // ---- the destination of lbs_get_state's gathering launch ----
 // A kernel needs the solver's device to be the current one and writes wherever it is told; a
 // copy runs whatever device is current and refuses what is not memory.  So the launch takes

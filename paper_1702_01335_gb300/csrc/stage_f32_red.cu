@@ -6,9 +6,9 @@
 namespace lbs {
 
 cudaError_t launch_stage_f32_red(int V, int stage, const InstDev* d, const Tile* t, int n, size_t smem,
-                                 int fuse, cudaStream_t st)
+                                 int fuse, bool early, cudaStream_t st)
 {
-    return launch_stage_m<float, true>(V, stage, d, t, n, smem, fuse, st);
+    return launch_stage_m<float, true>(V, stage, d, t, n, smem, fuse, early, st);
 }
 
 }  // namespace lbs
