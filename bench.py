@@ -292,7 +292,7 @@ def run_small(a):
                     "profiled_step_ms": k_step / nprof},
         "e2e": {"value": upd_step * e2e_steps / e2e_s, "unit": "updates/s",
                 "h2d_bytes_per_step": s.state_bytes(), "d2h_bytes_per_step": nrows * 8},
-        "gpu_launches": {0: 6, 1: 3, 2: 12}[tl["fuse"]] * a.steps,
+        "gpu_launches": {0: 6, 1: 3 if tl["ZT"] <= 8 else 6, 2: 12}[tl["fuse"]] * a.steps,
         "clocks": clk.summary(),
     }
     if a.workload == "luo":
@@ -431,7 +431,7 @@ def run_sweep(a):
     steps = gather([int(x) for x in steps], idx, len(inst_all), dist)
     res = gather(res, idx, len(inst_all), dist)
     conv = [r < 1e-8 for r in res]
-    launches = reduce({0: 6, 1: 3, 2: 12}[tl["fuse"]] * a.steps, "sum")
+    launches = reduce({0: 6, 1: 3 if tl["ZT"] <= 8 else 6, 2: 12}[tl["fuse"]] * a.steps, "sum")
     if dist is not None:
         dist.destroy_process_group()
     if rank != 0:
@@ -617,7 +617,7 @@ def main():
                     "h2d_bytes_per_step": s.state_bytes(), "d2h_bytes_per_step": nprof_rows * 8,
                     "what": "lbs_set_state(all, pinned host) + lbs_step(1) + lbs_moments(all, host) "
                             "per step"},
-            "gpu_launches": {0: 6, 1: 3, 2: 12}[tuned["fuse"]] * a.steps,
+            "gpu_launches": {0: 6, 1: 3 if tuned["ZT"] <= 8 else 6, 2: 12}[tuned["fuse"]] * a.steps,
             "clocks": clk.summary(),
         }
         if not a.no_cpu_baseline and world == 1:

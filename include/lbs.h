@@ -281,8 +281,9 @@ lbs_status lbs_profile_steps(lbs_handle h, long nsteps, double* out_ms);
  * whose Qy are all multiples of four gives each thread four adjacent velocities of one
  * (x, z) node, in
  * either precision (results agree to rounding).  fuse = 1 folds the per-cell and
- * per-instance finalisation into the stage kernel (the last CTA of a z-tile /
- * of an instance does it: 3 launches per step); fuse = 0 runs it as one
+ * per-instance finalisation into the stage kernel where ZT <= 8 (the last CTA of a
+ * z-tile / of an instance does it: 3 launches per step), and runs longer tiles, which
+ * one CTA would be slow to finalise, as fuse = 0; fuse = 0 runs it as one
  * further launch per stage; fuse = 2 does the
  * same for each half of the batch (about half the tiles each) on two streams,
  * so that one half's FP64 finalisation overlaps the other half's stage kernel

@@ -739,11 +739,18 @@ struct NvtxRange {
 };
 static const char* const kStageRange[4] = {"lbs analysis", "lbs RK stage 1", "lbs RK stage 2", "lbs RK stage 3"};
 
+// fuse = 1 folds the finalisation into the stage kernel for tiles of up to kFoldCells cells.  A
+// longer tile would be finalised four cells after four by one CTA; launches of their own spread
+// the cells.  Measured, us per step, folded -> by this rule: six C2 channels in FP32 at V = 2 and
+// 64 cells 412 -> 148, 16 cells 161 -> 104, eight cells 117 (folded); 200 C1 channels at V = 1 and
+// 64 cells 340 -> 152.
+static int folded(const lbs_solver* h) { return fold_finalisation(h->fuse, h->ZT); }
+
 // moments, records, wall densities and W_old of the current F0 (every active instance)
 static lbs_status analyse(lbs_solver* h)
 {
     NvtxRange r(kStageRange[0]);
-    CK(launch_stage(h->fp32, h->reduced, stage_layout(h), 0, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, true, h->ninst, h->maxNz,
+    CK(launch_stage(h->fp32, h->reduced, stage_layout(h), 0, h->d_inst, h->d_tiles, h->ntiles, h->smem, folded(h), true, h->ninst, h->maxNz,
                     h->fin_cells, h->nb, h->stream));
     return LBS_OK;
 }
@@ -768,7 +775,7 @@ static lbs_status ensure_stream2(lbs_solver* h)
 // (stage_starts_early; the tiles launched now, both halves of a split batch)
 static bool starts_early(const lbs_solver* h)
 {
-    if (h->fuse & 1) return true;  // no finalisation launches between
+    if (folded(h)) return true;  // no finalisation launches between
     // small batches whose warps split the cells: the low-Mach runs take 91 us per step instead of 93
     if (h->zsplit && h->V == 1) return true;
     const long fit = std::min<long>(stage_min_ctas(h->fp32, stage_layout(h)), kSmemPerSM / (h->smem + kSmemPerCTA));
@@ -782,7 +789,7 @@ static lbs_status enqueue_step(lbs_solver* h)
     if (!split(h)) {
         for (int s = 1; s <= 3; ++s) {
             NvtxRange r(kStageRange[s]);
-            CK(launch_stage(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, early, h->ninst,
+            CK(launch_stage(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, folded(h), early, h->ninst,
                             h->maxNz, h->fin_cells, h->nb, h->stream));
         }
         return LBS_OK;
@@ -1181,9 +1188,9 @@ lbs_status lbs_profile_steps(lbs_handle h, long nsteps, double* out_ms)
     for (long it = 0; it < nsteps && st == LBS_OK; ++it) {
         CK(cudaEventRecord(ev[0], h->stream));
         for (int s = 1; s <= 3; ++s) {
-            CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, h->fuse & 1, starts_early(h), h->stream));
+            CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), s, h->d_inst, h->d_tiles, h->ntiles, h->smem, folded(h), starts_early(h), h->stream));
             CK(cudaEventRecord(ev[2 * s - 1], h->stream));
-            if (!(h->fuse & 1)) CK(launch_finalize(h->fp32, s, h->d_inst, h->ninst, h->maxNz, h->fin_cells, h->nb, h->stream));
+            if (!folded(h)) CK(launch_finalize(h->fp32, s, h->d_inst, h->ninst, h->maxNz, h->fin_cells, h->nb, h->stream));
             CK(cudaEventRecord(ev[2 * s], h->stream));
         }
         CK(cudaEventSynchronize(ev[6]));
@@ -1513,8 +1520,8 @@ lbs_status lbs_set_state(lbs_handle h, int inst, const void* src, int from_host)
             // the same launches as analyse() (the fused finalisation counts per instance)
             NvtxRange ra(kStageRange[0]);
             CK(launch_stage_only(h->fp32, h->reduced, stage_layout(h), 0, h->d_inst, h->d_tiles + h->tile_first[c0],
-                                 h->tile_first[c1] - h->tile_first[c0], h->smem, h->fuse & 1, true, h->stream2));
-            if (!(h->fuse & 1))
+                                 h->tile_first[c1] - h->tile_first[c0], h->smem, folded(h), true, h->stream2));
+            if (!folded(h))
                 CK(launch_finalize(h->fp32, 0, h->d_inst + c0, c1 - c0, h->maxNz, h->fin_cells, h->nb, h->stream2));
         }
         c0 = c1;

@@ -30,6 +30,10 @@ constexpr int kGrouped = 8;     // four adjacent velocities of one x and z node 
 constexpr int kZSplit = 16;     // the CTA's warps split the tile's cells
 inline int layout_columns(int layout) { return (layout & 7) * (layout & kZSplit ? kThreads / 4 : kThreads); }
 
+// whether a tiling's finalisation is folded into the stage kernel (api.cu has the reason)
+constexpr int kFoldCells = 8;
+inline bool fold_finalisation(int fuse, int ZT) { return fuse == 1 && ZT <= kFoldCells; }
+
 enum { QUAD_FULL = 0, QUAD_HALF = 1 };
 
 // Cell record (storage type T): n, ux, uy, uz, T, qx, qy, qz, 1/tau,

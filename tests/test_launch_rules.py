@@ -22,3 +22,12 @@ def test_stage_ctas_do_not_pile_up_beside_the_finalisation(tmp_path):
     got = answers(tmp_path, "".join('std::printf("%%d %%d ", stage_starts_early(false, %d, %d, %d), '
                                     'stage_starts_early(true, %d, %d, %d));\n' % (c[:3] + c[:3]) for c in cases))
     assert [g == "1" for g in got] == [v for c in cases for v in (c[3], True)]
+
+
+def test_long_tiles_are_not_finalised_inside_the_stage_kernel(tmp_path):
+    """fuse = 1 folds the finalisation into the stage kernel for tiles of up to eight cells; one CTA
+    would finalise a longer one four cells after four.  The other modes never fold it."""
+    got = answers(tmp_path, """
+    for (int fuse : {0, 1, 2})
+        for (int ZT : {3, 4, 8, 9, 16, 64}) std::printf("%d ", fold_finalisation(fuse, ZT));""")
+    assert [g == "1" for g in got] == [f == 1 and z <= 8 for f in (0, 1, 2) for z in (3, 4, 8, 9, 16, 64)]
